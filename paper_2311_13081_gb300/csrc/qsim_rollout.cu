@@ -615,6 +615,7 @@ qsim_status launch_rollout_tc_range(qsim_handle* h, const float* actor, int T, u
 qsim_status launch_track_tc(qsim_handle* h, const float* actor, int T, const TrackArgs& tr, int chunk,
                             cudaStream_t st);
 int rollout_tc_warps_per_cta();
+size_t rollout_tc_sched_ints(int warps);
 
 // Launches T steps of the rollout as `parts` env partitions x chunks of `chunk` steps.
 // Partition p owns warps [W p / parts, W (p+1) / parts); its chunks run in order on its
@@ -642,10 +643,8 @@ qsim_status launch_rollout(qsim_handle* h, const float* actor, int hidden, int T
     if (tc) {
         if (parts == 1) {
             // one persistent launch walking (group of 384 envs, chunk of steps) units
-            if (!h->tc_sched) {
-                const int groups = (warps + rollout_tc_warps_per_cta() - 1) / rollout_tc_warps_per_cta();
-                QCHECK_CUDA(cudaMalloc((void**)&h->tc_sched, sizeof(int) * (size_t)(1 + groups)));
-            }
+            if (!h->tc_sched)
+                QCHECK_CUDA(cudaMalloc((void**)&h->tc_sched, sizeof(int) * rollout_tc_sched_ints(warps)));
             return launch_rollout_tc_range(h, actor, T, t0, h->head, sigma, 0, warps, st,
                                            chunk < T ? chunk : kTcChunk, h->tc_sched);
         }

@@ -234,7 +234,7 @@ template <bool TRACK>
 __global__ void __launch_bounds__(NT, 1) k_rollout_tc(EnvCfg C, EnvPtrs p, const float* __restrict__ actor,
                                                       int T, uint32_t t0, int64_t head0, int64_t capacity,
                                                       float sigma_in, int warp0, int warp_end,
-                                                      int n_groups, int chunk, int* sched, TrackArgs tr) {
+                                                      int n_groups, int chunk, int ct, int* sched, TrackArgs tr) {
     extern __shared__ __align__(1024) unsigned char smb[];
     __half* W1s = reinterpret_cast<__half*>(smb + OFF_W1);
     __half* W2s = reinterpret_cast<__half*>(smb + OFF_W2);
@@ -388,7 +388,9 @@ __global__ void __launch_bounds__(NT, 1) k_rollout_tc(EnvCfg C, EnvPtrs p, const
         const int Tu = min(chunk, T - uk * chunk);
         const uint32_t t0u = t0 + (uint32_t)(uk * chunk);
         const int64_t headu = head0 + (int64_t)uk * chunk;
-        if (mma_warp) {
+        if (tile >= ct) {
+            // this call's groups have ct tiles: the others' warps only follow the unit barriers
+        } else if (mma_warp) {
             // ================= MMA warp of this tile: lane 0 issues, the warp follows the waits
             // (descriptors from the table built at setup: the issue loops are MMAs only)
             const uint64_t* d1 = reinterpret_cast<const uint64_t*>(smb + OFF_DESC);
@@ -434,7 +436,7 @@ __global__ void __launch_bounds__(NT, 1) k_rollout_tc(EnvCfg C, EnvPtrs p, const
             // ================= compute warps: thread r of the tile owns env r and TMEM lane r
             const int r = tid & (TILE - 1);
             const uint32_t tl = tmem + ((uint32_t)(32 * (warp & 3)) << 16);  // this warp's lanes
-            const int gw = warp0 + ug * NCW + warp;                          // global warp (32 envs)
+            const int gw = warp0 + ug * (4 * ct) + warp;                     // global warp (32 envs)
             const bool active = gw < warp_end;                               // warp-uniform
             const int g = active ? gw * 32 + lane : lane;  // inactive warps: an in-range index, never stored to
 
@@ -843,9 +845,36 @@ __global__ void __launch_bounds__(NT, 1) k_rollout_tc(EnvCfg C, EnvPtrs p, const
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(*tslot), "r"(T_ALLOC) : "memory");
 }
 
-// Launches T steps on env warps [w0, w1) (12 env warps = 384 envs per CTA, plus 3 MMA warps):
-// one CTA per group of 12 warps, or, with chunk > 0 and `sched` (1 + groups ints of device
-// memory), a persistent grid of at most one CTA per SM walking (group, chunk) units.
+// Tiles of 128 envs a CTA of the persistent schedule works on (1..TILES).  A CTA's tiles
+// share its SM's issue slots, so a step takes longer the more of them there are: 4.4, 5.5
+// and 6.6 us with one, two and three (1,000 envs; 4.9, 5.9, 6.8 with every SM busy).  Few
+// envs therefore spread over more SMs, one tile each; with more tiles than SMs the units of
+// a smaller group queue up instead, and the larger group wins where its step costs less
+// than the extra rounds.  200 steps, three tiles always / by this rule, us: 1,000 envs
+// 1319 / 875, 19,456 1339 / 975, 38,912 1367 / 1172, 45,000 1398 / 1398 (two: 1435).
+static int tiles_per_cta(int tiles, int n_chunks, int sms) {
+    static const double kStepUs[TILES] = {4.5, 5.6, 6.75};
+    int best = TILES;
+    double best_t = 1e30;
+    for (int ct = 1; ct <= TILES; ++ct) {
+        const int64_t groups = (tiles + ct - 1) / ct;
+        const int64_t rounds = groups <= sms ? n_chunks : (groups * n_chunks + sms - 1) / sms;
+        const double t = (double)rounds * kStepUs[ct - 1];
+        if (t < best_t) {
+            best_t = t;
+            best = ct;
+        }
+    }
+    return best;
+}
+
+// Ints of the persistent schedule's device counters for `warps` env warps.
+size_t rollout_tc_sched_ints(int warps) { return 1 + (size_t)((warps + 3) / 4); }
+
+// Launches T steps on env warps [w0, w1) (up to 12 env warps = 384 envs per CTA, plus 3 MMA
+// warps): one CTA per group of 12 warps, or, with chunk > 0 and `sched`
+// (rollout_tc_sched_ints of device memory), a persistent grid of at most one CTA per SM
+// walking (group, chunk) units.
 qsim_status launch_rollout_tc_range(qsim_handle* h, const float* actor, int T, uint32_t t0, int64_t head,
                                     float sigma, int w0, int w1, cudaStream_t st, int chunk, int* sched) {
     static bool configured = false;
@@ -853,17 +882,20 @@ qsim_status launch_rollout_tc_range(qsim_handle* h, const float* actor, int T, u
         QCHECK_CUDA(cudaFuncSetAttribute(k_rollout_tc<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM));
         configured = true;
     }
-    const int groups = (w1 - w0 + NCW - 1) / NCW;
     if (sched && chunk > 0) {
         int sms = 152;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+        chunk = std::min(chunk, T);
+        const int ct = tiles_per_cta((w1 - w0 + 3) / 4, (T + chunk - 1) / chunk, sms);
+        const int groups = (w1 - w0 + 4 * ct - 1) / (4 * ct);
         QCHECK_CUDA(cudaMemsetAsync(sched, 0, sizeof(int) * (size_t)(1 + groups), st));
         const int grid = std::min(sms, groups);
         k_rollout_tc<false><<<grid, NT, SMEM, st>>>(h->dc, h->p, actor, T, t0, head, h->capacity, sigma, w0, w1,
-                                                    groups, std::min(chunk, T), sched, TrackArgs{});
+                                                    groups, chunk, ct, sched, TrackArgs{});
     } else {
+        const int groups = (w1 - w0 + NCW - 1) / NCW;
         k_rollout_tc<false><<<groups, NT, SMEM, st>>>(h->dc, h->p, actor, T, t0, head, h->capacity, sigma, w0, w1,
-                                                      groups, T, nullptr, TrackArgs{});
+                                                      groups, T, TILES, nullptr, TrackArgs{});
     }
     QCHECK_LAUNCH("k_rollout_tc");
     return QSIM_OK;
@@ -916,7 +948,11 @@ qsim_status launch_track_tc(qsim_handle* h, const float* actor, int T, const Tra
         configured = true;
     }
     const int ld = h->ld, warps = ld / 32;
-    const int groups = (warps + NCW - 1) / NCW;
+    int sms = 152;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+    chunk = std::max(1, std::min(chunk, T));
+    const int ct = tiles_per_cta((warps + 3) / 4, (T + chunk - 1) / chunk, sms);
+    const int groups = (warps + 4 * ct - 1) / (4 * ct);
     const size_t n = (size_t)ld;
     float* scr = nullptr;
     QCHECK_CUDA(cudaMallocAsync((void**)&scr, sizeof(float) * (n * (NS + 8 + 6 + 4 * HMAX + 6) + 1 + groups), st));
@@ -942,11 +978,9 @@ qsim_status launch_track_tc(qsim_handle* h, const float* actor, int T, const Tra
     k_track_init<<<(ld + 127) / 128, 128, 0, st>>>(C, p, tr);
     QCHECK_LAUNCH("k_track_init");
     if (T > 0) {
-        int sms = 152;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
         QCHECK_CUDA(cudaMemsetAsync(sched, 0, sizeof(int) * (size_t)(1 + groups), st));
         k_rollout_tc<true><<<std::min(sms, groups), NT, SMEM, st>>>(C, p, actor, T, 0u, 0, 0, 0.0f, 0, warps,
-                                                                     groups, std::min(chunk, T), sched, tr);
+                                                                     groups, chunk, ct, sched, tr);
         QCHECK_LAUNCH("k_rollout_tc<track>");
     }
     QCHECK_CUDA(cudaFreeAsync(scr, st));

@@ -48,3 +48,25 @@ def test_step_writes_what_observe_reads(gpu, n, n_hist, layout):
         assert (cpu(info["n_done"])[:n] > 0).all()
     finally:
         q.qsim_destroy(h)
+
+
+@pytest.mark.parametrize("n", [1, 129, 152 * 128 + 1, 2 * 152 * 128 + 1])
+def test_tensor_core_tiles_per_block_agree(gpu, n):
+    """One, two or three tiles per block (chosen by the env count) against two partitions,
+    which always run three."""
+    q = gpu
+    outs = []
+    for parts in (0, 2):
+        d, cfg, veh = lib_config(q, "c2", n_envs=n, capacity=12, learning_starts=1, episode_len=9, sig_p=0.01)
+        h = q.qsim_create(cfg, veh)
+        try:
+            A = torch.tensor(_actor(d, 64), device="cuda")
+            q.qsim_rollout_engine(h, 2)
+            q.qsim_rollout_schedule(h, parts, 0)
+            q.qsim_rollout(h, A, 64, 12, 0.1)
+            q.qsim_sync(h)
+            outs.append(_bits(q.qsim_info_get(h), n))
+        finally:
+            q.qsim_destroy(h)
+    for x, y in zip(*outs):
+        assert np.array_equal(x, y)
