@@ -32,7 +32,7 @@
 
 namespace qsim {
 
-template <int H>
+template <int H, int EPW = 32>
 struct RollLayout {
     static constexpr int OBS_MAX = 18 + 4 * HMAX;  // 82
     static constexpr int W1 = 0;
@@ -42,8 +42,11 @@ struct RollLayout {
     static constexpr int W3 = B2 + H;      // transposed [H][4]
     static constexpr int B3 = W3 + 4 * H;
     static constexpr int WEIGHTS = ((B3 + 4) + 3) & ~3;
-    static constexpr int OBS = OBS_MAX * 32;
-    static constexpr int HID = H * 32;
+    static constexpr int OBS = OBS_MAX * EPW;
+    // hidden tile rows of EPW floats; with 8 envs a warp the rows of each lane group of
+    // outputs start 8 floats further on, so that the groups' stores fall into distinct banks
+    static constexpr int SKEW = EPW == 32 ? 0 : 8;
+    static constexpr int HID = H * EPW + 8 * SKEW;
     static constexpr int PER_WARP = OBS + HID;
     static size_t bytes(int nw) { return sizeof(float) * (size_t)(WEIGHTS + nw * PER_WARP); }
 };
@@ -58,18 +61,27 @@ __device__ __forceinline__ int wpos(int o) {
     return (r >> 2) * 32 + ty * 4 + (r & 3);
 }
 
-template <int H, int NW, bool PK, bool TRACK = false>
-__global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
+// EPW = 32: one env per lane.  EPW = 8 (paired FMA only): a warp takes 8 envs, so that few
+// envs spread over four times as many warps.  The GEMMs give lane (tx, ty) the same H/8
+// outputs of 2 envs instead of 8; every output and every partial sum of layer 3 is formed
+// in the same order, so the results are those of EPW = 32.  Lane (tx, ty) owns env 2 tx +
+// (ty & 1): four lanes (copies cp = ty >> 1) run the same env's dynamics and bookkeeping,
+// share its noise blocks, and copy 0 stores.
+template <int H, int NW, bool PK, bool TRACK = false, int EPW = 32>
+__global__ void __launch_bounds__(NW ? NW * 32 : 256) k_rollout(EnvCfg C, EnvPtrs p,
                                                      const float* __restrict__ actor, int T,
                                                      uint32_t t0, int64_t head0,
                                                      int64_t capacity, float sigma_in,
                                                      int warp0, int warp_end, TrackArgs tr) {
-    using L = RollLayout<H>;
+    using L = RollLayout<H, EPW>;
+    static_assert(EPW == 32 || (EPW == 8 && PK), "envs per warp");
+    constexpr int EG = EPW / 4;  // envs per lane in the GEMMs
     constexpr int OP = H / 8;  // outputs per lane
     constexpr int NQ = OP / 4; // float4 chunks per lane per weight row
     extern __shared__ __align__(16) float smem[];
     const int DA = C.obs_dim;
     const int ld = C.ld;
+    const int nthr = NW ? NW * 32 : (int)blockDim.x;  // NW = 0: warps per CTA chosen at launch
 
     // ---- stage the actor weights (canonical W1[H][DA] b1 W2[H][H] b2 W3[4][H] b3)
     {
@@ -81,19 +93,19 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
         const float* gb2 = gW2 + H * H;
         const float* gW3 = gb2 + H;
         const float* gb3 = gW3 + 4 * H;
-        for (int i = threadIdx.x; i < H * DA; i += NW * 32) {
+        for (int i = threadIdx.x; i < H * DA; i += nthr) {
             const int o = i / DA, k = i - o * DA;
             sW1[k * H + wpos<H>(o)] = gW1[i];
         }
-        for (int i = threadIdx.x; i < H * H; i += NW * 32) {
+        for (int i = threadIdx.x; i < H * H; i += nthr) {
             const int o = i / H, k = i - o * H;
             sW2[k * H + wpos<H>(o)] = gW2[i];
         }
-        for (int i = threadIdx.x; i < H; i += NW * 32) {
+        for (int i = threadIdx.x; i < H; i += nthr) {
             smem[L::B1 + i] = gb1[i];
             smem[L::B2 + i] = gb2[i];
         }
-        for (int i = threadIdx.x; i < 4 * H; i += NW * 32) {
+        for (int i = threadIdx.x; i < 4 * H; i += nthr) {
             const int j = i / H, k = i - j * H;
             smem[L::W3 + k * 4 + j] = gW3[i];
         }
@@ -102,10 +114,13 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
     __syncthreads();
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int gw = warp0 + blockIdx.x * NW + warp;  // global warp (32 envs)
-    const int g = gw * 32 + lane;                      // global env index
+    const int gw = warp0 + blockIdx.x * (nthr / 32) + warp;  // global warp (EPW envs)
     if (gw >= warp_end) return;                        // warp-uniform
     const int tx = lane >> 3, ty = lane & 7;
+    const int eo = EPW == 32 ? lane : 2 * tx + (ty & 1);  // this lane's env within the warp
+    const int cp = EPW == 32 ? 0 : ty >> 1;               // which of its copies
+    const bool own = cp == 0;
+    const int g = gw * EPW + eo;                          // global env index
     float* sObs = smem + L::WEIGHTS + warp * L::PER_WARP;
     float* sHid = sObs + L::OBS;
     const float* sW1 = smem + L::W1;
@@ -152,14 +167,14 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
     const float sigma = sigma_in >= 0.0f ? sigma_in : p.rewardC[7];
     const int nh = C.n_hist;
     if constexpr (TRACK) {
-        for (int k = 18; k < 18 + 4 * HMAX; ++k) sObs[k * 32 + lane] = 0.0f;
+        for (int k = 18; k < 18 + 4 * HMAX; ++k) sObs[k * EPW + eo] = 0.0f;
     } else
     // history (newest first in global) -> ring slot (t0 - i) mod 16
     for (int i = 1; i <= nh; ++i) {
         const int slot = (int)((t0 - (uint32_t)i) & 15u);
 #pragma unroll
         for (int c = 0; c < 4; ++c)
-            sObs[(18 + 4 * slot + c) * 32 + lane] = p.hist[(4 * (i - 1) + c) * ld + g];
+            sObs[(18 + 4 * slot + c) * EPW + eo] = p.hist[(4 * (i - 1) + c) * ld + g];
     }
     int64_t slot = capacity > 0 ? head0 % capacity : 0;
     const int F = C.F;
@@ -178,14 +193,29 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
                     o[k] = clampf(o[k] - pr[k], -tr.clip_p, tr.clip_p);
                     o[12 + k] = clampf(o[12 + k] - vr[k], -tr.clip_v, tr.clip_v);
                 }
-            } else if (C.any_noise) {
+            } else if (EPW == 32 && C.any_noise) {
                 float nz[18];
                 obs_noise(C, (uint32_t)g, t, nz);
 #pragma unroll
                 for (int k = 0; k < 18; ++k) o[k] += nz[k];
             }
+            // (every copy stores all of its entries: a store under a condition moves their
+            // arithmetic into its block, where other products are fused)
 #pragma unroll
-            for (int k = 0; k < 18; ++k) sObs[k * 32 + lane] = o[k];
+            for (int k = 0; k < 18; ++k) sObs[k * EPW + eo] = o[k];
+            if (!TRACK && EPW != 32 && C.any_noise) {
+                // copy cp adds the noise of the pairs b = cp, cp + 4, ..
+                __syncwarp();
+#pragma unroll 1
+                for (int b = cp; b < 9; b += 4) {
+                    float n0, n1;
+                    obs_noise_pair(C, (uint32_t)g, t, b, n0, n1);
+                    // (a plain sum, as where the noise comes from an array: never fused
+                    // with the product that made it)
+                    sObs[2 * b * EPW + eo] = __fadd_rn(sObs[2 * b * EPW + eo], n0);
+                    sObs[(2 * b + 1) * EPW + eo] = __fadd_rn(sObs[(2 * b + 1) * EPW + eo], n1);
+                }
+            }
         }
         __syncwarp();
         float a[4];
@@ -197,17 +227,17 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
             a[3] = 2.0f * u01(r.w) - 1.0f;
         } else {
             // ---------------- layer 1: obs (DA) -> H, ReLU
-            float acc[OP][8];
+            float acc[OP][EG];
             if constexpr (PK) {
                 // paired FMAs: acc2[q][e] holds outputs (2q, 2q+1) of env e; weight pairs come
                 // straight from the 128-bit shared loads, activations are duplicated
-                unsigned long long acc2[OP / 2][8];
+                unsigned long long acc2[OP / 2][EG];
 #pragma unroll
                 for (int q = 0; q < OP / 2; ++q) {
                     const unsigned long long b = f2pack(smem[L::B1 + ty * OP + 2 * q],
                                                         smem[L::B1 + ty * OP + 2 * q + 1]);
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) acc2[q][e] = b;
+                    for (int e = 0; e < EG; ++e) acc2[q][e] = b;
                 }
                 auto fma_row2 = [&](const float* wrow, const float* xrow) {
                     unsigned long long w2[OP / 2];
@@ -217,34 +247,41 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
                         w2[2 * q] = f2pack(v.x, v.y);
                         w2[2 * q + 1] = f2pack(v.z, v.w);
                     }
-                    const float4 x0 = *reinterpret_cast<const float4*>(xrow + 8 * tx);
-                    const float4 x1 = *reinterpret_cast<const float4*>(xrow + 8 * tx + 4);
-                    const float x[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+                    float x[EG];
+                    if constexpr (EPW == 32) {
+                        const float4 x0 = *reinterpret_cast<const float4*>(xrow + 8 * tx);
+                        const float4 x1 = *reinterpret_cast<const float4*>(xrow + 8 * tx + 4);
+                        x[0] = x0.x; x[1] = x0.y; x[2] = x0.z; x[3] = x0.w;
+                        x[4] = x1.x; x[5] = x1.y; x[6] = x1.z; x[7] = x1.w;
+                    } else {
+                        const float2 x0 = *reinterpret_cast<const float2*>(xrow + 2 * tx);
+                        x[0] = x0.x; x[1] = x0.y;
+                    }
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) {
+                    for (int e = 0; e < EG; ++e) {
                         const unsigned long long xb = f2pack(x[e], x[e]);
 #pragma unroll
                         for (int q = 0; q < OP / 2; ++q) acc2[q][e] = f2fma(w2[q], xb, acc2[q][e]);
                     }
                 };
-#pragma unroll 2
-                for (int k = 0; k < 18; ++k) fma_row2(sW1 + k * H, sObs + k * 32);
+#pragma unroll (EPW == 32 ? 2 : 3)
+                for (int k = 0; k < 18; ++k) fma_row2(sW1 + k * H, sObs + k * EPW);
                 for (int i = 1; i <= nh; ++i) {
                     const int base = 18 + 4 * (int)((t - (uint32_t)i) & 15u);
                     const int kw = 18 + 4 * (i - 1);
 #pragma unroll
-                    for (int c = 0; c < 4; ++c) fma_row2(sW1 + (kw + c) * H, sObs + (base + c) * 32);
+                    for (int c = 0; c < 4; ++c) fma_row2(sW1 + (kw + c) * H, sObs + (base + c) * EPW);
                 }
 #pragma unroll
                 for (int q = 0; q < OP / 2; ++q)
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) f2unpack(acc2[q][e], acc[2 * q][e], acc[2 * q + 1][e]);
+                    for (int e = 0; e < EG; ++e) f2unpack(acc2[q][e], acc[2 * q][e], acc[2 * q + 1][e]);
             } else {
 #pragma unroll
             for (int i = 0; i < OP; ++i) {
                 const float b = smem[L::B1 + ty * OP + i];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) acc[i][e] = b;
+                for (int e = 0; e < EG; ++e) acc[i][e] = b;
             }
             auto fma_row = [&](const float* wrow, const float* xrow) {
                 float w[OP];
@@ -259,7 +296,7 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
 #pragma unroll
                 for (int i = 0; i < OP; ++i)
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) acc[i][e] = fmaf(w[i], x[e], acc[i][e]);
+                    for (int e = 0; e < EG; ++e) acc[i][e] = fmaf(w[i], x[e], acc[i][e]);
             };
 #pragma unroll 2
             for (int k = 0; k < 18; ++k) fma_row(sW1 + k * H, sObs + k * 32);
@@ -273,30 +310,35 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
 #pragma unroll
             for (int i = 0; i < OP; ++i) {
                 const int o = ty * OP + i;
-                float* row = sHid + o * 32;
+                float* row = sHid + o * EPW + ty * L::SKEW;
+                if constexpr (EPW != 32) {
+                    *reinterpret_cast<float2*>(row + 2 * tx) = make_float2(fmaxf(acc[i][0], 0.f), fmaxf(acc[i][1], 0.f));
+                    continue;
+                } else {
                 const float4 v0 = make_float4(fmaxf(acc[i][0], 0.f), fmaxf(acc[i][1], 0.f),
                                               fmaxf(acc[i][2], 0.f), fmaxf(acc[i][3], 0.f));
                 const float4 v1 = make_float4(fmaxf(acc[i][4], 0.f), fmaxf(acc[i][5], 0.f),
                                               fmaxf(acc[i][6], 0.f), fmaxf(acc[i][7], 0.f));
                 *reinterpret_cast<float4*>(row + 4 * ((2 * tx) ^ ty)) = v0;
                 *reinterpret_cast<float4*>(row + 4 * ((2 * tx + 1) ^ ty)) = v1;
+                }
             }
             __syncwarp();
             // ---------------- layer 2: H -> H, ReLU (in registers)
             if constexpr (PK) {
-                unsigned long long acc2[OP / 2][8];
+                unsigned long long acc2[OP / 2][EG];
 #pragma unroll
                 for (int q = 0; q < OP / 2; ++q) {
                     const unsigned long long b = f2pack(smem[L::B2 + ty * OP + 2 * q],
                                                         smem[L::B2 + ty * OP + 2 * q + 1]);
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) acc2[q][e] = b;
+                    for (int e = 0; e < EG; ++e) acc2[q][e] = b;
                 }
-#pragma unroll 2
+#pragma unroll (EPW == 32 ? 2 : 4)
                 for (int k = 0; k < H; ++k) {
                     const float* wrow = sW2 + k * H;
-                    const float* xrow = sHid + k * 32;
                     const int sw = (k / OP) & 7;
+                    const float* xrow = sHid + k * EPW + sw * L::SKEW;
                     unsigned long long w2[OP / 2];
 #pragma unroll
                     for (int q = 0; q < NQ; ++q) {
@@ -304,11 +346,18 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
                         w2[2 * q] = f2pack(v.x, v.y);
                         w2[2 * q + 1] = f2pack(v.z, v.w);
                     }
-                    const float4 x0 = *reinterpret_cast<const float4*>(xrow + 4 * ((2 * tx) ^ sw));
-                    const float4 x1 = *reinterpret_cast<const float4*>(xrow + 4 * ((2 * tx + 1) ^ sw));
-                    const float x[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+                    float x[EG];
+                    if constexpr (EPW == 32) {
+                        const float4 x0 = *reinterpret_cast<const float4*>(xrow + 4 * ((2 * tx) ^ sw));
+                        const float4 x1 = *reinterpret_cast<const float4*>(xrow + 4 * ((2 * tx + 1) ^ sw));
+                        x[0] = x0.x; x[1] = x0.y; x[2] = x0.z; x[3] = x0.w;
+                        x[4] = x1.x; x[5] = x1.y; x[6] = x1.z; x[7] = x1.w;
+                    } else {
+                        const float2 x0 = *reinterpret_cast<const float2*>(xrow + 2 * tx);
+                        x[0] = x0.x; x[1] = x0.y;
+                    }
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) {
+                    for (int e = 0; e < EG; ++e) {
                         const unsigned long long xb = f2pack(x[e], x[e]);
 #pragma unroll
                         for (int q = 0; q < OP / 2; ++q) acc2[q][e] = f2fma(w2[q], xb, acc2[q][e]);
@@ -317,13 +366,13 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
 #pragma unroll
                 for (int q = 0; q < OP / 2; ++q)
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) f2unpack(acc2[q][e], acc[2 * q][e], acc[2 * q + 1][e]);
+                    for (int e = 0; e < EG; ++e) f2unpack(acc2[q][e], acc[2 * q][e], acc[2 * q + 1][e]);
             } else {
 #pragma unroll
             for (int i = 0; i < OP; ++i) {
                 const float b = smem[L::B2 + ty * OP + i];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) acc[i][e] = b;
+                for (int e = 0; e < EG; ++e) acc[i][e] = b;
             }
 #pragma unroll 2
             for (int k = 0; k < H; ++k) {
@@ -342,20 +391,20 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
 #pragma unroll
                 for (int i = 0; i < OP; ++i)
 #pragma unroll
-                    for (int e = 0; e < 8; ++e) acc[i][e] = fmaf(w[i], x[e], acc[i][e]);
+                    for (int e = 0; e < EG; ++e) acc[i][e] = fmaf(w[i], x[e], acc[i][e]);
             }
             }
             // ---------------- layer 3: H -> 4, partial over this lane's H/8 units
-            float pp[4][8];
+            float pp[4][EG];
 #pragma unroll
             for (int j = 0; j < 4; ++j)
 #pragma unroll
-                for (int e = 0; e < 8; ++e) pp[j][e] = 0.0f;
+                for (int e = 0; e < EG; ++e) pp[j][e] = 0.0f;
 #pragma unroll
             for (int i = 0; i < OP; ++i) {
                 const float4 w3 = *reinterpret_cast<const float4*>(sW3 + (ty * OP + i) * 4);
 #pragma unroll
-                for (int e = 0; e < 8; ++e) {
+                for (int e = 0; e < EG; ++e) {
                     const float h = fmaxf(acc[i][e], 0.0f);
                     pp[0][e] = fmaf(w3.x, h, pp[0][e]);
                     pp[1][e] = fmaf(w3.y, h, pp[1][e]);
@@ -364,6 +413,20 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
                 }
             }
             // butterfly reduce-scatter over ty: lane ends with env 8*tx + ty == lane
+            float mu[4];
+            if constexpr (EPW != 32) {
+                // the same sums (ty with ty ^ 4, then ^ 2, then ^ 1) for both envs on every lane
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+#pragma unroll
+                    for (int e = 0; e < EG; ++e) {
+                        pp[j][e] += __shfl_xor_sync(0xffffffffu, pp[j][e], 4);
+                        pp[j][e] += __shfl_xor_sync(0xffffffffu, pp[j][e], 2);
+                        pp[j][e] += __shfl_xor_sync(0xffffffffu, pp[j][e], 1);
+                    }
+                    mu[j] = tanhf(((ty & 1) ? pp[j][1] : pp[j][0]) + smem[L::B3 + j]);
+                }
+            } else {
             float q4[4][4];
             {
                 const bool hi = (ty & 4) != 0;
@@ -388,7 +451,6 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
                         q2[j][e] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
                     }
             }
-            float mu[4];
             {
                 const bool hi = (ty & 1) != 0;
 #pragma unroll
@@ -397,6 +459,7 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
                     const float keep = hi ? q2[j][1] : q2[j][0];
                     mu[j] = tanhf(keep + __shfl_xor_sync(0xffffffffu, send, 1) + smem[L::B3 + j]);
                 }
+            }
             }
             if (!TRACK && sigma > 0.0f) {
                 const uint4 r0 = draw(C, (uint32_t)g, t, TAG_EXPL, 0);
@@ -438,7 +501,7 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
             if (nh > 0) {
                 const int hs = 18 + 4 * (int)(t & 15u);
 #pragma unroll
-                for (int c = 0; c < 4; ++c) sObs[(hs + c) * 32 + lane] = a[c];
+                for (int c = 0; c < 4; ++c) sObs[(hs + c) * EPW + eo] = a[c];
             }
             __syncwarp();
             continue;
@@ -449,7 +512,7 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
         const bool trunc = !term && (int)ep_after >= C.episode_len;
         // ---------------- transition record (field-major, streaming stores)
         if (capacity > 0) {
-            if (in_bounds(p.status, slot, p.rows, SITE_RING_WRITE) && in_bounds(p.status, g, ld, SITE_SOA)) {
+            if (own && in_bounds(p.status, slot, p.rows, SITE_RING_WRITE) && in_bounds(p.status, g, ld, SITE_SOA)) {
                 float* rec = p.rec + (size_t)slot * F * ld + g;
 #pragma unroll
                 for (int i = 0; i < NS; ++i) __stcs(rec + i * ld, s[i]);
@@ -474,7 +537,7 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
         if (nh > 0) {
             const int hs = 18 + 4 * (int)(t & 15u);
 #pragma unroll
-            for (int c = 0; c < 4; ++c) sObs[(hs + c) * 32 + lane] = a[c];
+            for (int c = 0; c < 4; ++c) sObs[(hs + c) * EPW + eo] = a[c];
         }
         ep_ret += r;
         if (term || trunc) {
@@ -485,7 +548,7 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
             float prm7[7];
             reset_env(C, (uint32_t)g, ep_index, s, prm7, d);
             P = make_prm(prm7[0], prm7[1], prm7[2], prm7[3], prm7[4], prm7[5], prm7[6]);
-            for (int k = 18; k < 18 + 4 * HMAX; ++k) sObs[k * 32 + lane] = 0.0f;
+            for (int k = 18; k < 18 + 4 * HMAX; ++k) sObs[k * EPW + eo] = 0.0f;
             ep_step = 0;
             ep_ret = 0.0f;
         } else {
@@ -496,6 +559,7 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
         __syncwarp();
     }
 
+    if (!own) return;
     if constexpr (TRACK) {
         tr.sq_err[g] = e3;
         tr.sq_err[ld + g] = exy;
@@ -514,7 +578,7 @@ __global__ void __launch_bounds__(NW * 32) k_rollout(EnvCfg C, EnvPtrs p,
         const int sl = (int)((t_end - (uint32_t)i) & 15u);
 #pragma unroll
         for (int c = 0; c < 4; ++c)
-            p.hist[(4 * (i - 1) + c) * ld + g] = sObs[(18 + 4 * sl + c) * 32 + lane];
+            p.hist[(4 * (i - 1) + c) * ld + g] = sObs[(18 + 4 * sl + c) * EPW + eo];
     }
     p.ep_index[g] = ep_index; p.ep_step[g] = ep_step; p.ep_ret[g] = ep_ret;
     p.n_done[g] = n_done; p.len_sum[g] = len_sum; p.ret_sum[g] = ret_sum;
@@ -540,6 +604,55 @@ static RollFn roll_fn(int hidden, int nw, bool pk = false) {
     if (hidden == 64) return pk ? pick<64, true>(nw) : pick<64, false>(nw);
     if (hidden == 128) return pk ? pick<128, true>(nw) : pick<128, false>(nw);
     return nullptr;
+}
+
+// The 8-envs-per-warp kernel (paired FMA, warps per CTA chosen at launch).
+template <bool TRACK>
+static RollFn roll8_fn(int hidden) {
+    if (hidden == 32) return k_rollout<32, 0, true, TRACK, 8>;
+    if (hidden == 64) return k_rollout<64, 0, true, TRACK, 8>;
+    return k_rollout<128, 0, true, TRACK, 8>;
+}
+
+static size_t roll8_smem(int hidden, int nw) {
+    if (hidden == 32) return RollLayout<32, 8>::bytes(nw);
+    if (hidden == 64) return RollLayout<64, 8>::bytes(nw);
+    return RollLayout<128, 8>::bytes(nw);
+}
+
+static int sm_count(int device) {
+    int sms = 152;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, device);
+    return sms;
+}
+
+// Whether the SIMT rollout of ld envs runs 8 envs per warp, and then with how many warps
+// per CTA (0: no).  A step of one warp is a chain (the GEMMs' shared loads, random blocks,
+// RK4), so few envs gain from four times the warps; once the SMs' warps share the FMA pipe
+// and the shared-memory port, 32 envs per warp are cheaper (a quarter of the weight loads,
+// no repeated dynamics).  Measured for 64 steps with observation noise, 32 / 8 per warp, us:
+// hidden 32 857 / 323 at 1,000 envs, 866 / 652 at 19,456, 872 / 1004 at 24,000; hidden 64
+// 927 / 451 at 1,000, 950 / 607 at 9,728, 957 / 1008 at 16,384; hidden 128 1595 / 729 at
+// 1,000, 1624 / 1196 at 9,728, 1626 / 2369 at 16,384: so up to 16 warps of 8 envs per SM at
+// hidden 32 and 8 above.
+static int roll8_warps(int hidden, int ld, int device) {
+    const int sms = sm_count(device), warps = ld / 8;
+    if (warps > (hidden == 32 ? 16 : 8) * sms) return 0;
+    int nw = 1;
+    while (nw < 8 && warps > nw * sms) nw *= 2;
+    return nw;
+}
+
+static qsim_status launch_roll8(const qsim_handle* h, const float* actor, int hidden, int T, uint32_t t0,
+                                float sigma, int nw, bool track, const TrackArgs& tr, cudaStream_t st) {
+    RollFn fn = track ? roll8_fn<true>(hidden) : roll8_fn<false>(hidden);
+    const size_t smem = roll8_smem(hidden, nw);
+    QCHECK_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)roll8_smem(hidden, 8)));
+    const int warps = h->ld / 8;
+    fn<<<(warps + nw - 1) / nw, nw * 32, smem, st>>>(h->dc, h->p, actor, T, t0, track ? 0 : h->head,
+                                                      track ? 0 : h->capacity, sigma, 0, warps, tr);
+    QCHECK_LAUNCH("k_rollout (8 envs per warp)");
+    return QSIM_OK;
 }
 
 static size_t roll_smem(int hidden, int nw) {
@@ -709,6 +822,15 @@ extern "C" int32_t qsim_rollout_tune(qsim_handle* h, int32_t warps_per_block) {
     return h->rollout_warps;
 }
 
+// The handle's counters after n_steps steps.
+static void advance_steps(qsim_handle* h, int n_steps) {
+    h->t_now += n_steps;
+    if (h->capacity > 0) {
+        h->head = (h->head + n_steps) % h->capacity;
+        h->size = std::min<int64_t>(h->capacity, h->size + n_steps);
+    }
+}
+
 extern "C" qsim_status qsim_rollout(qsim_handle* h, const float* actor, int32_t hidden,
                                     int32_t n_steps, float sigma_e, void* stream) {
     if (!h || !actor) return fail(QSIM_EINVAL, "qsim_rollout: null pointer");
@@ -734,14 +856,15 @@ extern "C" qsim_status qsim_rollout(qsim_handle* h, const float* actor, int32_t 
             chunk = parts > 1 ? 100 : 0;
         }
     }
-    qsim_status s = launch_rollout(h, actor, hidden, n_steps, sigma_e, (cudaStream_t)stream, nw,
-                                   parts, chunk, engine);
+    // few envs on the paired-FMA engine, nothing pinned or tuned: 8 envs per warp
+    const int nw8 = engine == 1 && h->rollout_warps == 0 && h->rollout_parts <= 0 && h->rollout_chunk == 0
+                        ? roll8_warps(hidden, h->ld, h->device) : 0;
+    qsim_status s = nw8 ? launch_roll8(h, actor, hidden, n_steps, (uint32_t)h->t_now, sigma_e, nw8, false,
+                                       TrackArgs{}, (cudaStream_t)stream)
+                        : launch_rollout(h, actor, hidden, n_steps, sigma_e, (cudaStream_t)stream, nw,
+                                         parts, chunk, engine);
     if (s != QSIM_OK) return s;
-    h->t_now += n_steps;
-    if (h->capacity > 0) {
-        h->head = (h->head + n_steps) % h->capacity;
-        h->size = std::min<int64_t>(h->capacity, h->size + n_steps);
-    }
+    advance_steps(h, n_steps);
     return QSIM_OK;
 }
 
@@ -779,20 +902,35 @@ extern "C" int32_t qsim_rollout_autotune(qsim_handle* h, const float* actor, int
                                            pk);
             cudaEventRecord(e1, st);
             if (s != QSIM_OK) { cudaEventDestroy(e0); cudaEventDestroy(e1); return s; }
-            h->t_now += n_steps;
-            if (h->capacity > 0) {
-                h->head = (h->head + n_steps) % h->capacity;
-                h->size = std::min<int64_t>(h->capacity, h->size + n_steps);
-            }
+            advance_steps(h, n_steps);
             cudaEventSynchronize(e1);
             float ms = 0.0f;
             cudaEventElapsedTime(&ms, e0, e1);
             if (ms < best) { best = ms; best_nw = nw; best_parts = sc.parts; best_pk = pk; best_chunk = sc.chunk; }
         }
     }
+    // few envs: 8 envs per warp (what an untuned handle on the paired-FMA engine runs)
+    const int nw8 = roll8_warps(hidden, h->ld, h->device);
+    bool roll8 = false;
+    if (nw8 && h->rollout_packed != 0 && h->rollout_packed != 2 && ((h->t_now + n_steps) >> 32) == 0) {
+        cudaEventRecord(e0, st);
+        const qsim_status s = launch_roll8(h, actor, hidden, n_steps, (uint32_t)h->t_now, -1.0f, nw8, false, TrackArgs{}, st);
+        cudaEventRecord(e1, st);
+        if (s != QSIM_OK) { cudaEventDestroy(e0); cudaEventDestroy(e1); return s; }
+        advance_steps(h, n_steps);
+        cudaEventSynchronize(e1);
+        float ms = 0.0f;
+        cudaEventElapsedTime(&ms, e0, e1);
+        roll8 = ms < best;
+    }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     QCHECK_LAUNCH("qsim_rollout_autotune");
+    if (roll8) {
+        h->rollout_warps = h->rollout_parts = h->rollout_chunk = 0;
+        h->rollout_packed = 1;
+        return nw8;
+    }
     if (best_nw) {
         h->rollout_warps = best_nw;
         h->rollout_parts = best_parts;
@@ -846,6 +984,8 @@ extern "C" qsim_status qsim_track(qsim_handle* h, const float* actor, int32_t hi
     // hidden 64 flies on the tensor-core kernel unless the handle pins a SIMT engine
     if (hidden == 64 && h->rollout_packed != 0 && h->rollout_packed != 1)
         return launch_track_tc(h, actor, n_steps, tr, kTcChunk, (cudaStream_t)stream);
+    if (const int nw8 = h->rollout_packed != 0 ? roll8_warps(hidden, h->ld, h->device) : 0)
+        return launch_roll8(h, actor, hidden, n_steps, 0u, 0.0f, nw8, true, tr, (cudaStream_t)stream);
     constexpr int nw = 4;
     RollFn fn = hidden == 32 ? track_fn<32>() : (hidden == 64 ? track_fn<64>() : track_fn<128>());
     const size_t smem = roll_smem(hidden, nw);

@@ -50,6 +50,32 @@ def test_step_writes_what_observe_reads(gpu, n, n_hist, layout):
         q.qsim_destroy(h)
 
 
+@pytest.mark.parametrize("hidden,n,n_hist,noise", [(32, 1, 16, 0.01), (32, 1000, 16, 0.0), (64, 33, 3, 0.01),
+                                                   (64, 2500, 16, 0.01), (128, 40, 0, 0.01), (128, 1300, 16, 0.01)])
+def test_few_envs_rollout_equals_32_per_warp(gpu, hidden, n, n_hist, noise):
+    """An untuned handle of few envs runs 8 envs per warp; a handle with its warps per block
+    pinned runs 32."""
+    q = gpu
+    outs = []
+    for pinned in (0, 2):
+        d, cfg, veh = lib_config(q, "c2", n_envs=n, capacity=30, learning_starts=2, n_hist=n_hist, episode_len=11,
+                                 sig_p=noise, sig_v=noise, dist_f=0.01)
+        h = q.qsim_create(cfg, veh)
+        try:
+            A = torch.tensor(_actor(d, hidden), device="cuda")
+            q.qsim_rollout_engine(h, 1)
+            if pinned:
+                q.qsim_rollout_tune(h, pinned)
+            q.qsim_rollout(h, A, hidden, 17, 0.1)
+            q.qsim_rollout(h, A, hidden, 9, 0.0)
+            torch.cuda.synchronize()
+            outs.append(_bits(q.qsim_info_get(h), n))
+        finally:
+            q.qsim_destroy(h)
+    for x, y in zip(*outs):
+        assert np.array_equal(x, y)
+
+
 @pytest.mark.parametrize("n", [1, 129, 152 * 128 + 1, 2 * 152 * 128 + 1])
 def test_tensor_core_tiles_per_block_agree(gpu, n):
     """One, two or three tiles per block (chosen by the env count) against two partitions,
