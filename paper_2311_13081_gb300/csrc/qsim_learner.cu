@@ -28,6 +28,7 @@
 #include "qsim_internal.h"
 #include "qsim_recalc.cuh"
 #include "qsim_tcgen05.cuh"
+#include "qsim_tcmlp.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -35,7 +36,9 @@ namespace qsim {
 
 
 constexpr int SMEM_ENGINE = smlp::floats() > smlp::floats2() ? smlp::floats() : smlp::floats2();
-constexpr int SMEM_MAIN = GEMM_SMEM > SMEM_ENGINE ? GEMM_SMEM : SMEM_ENGINE;
+constexpr int SMEM_TC = (tce::SMEM_BYTES + 3) / 4;
+constexpr int SMEM_MAIN = SMEM_TC > SMEM_ENGINE ? SMEM_TC : (GEMM_SMEM > SMEM_ENGINE ? GEMM_SMEM : SMEM_ENGINE);
+static_assert(4 * (SMEM_MAIN + 32) <= 227 * 1024, "learner shared memory");
 // the small-run env step keeps an actor of hidden <= 128 and <= 128 inputs in shared memory
 static_assert(SMEM_MAIN >= 128 * 128 + 128 + 128 * 128 + 128 + 4 * 128 + 4 + 4 + 8 * (132 + 2 * 132 + 4 + 32),
               "learner shared memory too small for the small-run env step");
@@ -156,32 +159,62 @@ __device__ __forceinline__ void cluster_sync_all(int S) {
 struct Scr {
     float *oa, *oa2, *oc, *oc2, *r, *term, *y, *q1, *q2, *mu, *da, *dz3, *X1, *X2, *H1a, *H2a,
         *H1b, *H2b, *dZ2, *dZ1, *ga, *g1, *g2, *loss, *env_obs, *env_h1, *env_h2, *env_mu;
+    // tensor-core passes (in the place of X1 .. dZ1): this CTA's share of the six networks'
+    // halves (net_img), and o_c in FP32 [critic input][Bc] with its rows' sums of magnitudes [Bc]
+    float *img, *x32, *xn;
 };
+enum Net { N_ACTOR, N_ACTOR_T, N_C1, N_C1_T, N_C2, N_C2_T };
+
+// Halves of network n of a run (for the tensor-core passes), from any CTA of its cluster.
+__device__ __forceinline__ unsigned char* net_img(const Scr& S, float* scr_base, size_t scr_stride, int rk, int nS, int H,
+                                                  int n) {
+    const ptrdiff_t at = (ptrdiff_t)(n % nS - rk) * (ptrdiff_t)scr_stride + (S.img - scr_base) +
+                         (ptrdiff_t)(n / nS) * tce::img_floats(H);
+    return reinterpret_cast<unsigned char*>(scr_base + at);
+}
+
+// Networks' halves per CTA of a cluster of nS: network n lies in the scratch of rank n mod nS.
+__host__ __device__ constexpr int imgs_per_cta(int nS) { return (6 + nS - 1) / nS; }
 
 __host__ __device__ inline size_t scratch_floats(int Bc, int H, int DA, int DC, int PA, int PC,
-                                                 int n_env) {
+                                                 int n_env, int nS) {
     size_t f = 0;
-    f += 2 * (size_t)Bc * DA + 2 * (size_t)Bc * DC;  // oa oa2 oc oc2
+    if (tce::shape_ok(Bc, H, DA, DC)) {
+        f += 4 * (size_t)(Bc / tce::TR) * tce::TILE_FLOATS;              // oa oa2 oc oc2: input tiles
+        f += (size_t)(tce::KP + 1) * Bc;                                 // x32 xn
+        f += (size_t)imgs_per_cta(nS) * tce::img_floats(H);              // img
+    } else {
+        f += 2 * (size_t)Bc * DA + 2 * (size_t)Bc * DC;  // oa oa2 oc oc2
+        f += 8 * (size_t)Bc * H;                         // X1 X2 H1a H2a H1b H2b dZ2 dZ1
+    }
     f += 5 * (size_t)Bc;                              // r term y q1 q2
     f += 3 * 4 * (size_t)Bc;                          // mu da dz3
-    f += 8 * (size_t)Bc * H;                          // X1 X2 H1a H2a H1b H2b dZ2 dZ1
     f += (size_t)PA + 2 * (size_t)PC + 8;             // partial grads + loss
     f += (size_t)n_env * (DA + 2 * H + 4);            // env-step tile
     return (f + 31) & ~(size_t)31;
 }
 
-__device__ Scr carve(float* base, int Bc, int H, int DA, int DC, int PA, int PC, int n_env) {
+__device__ Scr carve(float* base, int Bc, int H, int DA, int DC, int PA, int PC, int n_env, int nS, bool tiles) {
     Scr s;
     float* p = base;
     auto take = [&](size_t n) { float* q = p; p += n; return q; };
-    s.oa = take((size_t)Bc * DA); s.oa2 = take((size_t)Bc * DA);
-    s.oc = take((size_t)Bc * DC); s.oc2 = take((size_t)Bc * DC);
+    if (tiles) {  // (all multiples of 32 floats from a 128-byte aligned base)
+        const size_t nt = (size_t)(Bc / tce::TR) * tce::TILE_FLOATS;
+        s.oa = take(nt); s.oa2 = take(nt); s.oc = take(nt); s.oc2 = take(nt);
+        s.img = take((size_t)imgs_per_cta(nS) * tce::img_floats(H));
+        s.x32 = take((size_t)tce::KP * Bc); s.xn = take(Bc);
+        s.X1 = s.X2 = s.H1a = s.H2a = s.H1b = s.H2b = s.dZ2 = s.dZ1 = nullptr;
+    } else {
+        s.oa = take((size_t)Bc * DA); s.oa2 = take((size_t)Bc * DA);
+        s.oc = take((size_t)Bc * DC); s.oc2 = take((size_t)Bc * DC);
+        s.X1 = take((size_t)Bc * H); s.X2 = take((size_t)Bc * H);
+        s.H1a = take((size_t)Bc * H); s.H2a = take((size_t)Bc * H);
+        s.H1b = take((size_t)Bc * H); s.H2b = take((size_t)Bc * H);
+        s.dZ2 = take((size_t)Bc * H); s.dZ1 = take((size_t)Bc * H);
+        s.img = s.x32 = s.xn = nullptr;
+    }
     s.r = take(Bc); s.term = take(Bc); s.y = take(Bc); s.q1 = take(Bc); s.q2 = take(Bc);
     s.mu = take(4 * (size_t)Bc); s.da = take(4 * (size_t)Bc); s.dz3 = take(4 * (size_t)Bc);
-    s.X1 = take((size_t)Bc * H); s.X2 = take((size_t)Bc * H);
-    s.H1a = take((size_t)Bc * H); s.H2a = take((size_t)Bc * H);
-    s.H1b = take((size_t)Bc * H); s.H2b = take((size_t)Bc * H);
-    s.dZ2 = take((size_t)Bc * H); s.dZ1 = take((size_t)Bc * H);
     s.ga = take(PA); s.g1 = take(PC); s.g2 = take(PC); s.loss = take(8);
     s.env_obs = take((size_t)n_env * DA); s.env_h1 = take((size_t)n_env * H);
     s.env_h2 = take((size_t)n_env * H); s.env_mu = take((size_t)n_env * 4);
@@ -623,197 +656,236 @@ __device__ __forceinline__ int64_t ring(int64_t a, int64_t m) {
     return a < 0 ? a + m : (a >= m ? a - m : a);
 }
 
-// Gather samples [g0, g0 + G) (G <= 32) of this CTA's share of the minibatch: rebuilds o_a,
-// o_a', o_c (with the stored action), o_c' (action slot filled later), r and the
-// termination flag from the compact replay records.  Lane l handles sample g0 + l; warp 0
-// builds the s_t part, warp 1 the s_{t+1} part and warps 2..7 the action history, each
-// into a shared-memory tile laid out like the scratch rows, which is then written out with
-// coalesced stores.
-__device__ __noinline__ void gather_group(const RunDesc& R, int j0, int g0, int G, uint32_t u,
-                                          int64_t head, int64_t size, int64_t t_now, const Scr& S,
-                                          float* tile) {
+// ------------------------------------------------------------------------ replay gather
+// Rebuilds o_a, o_a', o_c (with the stored action), o_c' (action slot filled later), r and
+// the termination flag of this CTA's samples from the compact replay records, up to GS
+// samples a pass.  A sample is ~110 scattered 4-byte values (state, successor state, 17
+// actions), each its own 32-byte sector and, with rings beyond L2, its own DRAM access: what
+// bounds the pass is how many of them are in flight.  So all samples' indices and flags
+// come first (one round trip), then every value goes straight from the ring to shared
+// memory with asynchronous copies (no registers, nothing waited for in between; entries
+// before the episode start are zero-filled by the copy), and only then the observations are
+// formed and written out as coalesced rows.  256 samples on one CTA, values alone: 107 us
+// with the ring in DRAM and every SM at it, 27 us from L2 (two cycles a sector, the rate of
+// the load path); with the rows 140 and 57 us, against 177 and 72 us for one group of 32
+// samples after another through registers.
+namespace gat {
+constexpr int GS = 256, GP = GS + 1;  // samples a pass; row stride (odd: lanes along rows are conflict-free)
+// rows of the shared tile [row][sample]: s, s', a_t, the lags, privileged values, reward,
+// then the 18 observation entries of s and s' without and with the actor's noise
+constexpr int R_S = 0, R_S2 = NS, R_A = 2 * NS, R_L = R_A + 4, R_PV = R_L + 4 * HMAX, R_R = R_PV + NPRIV,
+              R_O = R_R + 1, R_O2 = R_O + 18, R_ON = R_O2 + 18, R_ON2 = R_ON + 18, ROWS = R_ON2 + 18;
+constexpr int MAPS = 128;  // entries of a column map (input widths are below that)
+static_assert(ROWS * GP + 3 * GS + 4 * MAPS / 2 <= SMEM_MAIN, "gather tile");
+
+// 4 bytes global -> shared, zero when !ok (nothing is read then)
+__device__ __forceinline__ void cp4(float* dst, const float* src, bool ok) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;"
+                 :: "r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 4 : 0) : "memory");
+}
+}  // namespace gat
+
+template <bool TILES>
+__device__ __noinline__ void gather_pass(const RunDesc& R, int j0, int Bc, int g0, int G, uint32_t u, int64_t head,
+                                         int64_t size, int64_t t_now, const Scr& S, float* sm) {
+    using namespace gat;
     const EnvCfg& C = R.C;
     const int ld = C.ld, F = C.F, NE = R.n_env, DA = R.DA, DC = R.DC, nh = C.n_hist;
     const int64_t CAP = R.capacity;
-    const int w = threadIdx.x >> 5, jl = threadIdx.x & 31;
-    float* T_oa = tile;
-    float* T_oa2 = T_oa + (size_t)G * DA;
-    float* T_oc = T_oa2 + (size_t)G * DA;
-    float* T_oc2 = T_oc + (size_t)G * DC;
-    float* T_r = T_oc2 + (size_t)G * DC;
-    float* T_term = T_r + G;
-    int* T_env = reinterpret_cast<int*>(T_term + G);  // sample's env (-1: skipped) and t_rec,
-    uint32_t* T_trec = reinterpret_cast<uint32_t*>(T_env + G);  // for the noise pass
+    const int tid = threadIdx.x;
+    float* tile = sm;
+    int* m_env = reinterpret_cast<int*>(sm + ROWS * GP);                 // sample's env (-1: skipped),
+    uint32_t* m_slot = reinterpret_cast<uint32_t*>(m_env + GS);          // slot,
+    uint32_t* m_flag = m_slot + GS;                                      // and flags
+    int16_t* map = reinterpret_cast<int16_t*>(m_flag + GS);              // tile row of o_a, o_a', o_c, o_c' column k
     int* const bst = R.E.status;
     const int64_t rows = R.E.rows;
-    if (jl < G) {
+    const int64_t lost = size == CAP ? nh : 0;
+    const int64_t first = head - size + lost;  // ring position of sample index 0 (before wrapping)
+    // ---- column maps
+    for (int k = tid; k < MAPS; k += LT) {
+        const bool noisy = C.any_noise != 0;
+        map[k] = (int16_t)(k < 18 ? (noisy ? R_ON : R_O) + k : R_L + k - 18);
+        map[MAPS + k] = (int16_t)(k < 18 ? (noisy ? R_ON2 : R_O2) + k : R_A + k - 18);
+        int c = -1, c2 = -1;
+        const int act = k - (DC - 4);
+        if (act >= 0) {
+            c = R_A + act;  // o_c' gets the target action later
+        } else if (C.critic_layout == 3) {
+            c = map[k];
+            c2 = map[MAPS + k];
+        } else {
+            const int x = k - (C.critic_layout == 2 ? 18 : DA);  // position past observation (and history)
+            if (k < 18) { c = R_O + k; c2 = R_O2 + k; }
+            else if (x < 0) { c = R_L + k - 18; c2 = R_A + k - 18; }
+            else if (x < 4) { c = R_S + 13 + x; c2 = R_S2 + 13 + x; }
+            else { c = c2 = R_PV + x - 4; }
+        }
+        map[2 * MAPS + k] = (int16_t)c;
+        map[3 * MAPS + k] = (int16_t)c2;
+    }
+    // ---- indices and flags
+    for (int jl = tid; jl < G; jl += LT) {
         const int j = j0 + g0 + jl;
-        const int64_t lost = size == CAP ? nh : 0;
         const uint32_t nvalid = (uint32_t)((size - 1 - lost) * NE);
         const uint4 rr = draw(C, (uint32_t)j >> 2, u, TAG_REPLAY, 0);
         const uint32_t x = (j & 3) == 0 ? rr.x : ((j & 3) == 1 ? rr.y : ((j & 3) == 2 ? rr.z : rr.w));
         const uint32_t idx = (uint32_t)(((uint64_t)x * (uint64_t)nvalid) >> 32);
-        if (w == 0 && R.idx_log) R.idx_log[j] = idx;
-        const int64_t k = idx / (uint32_t)NE;
-        const int env = (int)(idx % (uint32_t)NE);
-        const int64_t slot = ring(head - size + lost + k, CAP);
-        const uint32_t t_rec = (uint32_t)(t_now - size + lost + k);
+        if (R.idx_log) R.idx_log[j] = idx;
+        const uint32_t k = idx / (uint32_t)NE;
+        const int env = (int)(idx - k * (uint32_t)NE);
+        const int64_t slot = ring(first + k, CAP);
         // (debug builds) a slot or env outside the ring skips the sample, status set
-        const bool sample_ok = in_bounds(bst, slot, rows, SITE_RING_READ) && in_bounds(bst, env, ld, SITE_SOA);
-        if (w == 0) {
-            T_env[jl] = sample_ok ? env : -1;
-            T_trec[jl] = t_rec;
+        const bool ok = in_bounds(bst, slot, rows, SITE_RING_READ) && in_bounds(bst, env, ld, SITE_SOA);
+        m_env[jl] = ok ? env : -1;
+        m_slot[jl] = (uint32_t)slot;
+        const uint32_t fl = ok ? __float_as_uint(ldcg(R.E.rec + ((size_t)slot * F + 22) * ld + env)) : 0u;
+        m_flag[jl] = fl;
+        S.term[g0 + jl] = (fl & 1u) ? 1.0f : 0.0f;
+    }
+    __syncthreads();
+    // ---- every value of every sample, asynchronously: tps threads share a sample
+    int gp = 16;  // samples covered by the CTA at once (a power of two)
+    while (gp < G) gp *= 2;
+    const int tps = LT / gp, jl = tid & (gp - 1), sub = tid / gp;
+    if (jl < G && m_env[jl] >= 0) {
+        const int env = m_env[jl];
+        const int64_t slot = m_slot[jl];
+        const uint32_t fl = m_flag[jl], ep = fl >> 8;
+        const bool done = (fl & 3u) != 0;
+        const int64_t nslot = ring(slot + 1, CAP);
+        const bool nxt_ok = done || in_bounds(bst, nslot, rows, SITE_RING_READ);
+        float* T = tile + jl;
+        const float* rec = R.E.rec + (size_t)slot * F * ld + env;
+        // the side slot is env-major (an env's 17 values contiguous), the records field-major
+        const float* src2 = done ? R.E.side + ((size_t)slot * ld + env) * NS : R.E.rec + (size_t)nslot * F * ld + env;
+        const size_t st2 = done ? 1 : (size_t)ld;
+        for (int i = sub; i < NS; i += tps) {
+            cp4(T + (R_S + i) * GP, rec + (size_t)i * ld, true);
+            cp4(T + (R_S2 + i) * GP, nxt_ok ? src2 + i * st2 : rec, nxt_ok);
         }
-        if (sample_ok) {
-            const float* rec = R.E.rec + (size_t)slot * F * ld + env;
-            const uint32_t fl = __float_as_uint(ldcg(rec + 22 * ld));
-            const bool done = (fl & 3u) != 0;
-            const uint32_t ep = fl >> 8;
-            float* oa = T_oa + (size_t)jl * DA;
-            float* oa2 = T_oa2 + (size_t)jl * DA;
-            float* oc = T_oc + (size_t)jl * DC;
-            float* oc2 = T_oc2 + (size_t)jl * DC;
-            const bool nxt_ok = w != 1 || done || in_bounds(bst, ring(slot + 1, CAP), rows, SITE_RING_READ);
-            if (w < 2 && nxt_ok) {
-                // w == 0: s_t -> o_a, o_c (+ stored action, reward, flag); w == 1: s_{t+1} -> o_a', o_c'
-                // the side slot is env-major (an env's 17 values contiguous), the records field-major
-                const bool from_side = w == 1 && done;
-                const float* src = w == 0 ? rec
-                                          : (from_side ? R.E.side + ((size_t)slot * ld + env) * NS
-                                                       : R.E.rec + (size_t)ring(slot + 1, CAP) * F * ld + env);
-                const size_t sst = from_side ? 1 : (size_t)ld;
-                float st[NS], a[4], pv[NPRIV];
+        // a_t and the lags i = 1..n_hist; zeros before the episode start
+        for (int i = sub; i <= nh; i += tps) {
+            const int64_t sl = ring(slot - i, CAP);
+            const bool ok = i == 0 || ((uint32_t)i <= ep && in_bounds(bst, sl, rows, SITE_RING_READ));
+            const float* ap = ok ? R.E.rec + ((size_t)sl * F + 17) * ld + env : rec;
 #pragma unroll
-                for (int i = 0; i < NS; ++i) st[i] = ldcg(src + i * sst);
-#pragma unroll
-                for (int i = 0; i < 4; ++i) a[i] = w == 0 ? ldcg(rec + (17 + i) * ld) : 0.0f;
-#pragma unroll
-                for (int q = 0; q < NPRIV; ++q) pv[q] = C.n_priv ? ldcg(rec + (23 + q) * ld) : 0.0f;
-                const float r = w == 0 ? ldcg(rec + 21 * ld) : 0.0f;
-                float* ocx = w == 0 ? oc : oc2;
-                float* oax = w == 0 ? oa : oa2;
-                float o[18];
-                obs_state(st, o);
-                // critic observations (noise-free; the symmetric layout 3 copies the actor's
-                // noisy observation below)
-                if (C.critic_layout != 3) {
-#pragma unroll
-                    for (int q = 0; q < 18; ++q) ocx[q] = o[q];
-                    const int rpm_at = C.critic_layout == 2 ? 18 : DA;
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) ocx[rpm_at + i] = rpm_norm(C.veh, st[13 + i]);
-                    if (C.critic_layout != 0) {
-#pragma unroll
-                        for (int q = 0; q < 6; ++q) ocx[rpm_at + 4 + q] = pv[q];
-                    }
-                }
-                if (w == 0) {
-#pragma unroll
-                    for (int i = 0; i < 4; ++i) oc[DC - 4 + i] = a[i];
-                    T_r[jl] = r;
-                    T_term[jl] = (fl & 1u) ? 1.0f : 0.0f;
-                }
-                // the observation noise is added by all warps below
-#pragma unroll
-                for (int q = 0; q < 18; ++q) oax[q] = o[q];
-                if (C.critic_layout == 3) {
-#pragma unroll
-                    for (int q = 0; q < 18; ++q) ocx[q] = o[q];
-                }
-            } else if (w >= 2) {
-                // history: o_a has a_{t-1..t-NH}, o_a' has a_t, a_{t-1..t-NH+1}; zeros before the
-                // episode start.  Warp w handles lags i = w-1, w+5, w+11, all their loads issued
-                // before the first store.
-                static_assert(HMAX <= 18, "history lags: at most 3 per warp of 6");
-                float h[3][4], h2[3][4];
-#pragma unroll
-                for (int u3 = 0; u3 < 3; ++u3) {
-                    const int i = w - 1 + 6 * u3;
-                    const bool lag = i <= nh;
-                    const bool ok = lag && (uint32_t)i <= ep &&
-                                    in_bounds(bst, ring(slot - i, CAP), rows, SITE_RING_READ);
-                    const bool ok2 = lag && (i == 1 || ((uint32_t)(i - 1) <= ep &&
-                                                        in_bounds(bst, ring(slot - i + 1, CAP), rows, SITE_RING_READ)));
-                    const float* ap = R.E.rec + (size_t)ring(slot - i, CAP) * F * ld + env + 17 * ld;
-                    const float* ap2 = i == 1 ? rec + 17 * ld
-                                              : R.E.rec + (size_t)ring(slot - i + 1, CAP) * F * ld + env + 17 * ld;
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        h[u3][c] = ok ? ldcg(ap + c * ld) : 0.0f;
-                        h2[u3][c] = ok2 ? ldcg(ap2 + c * ld) : 0.0f;
-                    }
-                }
-#pragma unroll
-                for (int u3 = 0; u3 < 3; ++u3) {
-                    const int i = w - 1 + 6 * u3;
-                    if (i > nh) continue;
-#pragma unroll
-                    for (int c = 0; c < 4; ++c) {
-                        const int q = 18 + 4 * (i - 1) + c;
-                        oa[q] = h[u3][c];
-                        oa2[q] = h2[u3][c];
-                        if (C.critic_layout != 2) {
-                            oc[q] = h[u3][c];
-                            oc2[q] = h2[u3][c];
-                        }
-                    }
-                }
-            }
+            for (int c = 0; c < 4; ++c) cp4(T + (R_A + 4 * i + c) * GP, ap + (ok ? c * ld : 0), ok);
         }
+        if (sub == tps - 1) {
+            cp4(T + R_R * GP, rec + (size_t)21 * ld, true);
+            for (int k = 0; k < C.n_priv; ++k) cp4(T + (R_PV + k) * GP, rec + (size_t)(23 + k) * ld, true);
+        }
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    // ---- observations, one (sample, side) per thread
+    for (int i = tid; i < 2 * G; i += LT) {
+        const int side = i >= G, js = i - side * G;
+        if (m_env[js] < 0) continue;
+        float* T = tile + js;
+        float* st = T + (side ? R_S2 : R_S) * GP;
+        float sv[NS], o[18];
+#pragma unroll
+        for (int q = 0; q < NS; ++q) sv[q] = st[q * GP];
+        obs_state(sv, o);
+        float* ot = T + (side ? R_O2 : R_O) * GP;
+#pragma unroll
+        for (int q = 0; q < 18; ++q) ot[q * GP] = o[q];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) st[(13 + q) * GP] = rpm_norm(C.veh, sv[13 + q]);
+        if (side == 0) S.r[g0 + js] = T[R_R * GP];
     }
     __syncthreads();
     if (C.any_noise) {
         // the actor's observation noise of s_t (side 0, step t_rec) and s_{t+1} (side 1, step
-        // t_rec + 1): 9 Philox blocks per side, the 18 (side, block) pairs over the 8 warps
-        if (jl < G && T_env[jl] >= 0) {
-            const uint32_t env = (uint32_t)T_env[jl], t_rec = T_trec[jl];
-            for (int pr = w; pr < 18; pr += LT / 32) {
-                const int side = pr >= 9, blk = pr - 9 * side;
-                float n0, n1;
-                obs_noise_pair(C, env, t_rec + (uint32_t)side, blk, n0, n1);
-                float* oax = (side ? T_oa2 : T_oa) + (size_t)jl * DA;
-                oax[2 * blk] += n0;
-                oax[2 * blk + 1] += n1;
-                if (C.critic_layout == 3) {
-                    float* ocx = (side ? T_oc2 : T_oc) + (size_t)jl * DC;
-                    ocx[2 * blk] += n0;
-                    ocx[2 * blk + 1] += n1;
-                }
-            }
+        // t_rec + 1): 9 Philox blocks per side
+        for (int i = tid; i < 18 * G; i += LT) {
+            const int pr = i / G, js = i - pr * G, side = pr >= 9, blk = pr - 9 * side;
+            if (m_env[js] < 0) continue;
+            int64_t k = (int64_t)m_slot[js] - first;  // sample index's time slot
+            while (k < 0) k += CAP;
+            while (k >= CAP) k -= CAP;
+            float n0, n1;
+            obs_noise_pair(C, (uint32_t)m_env[js], (uint32_t)(t_now - size + lost + k) + (uint32_t)side, blk, n0, n1);
+            const float* ot = tile + ((side ? R_O2 : R_O) + 2 * blk) * GP + js;
+            float* nt = tile + ((side ? R_ON2 : R_ON) + 2 * blk) * GP + js;
+            nt[0] = ot[0] + n0;
+            nt[GP] = ot[GP] + n1;
         }
         __syncthreads();
     }
-    // coalesced write-out of the six scratch ranges of this group
-    const int n1 = G * DA, n2 = G * DC;
-    for (int i = threadIdx.x; i < n1; i += LT) {
-        S.oa[(size_t)g0 * DA + i] = T_oa[i];
-        S.oa2[(size_t)g0 * DA + i] = T_oa2[i];
-    }
-    for (int i = threadIdx.x; i < n2; i += LT) {
-        S.oc[(size_t)g0 * DC + i] = T_oc[i];
-        S.oc2[(size_t)g0 * DC + i] = T_oc2[i];
-    }
-    if (threadIdx.x < G) {
-        S.r[g0 + threadIdx.x] = T_r[threadIdx.x];
-        S.term[g0 + threadIdx.x] = T_term[threadIdx.x];
+    // ---- rows of the scratch
+    const int warp = tid >> 5, lane = tid & 31;
+    if constexpr (TILES) {
+        // input tiles of the tensor-core passes: lane = sample, 8 columns of one matrix at a
+        // time as hi / lo halves (zero past the input width; a core matrix row is 16 bytes,
+        // 8 samples make 128); o_c' gets the target action later
+        float* const dst[4] = {S.oa, S.oa2, S.oc, S.oc2};
+        for (int js = tid; js < G; js += LT) {
+            float n = 0.0f;
+            if (m_env[js] >= 0)
+                for (int k = 0; k < DC; ++k) n += fabsf(tile[map[2 * MAPS + k] * GP + js]);
+            S.xn[g0 + js] = n;
+        }
+        constexpr int KC = tce::KC1;
+        for (int i = warp; i < 4 * KC * (G / 32); i += LT / 32) {
+            const int js = 32 * (i / (4 * KC)) + lane, q = i % (4 * KC), mat = q / KC, kc = q - mat * KC;
+            const int w = mat < 2 ? DA : (mat == 2 ? DC : DC - 4);
+            float v[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const int k = 8 * kc + e;
+                v[e] = k < w ? tile[map[mat * MAPS + k] * GP + js] : 0.0f;
+            }
+            const int j = g0 + js;
+            if (mat == 2 && m_env[js] >= 0)
+#pragma unroll
+                for (int e = 0; e < 8; ++e) S.x32[(size_t)(8 * kc + e) * Bc + j] = v[e];
+            unsigned char* t = reinterpret_cast<unsigned char*>((mat < 2 ? (mat ? dst[1] : dst[0]) : (mat == 2 ? dst[2] : dst[3])) +
+                                                                (size_t)(j / tce::TR) * tce::TILE_FLOATS);
+            if (m_env[js] >= 0) tce::put8(t, t + 2 * tce::TILE_HALVES, KC, j % tce::TR, 8 * kc, v);
+        }
+    } else {
+        // FP32 rows, a warp per sample, 4 columns per lane and matrix in flight
+        for (int js = warp; js < G; js += LT / 32) {
+            if (m_env[js] < 0) continue;
+            const size_t j = (size_t)(g0 + js);
+            const float* T = tile + js;
+#pragma unroll
+            for (int mat = 0; mat < 4; ++mat) {
+                const int w = mat < 2 ? DA : DC, n = mat == 3 ? DC - 4 : w;
+                float* d = (mat == 0 ? S.oa : (mat == 1 ? S.oa2 : (mat == 2 ? S.oc : S.oc2))) + j * w;
+                float v[4];
+#pragma unroll
+                for (int e = 0; e < 4; ++e) v[e] = lane + 32 * e < n ? T[map[mat * MAPS + lane + 32 * e] * GP] : 0.0f;
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (lane + 32 * e < n) d[lane + 32 * e] = v[e];
+            }
+        }
     }
     __syncthreads();
 }
 
-// Gather of this CTA's Bc samples in groups of 32 (tile: shared memory, free at this point).
+// Gather of this CTA's Bc samples (sm: shared memory, free at this point).
+template <bool TILES>
 __device__ __forceinline__ void gather_all(const RunDesc& R, int j0, int Bc, uint32_t u,
                                            int64_t head, int64_t size, int64_t t_now,
                                            const Scr& S, float* sm) {
-    for (int g0 = 0; g0 < Bc; g0 += 32) gather_group(R, j0, g0, min(32, Bc - g0), u, head, size, t_now, S, sm);
+    for (int g0 = 0; g0 < Bc; g0 += gat::GS)
+        gather_pass<TILES>(R, j0, Bc, g0, min(gat::GS, Bc - g0), u, head, size, t_now, S, sm);
 }
 
 // Adam on parameters [lo, hi) from the sum of S gradient partials (partial s at
 // gpart_base + s * part_stride + goff, summed in the order s = 0..S-1); with tg != nullptr
 // the target copy also takes its Polyak step tg = tau th + (1 - tau) tg from the new th
-// (the fused form of polyak_slice, for steps that update the targets).
+// (the fused form of polyak_slice, for steps that update the targets).  img / timg: halves
+// of the network and its target for the tensor-core passes, kept in step (in, H: its shape).
 __device__ void adam_slice(float* th, const float* gpart_base, size_t part_stride, int S,
                            int goff, float* m, float* v, int lo, int hi, int64_t t,
-                           const LearnHyper& hp, float gscale, float* tg = nullptr) {
+                           const LearnHyper& hp, float gscale, float* tg = nullptr, unsigned char* img = nullptr,
+                           unsigned char* timg = nullptr, int in = 0, int H = 0) {
     const float bc1 = 1.0f - powf(hp.beta1, (float)t);
     const float bc2 = 1.0f - powf(hp.beta2, (float)t);
     const float tau = hp.tau;
@@ -858,7 +930,12 @@ __device__ void adam_slice(float* th, const float* gpart_base, size_t part_strid
             v[i] = vi;
             const float ti = to[k] - hp.lr * (mi / bc1) / (sqrtf(vi / bc2) + hp.eps);
             th[i] = ti;
-            if (tg) tg[i] = fmaf(tau, ti, (1.0f - tau) * tt[k]);
+            if (img) tce::img_put(img, i, in, H, ti);
+            if (tg) {
+                const float gi = fmaf(tau, ti, (1.0f - tau) * tt[k]);
+                tg[i] = gi;
+                if (timg) tce::img_put(timg, i, in, H, gi);
+            }
         }
     }
 }
@@ -900,7 +977,7 @@ __device__ __noinline__ void td3_update(RunDesc& R, int64_t head, int64_t size, 
     const LearnHyper& hp = R.hp;
     const int j0 = rk * Bc;
     // a9: gather
-    gather_all(R, j0, Bc, u, head, size, t_now, S, sm);
+    gather_all<false>(R, j0, Bc, u, head, size, t_now, S, sm);
     __syncthreads();
     // a10: target actor + smoothing
     mlp_fwd(R.actor_t, DA, H, 4, S.oa2, DA, Bc, S.X1, S.X2, S.mu, 4, true, sm);
@@ -1001,197 +1078,6 @@ __device__ __noinline__ void td3_update(RunDesc& R, int64_t head, int64_t size, 
     cluster_sync_all(nS);
 }
 
-// ------------------------------------------------ tensor-core forward pass (tcgen05)
-// Forward of a CTA's Bc rows (Bc a multiple of 128) through a network in -> H -> H -> out
-// (in <= 96, H in {32, 64, 128}): both hidden layers as tcgen05 MMAs (M 128 rows, N = H,
-// K = 16) on fp16 hi/lo operands in shared memory (three products per FP32-accurate
-// product), accumulators in tensor memory; bias, ReLU and the 4- or 1-wide output layer on
-// the CUDA cores.  One thread issues the MMAs and commits them to an mbarrier that every
-// thread waits on (bounded).  Shared memory is the learner's engine region, laid out here
-// per call: W1 hi/lo [H][96], W2 hi/lo [H][H], the tile operand hi/lo (X [128][96], then the
-// first hidden layer [128][H] in place), b1, b2, W3, b3, partial outputs, the mbarrier.
-namespace tcf {
-constexpr int KP = 96, KC1 = KP / 8;
-constexpr int TMEM_COLS = 256;  // D1 [128 x H] at column 0, D2 at column H (H <= 128)
-constexpr int WAIT_POLLS = 1 << 24;
-struct Lay {
-    int w1h, w1l, w2h, w2l, th, tl, b1, b2, w3, b3, part, bar, end;
-};
-__host__ __device__ constexpr Lay lay(int H) {
-    const int w1 = H * KP * 2, w2 = H * H * 2, t = 128 * (H > KP ? H : KP) * 2;
-    Lay L{};
-    L.w1h = 0; L.w1l = w1; L.w2h = 2 * w1; L.w2l = 2 * w1 + w2; L.th = 2 * w1 + 2 * w2; L.tl = L.th + t;
-    L.b1 = L.tl + t; L.b2 = L.b1 + 4 * H; L.w3 = L.b2 + 4 * H; L.b3 = L.w3 + 16 * H;
-    L.part = L.b3 + 16; L.bar = L.part + 2 * 128 * 4 * 4; L.end = L.bar + 16;
-    return L;
-}
-static_assert(lay(128).end <= 4 * SMEM_MAIN, "tensor-core forward: shared memory");
-
-__device__ __forceinline__ bool eligible(const RunDesc& R, int Bc) {
-    return Bc % 128 == 0 && (R.H == 32 || R.H == 64 || R.H == 128) && R.DA <= KP && R.DC <= KP;
-}
-
-// rows of 8 consecutive inputs -> packed hi / lo halves (zero beyond `in`)
-__device__ __forceinline__ void split8(const float* src, int k0, int in, uint4& hi, uint4& lo) {
-    float v[8];
-#pragma unroll
-    for (int e = 0; e < 8; ++e) v[e] = k0 + e < in ? ldcg(src + k0 + e) : 0.0f;
-    uint32_t h[4], l[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) tc::split2(v[2 * e], v[2 * e + 1], h[e], l[e]);
-    hi = make_uint4(h[0], h[1], h[2], h[3]);
-    lo = make_uint4(l[0], l[1], l[2], l[3]);
-}
-}  // namespace tcf
-
-__device__ __noinline__ void tc_forward(const float* W, int in, int H, int out, const float* X, int ldx,
-                                        int Bc, float* Y, int ldy, bool tanh_out, float* sm, uint32_t tmem,
-                                        int* status) {
-    using namespace tcf;
-    unsigned char* smb = reinterpret_cast<unsigned char*>(sm);
-    const Lay L = lay(H);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int KC2 = H / 8;
-    const float* gb1 = W + H * in;
-    const float* gW2 = gb1 + H;
-    const float* gb2 = gW2 + H * H;
-    const float* gW3 = gb2 + H;
-    const float* gb3 = gW3 + out * H;
-    __half* w1h = reinterpret_cast<__half*>(smb + L.w1h);
-    __half* w1l = reinterpret_cast<__half*>(smb + L.w1l);
-    __half* w2h = reinterpret_cast<__half*>(smb + L.w2h);
-    __half* w2l = reinterpret_cast<__half*>(smb + L.w2l);
-    __half* th = reinterpret_cast<__half*>(smb + L.th);
-    __half* tl = reinterpret_cast<__half*>(smb + L.tl);
-    float* b1 = reinterpret_cast<float*>(smb + L.b1);
-    float* b2 = reinterpret_cast<float*>(smb + L.b2);
-    float* W3 = reinterpret_cast<float*>(smb + L.w3);
-    float* b3 = reinterpret_cast<float*>(smb + L.b3);
-    float* part = reinterpret_cast<float*>(smb + L.part);  // [2][128][4]
-    const uint32_t bar = tc::smem_u32(smb + L.bar);
-    // stage the weights as hi / lo halves in the canonical K-major layout
-    for (int i = tid; i < H * KC1; i += LT) {
-        const int n = i / KC1, kc = i - n * KC1;
-        uint4 hi, lo;
-        split8(W + (size_t)n * in, 8 * kc, in, hi, lo);
-        *reinterpret_cast<uint4*>(w1h + tc::cano16(n, 8 * kc, KC1)) = hi;
-        *reinterpret_cast<uint4*>(w1l + tc::cano16(n, 8 * kc, KC1)) = lo;
-    }
-    for (int i = tid; i < H * KC2; i += LT) {
-        const int n = i / KC2, kc = i - n * KC2;
-        uint4 hi, lo;
-        split8(gW2 + (size_t)n * H, 8 * kc, H, hi, lo);
-        *reinterpret_cast<uint4*>(w2h + tc::cano16(n, 8 * kc, KC2)) = hi;
-        *reinterpret_cast<uint4*>(w2l + tc::cano16(n, 8 * kc, KC2)) = lo;
-    }
-    for (int i = tid; i < H; i += LT) {
-        b1[i] = ldcg(gb1 + i);
-        b2[i] = ldcg(gb2 + i);
-    }
-    for (int i = tid; i < out * H; i += LT) W3[i] = ldcg(gW3 + i);
-    if (tid < out) b3[tid] = ldcg(gb3 + tid);
-    if (tid == 0) tc::bar_init(bar, 1);
-    uint32_t phase = 0;
-    const uint32_t idesc = tc::idesc_f16(H);
-    const uint32_t d1 = tmem, d2 = tmem + (uint32_t)H;
-    const uint32_t lane_off = (uint32_t)(32 * (warp & 3)) << 16;
-    const int half = warp >> 2;                 // column half of the epilogues
-    const int r = 32 * (warp & 3) + lane;       // tile row of this thread in the epilogues
-    const int cbeg = half * (H / 2), cend = cbeg + H / 2;
-    for (int t0 = 0; t0 < Bc; t0 += 128) {
-        // input tile -> hi / lo halves
-        for (int i = tid; i < 128 * KC1; i += LT) {
-            const int rr = i / KC1, kc = i - rr * KC1;
-            uint4 hi, lo;
-            split8(X + (size_t)(t0 + rr) * ldx, 8 * kc, in, hi, lo);
-            *reinterpret_cast<uint4*>(th + tc::cano16(rr, 8 * kc, KC1)) = hi;
-            *reinterpret_cast<uint4*>(tl + tc::cano16(rr, 8 * kc, KC1)) = lo;
-        }
-        tc::fence_async_smem();
-        tc::fence_before();
-        __syncthreads();
-        tc::fence_after();
-        if (tid == 0) {
-#pragma unroll
-            for (int j = 0; j < KP / 16; ++j) {
-                const uint32_t ko = (uint32_t)j * 256u;
-                const uint64_t ah = tc::sdesc(tc::smem_u32(th) + ko, KC1), al = tc::sdesc(tc::smem_u32(tl) + ko, KC1);
-                const uint64_t bh = tc::sdesc(tc::smem_u32(w1h) + ko, KC1), bl = tc::sdesc(tc::smem_u32(w1l) + ko, KC1);
-                tc::mma_ss(d1, ah, bh, idesc, j > 0);
-                tc::mma_ss(d1, ah, bl, idesc, 1);
-                tc::mma_ss(d1, al, bh, idesc, 1);
-            }
-            tc::commit(bar);
-        }
-        if (!tc::bar_wait(bar, phase, WAIT_POLLS) && lane == 0 && status) atomicCAS(status, DEV_OK, DEV_TIMEOUT);
-        phase ^= 1u;
-        tc::fence_after();
-        // epilogue 1: bias, ReLU, split -> the tile buffer as the layer-2 operand
-        for (int c0 = cbeg; c0 < cend; c0 += 16) {
-            uint32_t v[16];
-            tc::ld16(d1 + lane_off + (uint32_t)c0, v);
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                uint32_t h[4], l[4];
-#pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int c = c0 + 8 * q + 2 * e;
-                    const float x0 = fmaxf(__uint_as_float(v[8 * q + 2 * e]) + b1[c], 0.0f);
-                    const float x1 = fmaxf(__uint_as_float(v[8 * q + 2 * e + 1]) + b1[c + 1], 0.0f);
-                    tc::split2(x0, x1, h[e], l[e]);
-                }
-                const int off = tc::cano16(r, c0 + 8 * q, KC2);
-                *reinterpret_cast<uint4*>(th + off) = make_uint4(h[0], h[1], h[2], h[3]);
-                *reinterpret_cast<uint4*>(tl + off) = make_uint4(l[0], l[1], l[2], l[3]);
-            }
-        }
-        tc::fence_async_smem();
-        tc::fence_before();
-        __syncthreads();
-        tc::fence_after();
-        if (tid == 0) {
-            for (int j = 0; j < H / 16; ++j) {
-                const uint32_t ko = (uint32_t)j * 256u;
-                const uint64_t ah = tc::sdesc(tc::smem_u32(th) + ko, KC2), al = tc::sdesc(tc::smem_u32(tl) + ko, KC2);
-                const uint64_t bh = tc::sdesc(tc::smem_u32(w2h) + ko, KC2), bl = tc::sdesc(tc::smem_u32(w2l) + ko, KC2);
-                tc::mma_ss(d2, ah, bh, idesc, j > 0);
-                tc::mma_ss(d2, ah, bl, idesc, 1);
-                tc::mma_ss(d2, al, bh, idesc, 1);
-            }
-            tc::commit(bar);
-        }
-        if (!tc::bar_wait(bar, phase, WAIT_POLLS) && lane == 0 && status) atomicCAS(status, DEV_OK, DEV_TIMEOUT);
-        phase ^= 1u;
-        tc::fence_after();
-        // epilogue 2: bias, ReLU, the output layer's partial sums over this warp's columns
-        float po[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-        for (int c0 = cbeg; c0 < cend; c0 += 16) {
-            uint32_t v[16];
-            tc::ld16(d2 + lane_off + (uint32_t)c0, v);
-#pragma unroll
-            for (int e = 0; e < 16; ++e) {
-                const int c = c0 + e;
-                const float h2 = fmaxf(__uint_as_float(v[e]) + b2[c], 0.0f);
-#pragma unroll
-                for (int o = 0; o < 4; ++o)
-                    if (o < out) po[o] = fmaf(W3[o * H + c], h2, po[o]);
-            }
-        }
-#pragma unroll
-        for (int o = 0; o < 4; ++o) part[(half * 128 + r) * 4 + o] = po[o];
-        tc::fence_before();
-        __syncthreads();
-        tc::fence_after();
-        if (tid < 128) {
-            for (int o = 0; o < out; ++o) {
-                const float y = part[tid * 4 + o] + part[(128 + tid) * 4 + o] + b3[o];
-                Y[(size_t)(t0 + tid) * ldy + o] = tanh_out ? tanhf(y) : y;
-            }
-        }
-        __syncthreads();  // the tile buffer and the partials are reused by the next tile
-    }
-}
-
 // One TD3 update with every network pass resident in shared memory (hidden <= 64, or the
 // 128-wide engine shape for HT = 128): same phases and cluster reduction as td3_update.  HT/DAT/DCT fix the hidden width and the
 // actor/critic input widths at compile time (0: taken from the run descriptor), so that the
@@ -1200,7 +1086,7 @@ template <int HT, int DAT, int DCT>
 __device__ __noinline__ void td3_update_smem(RunDesc& R, int64_t head, int64_t size, int64_t t_now,
                                              uint32_t u, int64_t& t_a, int64_t& t_c, const Scr& S,
                                              float* scr_base, size_t scr_stride, int rk, int nS,
-                                             float* sm, uint32_t tmem, bool tmem_ok) {
+                                             float* sm) {
     using namespace smlp;
     const int B = R.B, Bc = B / nS, PA = R.PA, PC = R.PC;
     const int H = HT ? HT : R.H, DA = DAT ? DAT : R.DA, DC = DCT ? DCT : R.DC;
@@ -1210,26 +1096,19 @@ __device__ __noinline__ void td3_update_smem(RunDesc& R, int64_t head, int64_t s
     const int MC = b.mc;
     float* red = sm + SMEM_MAIN;
     // a9: gather
-    gather_all(R, j0, Bc, u, head, size, t_now, S, sm);
+    gather_all<false>(R, j0, Bc, u, head, size, t_now, S, sm);
     __syncthreads();
-    // the pure forward passes (target actor, target critics) on the tensor cores when the
-    // CTA holds whole 128-row tiles
-    const bool tcf_on = tmem_ok && tcf::eligible(R, Bc);
     // With an even cluster whose CTA pairs' rows fit one chunk, the twin critics are split
     // over the two halves: CTA rk runs critic cs = rk / half (target and current) on the
     // rows of the pair (rr, rr + half), rr = rk mod half, read from both owners' scratch.
     const int half = nS >> 1;
-    const bool split = !tcf_on && half > 0 && (nS & 1) == 0 && 2 * Bc <= MC;
+    const bool split = half > 0 && (nS & 1) == 0 && 2 * Bc <= MC;
     const int cs = split ? rk / half : 0, rr = split ? rk - cs * half : rk;
     const ptrdiff_t d0 = (ptrdiff_t)(rr - rk) * (ptrdiff_t)scr_stride;
     const ptrdiff_t d1 = (ptrdiff_t)(rr + half - rk) * (ptrdiff_t)scr_stride;
     // a10: target actor + smoothing
-    if (tcf_on) {
-        tc_forward(R.actor_t, DA, H, 4, S.oa2, DA, Bc, S.mu, 4, true, sm, tmem, R.E.status);
-    } else {
-        stage(R.actor_t, DA, H, 4, b);
-        for (int r0 = 0; r0 < Bc; r0 += MC) forward(DA, H, 4, S.oa2, DA, r0, min(MC, Bc - r0), b, S.mu, 4, true);
-    }
+    stage(R.actor_t, DA, H, 4, b);
+    for (int r0 = 0; r0 < Bc; r0 += MC) forward(DA, H, 4, S.oa2, DA, r0, min(MC, Bc - r0), b, S.mu, 4, true);
     for (int jl = threadIdx.x; jl < Bc; jl += LT) {
         const uint32_t j = (uint32_t)(j0 + jl);
         const uint4 r0 = draw(R.C, j, u, TAG_SMOOTH, 0), r1 = draw(R.C, j, u, TAG_SMOOTH, 1);
@@ -1248,9 +1127,6 @@ __device__ __noinline__ void td3_update_smem(RunDesc& R, int64_t head, int64_t s
         stage(cs ? R.c2_t : R.c1_t, DC, H, 1, b);
         forward2(DC, H, 1, S.oc2 + d0, S.oc2 + d1, DC, Bc, 2 * Bc, b, qt + d0, qt + d1, 1, false);
         cluster_sync_all(nS);  // both target values of the pair's rows are complete
-    } else if (tcf_on) {
-        tc_forward(R.c1_t, DC, H, 1, S.oc2, DC, Bc, S.q1, 1, false, sm, tmem, R.E.status);
-        tc_forward(R.c2_t, DC, H, 1, S.oc2, DC, Bc, S.q2, 1, false, sm, tmem, R.E.status);
     } else {
         stage(R.c1_t, DC, H, 1, b);
         for (int r0 = 0; r0 < Bc; r0 += MC) forward(DC, H, 1, S.oc2, DC, r0, min(MC, Bc - r0), b, S.q1, 1, false);
@@ -1330,14 +1206,9 @@ __device__ __noinline__ void td3_update_smem(RunDesc& R, int64_t head, int64_t s
     cluster_sync_all(nS);
     // a13: delayed actor update through the updated first critic
     if ((int64_t)(u % (uint32_t)hp.policy_delay) != (int64_t)(hp.policy_delay - 1)) return;
-    // mu(o_a) alone (no activations kept): a pure forward pass, on the tensor cores when the
-    // CTA holds whole 128-row tiles
-    if (tcf_on) {
-        tc_forward(R.actor, DA, H, 4, S.oa, DA, Bc, S.mu, 4, true, sm, tmem, R.E.status);
-    } else {
-        stage(R.actor, DA, H, 4, b);
-        for (int r0 = 0; r0 < Bc; r0 += MC) forward(DA, H, 4, S.oa, DA, r0, min(MC, Bc - r0), b, S.mu, 4, true);
-    }
+    // mu(o_a) alone (no activations kept)
+    stage(R.actor, DA, H, 4, b);
+    for (int r0 = 0; r0 < Bc; r0 += MC) forward(DA, H, 4, S.oa, DA, r0, min(MC, Bc - r0), b, S.mu, 4, true);
     for (int i = threadIdx.x; i < Bc * 4; i += LT) {
         const int jl = i >> 2, c = i & 3;
         S.oc[(size_t)jl * DC + DC - 4 + c] = S.mu[i];
@@ -1390,6 +1261,115 @@ __device__ __noinline__ void td3_update_smem(RunDesc& R, int64_t head, int64_t s
     cluster_sync_all(nS);
 }
 
+// One TD3 update with every network pass on the tensor cores (tce::pass): a CTA holds whole
+// 128-sample tiles, at most 96 inputs.  Same phases, random streams and cluster reduction as
+// td3_update.  One CTA, 256 samples at hidden 64, us (SIMT engine -> here): target actor 20
+// -> 13, target critics 34 -> 19, critic regression 156 -> 54, mu 18 -> 11, dQ/da 55 -> 15,
+// actor gradient 105 -> 26; at hidden 128 regression 404 -> 114, actor gradient 234 -> 44.
+template <int H>
+__device__ __noinline__ void td3_update_tc(RunDesc& R, int64_t head, int64_t size, int64_t t_now, uint32_t u,
+                                           int64_t& t_a, int64_t& t_c, const Scr& S, float* scr_base,
+                                           size_t scr_stride, int rk, int nS, float* sm, uint32_t tmem) {
+    using namespace tce;
+    const int B = R.B, Bc = B / nS, PA = R.PA, PC = R.PC, DA = R.DA, DC = R.DC;
+    const LearnHyper& hp = R.hp;
+    const int j0 = rk * Bc;
+    int* const st = R.E.status;
+    float* red = sm + SMEM_MAIN;
+    const float invB = 1.0f / (float)B;
+    gather_all<true>(R, j0, Bc, u, head, size, t_now, S, sm);
+    // target actor + smoothing; the target action goes into o_c' tiles' last columns
+    const float* cl0 = scr_base - (size_t)rk * scr_stride;  // scratch of cluster rank 0
+    auto img = [&](Net n) { return net_img(S, scr_base, scr_stride, rk, nS, H, n); };
+    Args f{};
+    f.Bc = Bc;
+    f.x32 = S.x32;
+    f.xn = S.xn;
+    f.invB = invB;
+    f.W = R.actor_t; f.img = img(N_ACTOR_T); f.in = DA; f.out = 4; f.X = S.oa2; f.Y = S.mu; f.tanh_out = true;
+    pass<H, FWD>(f, sm, tmem, st);
+    for (int jl = threadIdx.x; jl < Bc; jl += LT) {
+        const uint32_t j = (uint32_t)(j0 + jl);
+        const uint4 r0 = draw(R.C, j, u, TAG_SMOOTH, 0), r1 = draw(R.C, j, u, TAG_SMOOTH, 1);
+        const float z[4] = {gauss(r0.x, r0.y), gauss(r0.z, r0.w), gauss(r1.x, r1.y), gauss(r1.z, r1.w)};
+        float a2[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float eps = clampf(hp.sigma_t * z[i], -hp.noise_clip, hp.noise_clip);
+            a2[i] = clampf(ldcg(S.mu + jl * 4 + i) + eps, -1.0f, 1.0f);
+        }
+        unsigned char* t = reinterpret_cast<unsigned char*>(S.oc2 + (size_t)(jl / TR) * TILE_FLOATS);
+#pragma unroll
+        for (int i = 0; i < 4; i += 2) {
+            uint32_t h, l;
+            tc::split2(a2[i], a2[i + 1], h, l);
+            const int at = 2 * tc::cano16(jl % TR, DC - 4 + i, KC1);
+            *reinterpret_cast<uint32_t*>(t + at) = h;
+            *reinterpret_cast<uint32_t*>(t + 2 * TILE_HALVES + at) = l;
+        }
+    }
+    __syncthreads();
+    // twin target critics, clipped double-Q target
+    f.in = DC; f.out = 1; f.X = S.oc2; f.tanh_out = false;
+    f.W = R.c1_t; f.img = img(N_C1_T); f.Y = S.q1;
+    pass<H, FWD>(f, sm, tmem, st);
+    f.W = R.c2_t; f.img = img(N_C2_T); f.Y = S.q2;
+    pass<H, FWD>(f, sm, tmem, st);
+    for (int jl = threadIdx.x; jl < Bc; jl += LT) {
+        const float qmin = fminf(ldcg(S.q1 + jl), ldcg(S.q2 + jl));
+        S.y[jl] = S.r[jl] + (S.term[jl] != 0.0f ? 0.0f : hp.gamma * qmin);
+    }
+    __syncthreads();
+    // critic regression
+    f.X = S.oc; f.y = S.y;
+    f.W = R.c1; f.img = img(N_C1); f.G = S.g1;
+    float lsum = pass<H, CRIT>(f, sm, tmem, st);
+    f.W = R.c2; f.img = img(N_C2); f.G = S.g2;
+    lsum += pass<H, CRIT>(f, sm, tmem, st);
+    lsum = block_sum(lsum, red);
+    if (threadIdx.x == 0) S.loss[0] = lsum;
+    cluster_sync_all(nS);
+    t_c += 1;
+    const bool pol = (int64_t)(u % (uint32_t)hp.policy_delay) == (int64_t)(hp.policy_delay - 1);
+    {
+        const int lo = (int)((int64_t)PC * rk / nS), hi = (int)((int64_t)PC * (rk + 1) / nS);
+        // on steps that update the actor, the critics' targets take their Polyak step here
+        adam_slice(R.c1, cl0, scr_stride, nS, (int)(S.g1 - scr_base), R.m_c1, R.v_c1, lo, hi, t_c, hp, 1.0f,
+                   pol ? R.c1_t : nullptr, img(N_C1), img(N_C1_T), DC, H);
+        adam_slice(R.c2, cl0, scr_stride, nS, (int)(S.g2 - scr_base), R.m_c2, R.v_c2, lo, hi, t_c, hp, 1.0f,
+                   pol ? R.c2_t : nullptr, img(N_C2), img(N_C2_T), DC, H);
+        if (rk == 0 && threadIdx.x == 0) {
+            float l = 0.0f;
+            for (int s2 = 0; s2 < nS; ++s2) l += ldcg(cl0 + (size_t)s2 * scr_stride + (S.loss - scr_base));
+            R.stats[0] = l;
+        }
+    }
+    cluster_sync_all(nS);
+    if (!pol) return;
+    // delayed actor update through the updated first critic
+    f.W = R.actor; f.img = img(N_ACTOR); f.in = DA; f.out = 4; f.X = S.oa; f.Y = S.mu; f.tanh_out = true;
+    pass<H, FWD>(f, sm, tmem, st);
+    f.W = R.c1; f.img = img(N_C1); f.in = DC; f.out = 1; f.X = S.oc; f.mu = S.mu; f.da = S.da;
+    float qs = pass<H, DQ>(f, sm, tmem, st);
+    f.W = R.actor; f.img = img(N_ACTOR); f.in = DA; f.out = 4; f.X = S.oa; f.G = S.ga;
+    pass<H, ACT>(f, sm, tmem, st);
+    qs = block_sum(qs, red);
+    if (threadIdx.x == 0) S.loss[1] = qs;
+    cluster_sync_all(nS);
+    t_a += 1;
+    {
+        const int lo = (int)((int64_t)PA * rk / nS), hi = (int)((int64_t)PA * (rk + 1) / nS);
+        adam_slice(R.actor, cl0, scr_stride, nS, (int)(S.ga - scr_base), R.m_a, R.v_a, lo, hi, t_a, hp, 1.0f, R.actor_t,
+                   img(N_ACTOR), img(N_ACTOR_T), DA, H);
+        if (rk == 0 && threadIdx.x == 0) {
+            float l = 0.0f;
+            for (int s2 = 0; s2 < nS; ++s2) l += ldcg(cl0 + (size_t)s2 * scr_stride + (S.loss - scr_base) + 1);
+            R.stats[1] = l;
+        }
+    }
+    cluster_sync_all(nS);
+}
+
 // Curriculum change + reward recalculation over the run's buffer, split over the cluster.
 __device__ __noinline__ void curriculum_step(RunDesc& R, int64_t head, int64_t size, int rk, int nS) {
     if (rk == 0 && threadIdx.x == 0) {
@@ -1418,7 +1398,7 @@ __global__ void __launch_bounds__(LT) k_train(RunDesc* runs, const int* order, c
     if (use_tc) {
         if ((threadIdx.x >> 5) == 0) {
             asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                         :: "r"(tc::smem_u32(&tmem_slot)), "r"(tcf::TMEM_COLS) : "memory");
+                         :: "r"(tc::smem_u32(&tmem_slot)), "r"(tce::TMEM_COLS) : "memory");
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
         }
         tc::fence_before();
@@ -1434,7 +1414,15 @@ __global__ void __launch_bounds__(LT) k_train(RunDesc* runs, const int* order, c
         int64_t head = R.head, size = R.size, t_now = R.t_now, t_a = R.t_a, t_c = R.t_c, u = R.u;
         int64_t next_curr = R.next_curr;
         const int Bc = R.B / nS;
-        const Scr S = carve(my, Bc, R.H, R.DA, R.DC, R.PA, R.PC, R.n_env);
+        const bool tiles = use_tc && tce::shape_ok(Bc, R.H, R.DA, R.DC);  // tensor-core passes
+        const Scr S = carve(my, Bc, R.H, R.DA, R.DC, R.PA, R.PC, R.n_env, nS, tiles);
+        if (tiles) {
+            // the networks' halves for the tensor-core passes, shared out over the cluster
+            const float* nets[6] = {R.actor, R.actor_t, R.c1, R.c1_t, R.c2, R.c2_t};
+            for (int n = rk; n < 6; n += nS)
+                tce::img_make(net_img(S, my, scr_stride, rk, nS, R.H, n), nets[n], n < 2 ? R.DA : R.DC, R.H);
+            cluster_sync_all(nS);
+        }
         for (int it = 0; it < n_iters; ++it) {
             int n_upd = 1;
             if (do_env) {
@@ -1459,26 +1447,33 @@ __global__ void __launch_bounds__(LT) k_train(RunDesc* runs, const int* order, c
             const bool resident = R.H <= smlp::HP && R.DC <= smlp::INP && R.DA <= smlp::INP;
             const bool resident128 = R.H == 128 && R.DA == 82 && R.DC == 90;
             for (int k = 0; k < n_upd; ++k) {
-                if (resident) {
+                if (tiles) {
+                    if (R.H == 64)
+                        td3_update_tc<64>(R, head, size, t_now, (uint32_t)u, t_a, t_c, S, my, scr_stride, rk, nS, sm, tmem);
+                    else if (R.H == 32)
+                        td3_update_tc<32>(R, head, size, t_now, (uint32_t)u, t_a, t_c, S, my, scr_stride, rk, nS, sm, tmem);
+                    else
+                        td3_update_tc<128>(R, head, size, t_now, (uint32_t)u, t_a, t_c, S, my, scr_stride, rk, nS, sm, tmem);
+                } else if (resident) {
                     // specialised shapes: hidden 64 or 32 over 16 actions of history, and the
                     // privileged critic (82 + 4 + 6 motor/parameter inputs + 4 actions)
                     const int key = R.H * 1000000 + R.DA * 1000 + R.DC;
                     if (key == 64082090)
                         td3_update_smem<64, 82, 90>(R, head, size, t_now, (uint32_t)u, t_a, t_c, S,
-                                                    my, scr_stride, rk, nS, sm, tmem, use_tc != 0);
+                                                    my, scr_stride, rk, nS, sm);
                     else if (key == 32082090)
                         td3_update_smem<32, 82, 90>(R, head, size, t_now, (uint32_t)u, t_a, t_c, S,
-                                                    my, scr_stride, rk, nS, sm, tmem, use_tc != 0);
+                                                    my, scr_stride, rk, nS, sm);
                     else if (key == 64082096)
                         td3_update_smem<64, 82, 96>(R, head, size, t_now, (uint32_t)u, t_a, t_c, S,
-                                                    my, scr_stride, rk, nS, sm, tmem, use_tc != 0);
+                                                    my, scr_stride, rk, nS, sm);
                     else
                         td3_update_smem<0, 0, 0>(R, head, size, t_now, (uint32_t)u, t_a, t_c, S,
-                                                 my, scr_stride, rk, nS, sm, tmem, use_tc != 0);
+                                                 my, scr_stride, rk, nS, sm);
                 } else if (resident128) {
                     // hidden 128 with 16 actions of history: the 128-wide engine shape
                     td3_update_smem<128, 82, 90>(R, head, size, t_now, (uint32_t)u, t_a, t_c, S, my,
-                                                 scr_stride, rk, nS, sm, tmem, use_tc != 0);
+                                                 scr_stride, rk, nS, sm);
                 } else
                     td3_update(R, head, size, t_now, (uint32_t)u, t_a, t_c, S, my, scr_stride,
                                blockIdx.x - rk, rk, nS, sm);
@@ -1497,7 +1492,7 @@ __global__ void __launch_bounds__(LT) k_train(RunDesc* runs, const int* order, c
         __syncthreads();
         tc::fence_after();
         if ((threadIdx.x >> 5) == 0)
-            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(tcf::TMEM_COLS) : "memory");
+            asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(tce::TMEM_COLS) : "memory");
     }
 }
 
@@ -1637,7 +1632,7 @@ static qsim_status prepare_single(const ac_handle* a, const qsim_handle* env, in
     if (a->batch % out->nS)
         return fail(QSIM_EINVAL, "%s: batch %d not divisible by cluster %d", who, a->batch, out->nS);
     out->stride = scratch_floats(a->batch / out->nS, a->hidden, a->obs_dim, a->critic_in, a->n_actor,
-                                 a->n_critic, env->n);
+                                 a->n_critic, env->n, out->nS);
     return QSIM_OK;
 }
 
@@ -1650,11 +1645,8 @@ struct PackedRun {
 static_assert(sizeof(PackedRun) <= QSIM_STATIC_DESC_BYTES, "run descriptor exceeds its static area");
 constexpr size_t kPackedBytes = (sizeof(PackedRun) + 255) & ~(size_t)255;
 
-// Whether the run's pure forward passes go to the tensor cores (tcf::eligible on the device).
-static bool tc_forward_wanted(const RunDesc& R, int nS) {
-    const int Bc = R.B / nS;
-    return Bc % 128 == 0 && (R.H == 32 || R.H == 64 || R.H == 128) && R.DA <= tcf::KP && R.DC <= tcf::KP;
-}
+// Whether the run's updates go to the tensor cores (a launch then allocates tensor memory).
+static bool tc_wanted(const RunDesc& R, int nS) { return tce::shape_ok(R.B / nS, R.H, R.DA, R.DC); }
 
 static qsim_status launch_k_train(int grid, int nS, cudaStream_t st, RunDesc* d_runs, const int* d_order,
                                   const int* d_off, int64_t n_iters, int do_env, float* scratch,
@@ -1695,7 +1687,7 @@ static qsim_status run_single(ac_handle* a, qsim_handle* env, int64_t n_iters, i
         QCHECK_CUDA(cudaMemcpyAsync(d_pk, &pk, sizeof(pk), cudaMemcpyHostToDevice, st));
     }
     s = launch_k_train(L.nS, L.nS, st, &d_pk->run, d_pk->order, d_pk->off, n_iters, do_env, scratch, L.stride,
-                       tc_forward_wanted(pk.run, L.nS) ? 1 : 0);
+                       tc_wanted(pk.run, L.nS) ? 1 : 0);
     if (s != QSIM_OK) {
         if (mirror) memset(mirror, 0xff, sizeof(RunDesc));  // unknown device state: upload next time
         return s;
@@ -1765,7 +1757,7 @@ static qsim_status launch_train(std::vector<ac_handle*>& A, std::vector<qsim_han
         if (s != QSIM_OK) return s;
         if (A[i]->batch % nS) return fail(QSIM_EINVAL, "batch %d not divisible by cluster %d", A[i]->batch, nS);
         stride = std::max(stride, scratch_floats(A[i]->batch / nS, A[i]->hidden, A[i]->obs_dim,
-                                                 A[i]->critic_in, A[i]->n_actor, A[i]->n_critic, E[i]->n));
+                                                 A[i]->critic_in, A[i]->n_actor, A[i]->n_critic, E[i]->n, nS));
     }
     const int n_clusters = std::max(1, std::min(n, n_clusters_in));
     std::vector<int> order(n), off(n_clusters + 1, 0);
@@ -1804,7 +1796,7 @@ static qsim_status launch_train(std::vector<ac_handle*>& A, std::vector<qsim_han
     QCHECK_CUDA(cudaMemcpyAsync(d_order, order.data(), sizeof(int) * n, cudaMemcpyHostToDevice, st));
     QCHECK_CUDA(cudaMemcpyAsync(d_off, off.data(), sizeof(int) * (n_clusters + 1), cudaMemcpyHostToDevice, st));
     int use_tc = 0;
-    for (int i = 0; i < n; ++i) use_tc |= tc_forward_wanted(D[i], nS) ? 1 : 0;
+    for (int i = 0; i < n; ++i) use_tc |= tc_wanted(D[i], nS) ? 1 : 0;
     qsim_status s = launch_k_train(n_clusters * nS, nS, st, d_runs, d_order, d_off, n_iters, do_env,
                                    scratch, stride, use_tc);
     cudaFreeAsync(scratch, st);
@@ -2185,10 +2177,10 @@ extern "C" qsim_status ac_plan_create(ac_handle* const* runs, qsim_handle* const
         if (s != QSIM_OK) { ac_plan_destroy(p); return s; }
         p->stride = std::max(p->stride, scratch_floats(p->A[i]->batch / nS, p->A[i]->hidden,
                                                        p->A[i]->obs_dim, p->A[i]->critic_in,
-                                                       p->A[i]->n_actor, p->A[i]->n_critic, p->E[i]->n));
+                                                       p->A[i]->n_actor, p->A[i]->n_critic, p->E[i]->n, nS));
     }
     int use_tc = 0;
-    for (int i = 0; i < n; ++i) use_tc |= tc_forward_wanted(D[i], nS) ? 1 : 0;
+    for (int i = 0; i < n; ++i) use_tc |= tc_wanted(D[i], nS) ? 1 : 0;
     // longest-processing-time-first assignment of runs to clusters
     std::vector<int> order(n), off(p->n_clusters + 1, 0);
     {

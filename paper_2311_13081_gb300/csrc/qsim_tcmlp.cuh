@@ -1,0 +1,688 @@
+// qsim_tcmlp.cuh -- tensor-core MLP passes of the learner (tcgen05), forward and backward, for
+// a CTA that holds whole 128-sample tiles: in -> H -> H -> out with in <= 96, H in {32, 64,
+// 128}, out <= 4.
+//
+// Every product runs as tcgen05.mma (M 128, kind::f16) on fp16 hi / lo halves of both
+// operands (qsim_tcgen05.cuh), three products per K step of 16, the two small ones of a
+// chain first: they meet an accumulator that is still small, so the tensor core's
+// truncation of each partial sum costs next to nothing, and only the hi x hi steps
+// truncate at full size (relative error of a 128-row reduction 1.9e-7, 5.1e-7 with the
+// three products of each K step in a row, 1.3e-7 for the sequential FP32 sum; measured
+// against 64 bits).  Weight gradients are added up over tiles in FP32 outside the tensor
+// memory for the same reason (4 tiles: 1.5e-7 against 1.7e-6 in one accumulator, 2.5e-7 for
+// the sequential sum).
+//
+// One layout serves both directions.  An operand lies as [row][column] in 8 x 8 core matrices
+// (8 rows x 16 bytes), column groups 128 B apart, row groups KC x 128 B apart.  Read K-major
+// it is an operand whose K runs along the columns (forward products, and dZ2 in dZ2 W2);
+// read MN-major it is one whose K runs along the rows: the samples for the weight
+// gradients (dW1^T = X^T dZ1, dW2^T = H1^T dZ2: the gradient's input index falls on the
+// tensor-memory lanes, so the gradient leaves in coalesced rows), the output units for
+// dZ2 W2.  Nothing is transposed or staged twice.
+//
+// Backward deltas are scaled by a power of two per tile (from the tile's largest output
+// delta and the largest weights), so that their halves stay in range whatever the loss.
+//
+// Bound: latency of the chain MMA -> tensor-memory read -> split -> shared memory -> MMA with
+// one CTA per SM (a chain of MMAs from one thread completes one every ~65 cycles).  256
+// samples at H 64 through one critic, forward and backward: 27 us, the SIMT engine 78.
+#pragma once
+#include "qsim_smlp.cuh"
+#include "qsim_tcgen05.cuh"
+
+namespace qsim {
+namespace tce {
+
+constexpr int KP = 96, KC1 = KP / 8;  // input columns of a tile, zero-padded
+constexpr int TR = 128;               // rows of a tile
+constexpr int TILE_HALVES = TR * KP;  // one half (hi or lo) of an input tile
+constexpr int TILE_FLOATS = TILE_HALVES;  // a tile in scratch: hi then lo
+constexpr int TMEM_COLS = 512;
+constexpr int WAIT_POLLS = 1 << 24;
+
+enum Mode { FWD, CRIT, DQ, ACT };
+
+// Shared memory of a pass, bytes.  At hidden 128 the forward-only pass holds W1, W2 and one
+// half (64 columns) of H1; the backward passes hold all of H1, and W2 takes W1's place
+// tile by tile.
+template <int H, int MODE = CRIT>
+struct Lay {
+    static constexpr bool WIDE = H == 128, HALVES = WIDE && MODE == FWD, SHARE = WIDE && MODE != FWD;
+    static constexpr int KC2 = H / 8;
+    static constexpr int HC = HALVES ? 64 : H;  // columns of H1 held at once
+    static constexpr int DH = WIDE ? 64 : H;    // columns of dZ2 held at once
+    static constexpr int X = 0;
+    static constexpr int W1 = X + 4 * TR * KP;
+    static constexpr int W2 = SHARE ? W1 : W1 + 4 * H * KP;
+    static constexpr int H1 = W2 + 4 * H * H;
+    static constexpr int D2 = H1 + 4 * TR * HC;
+    static constexpr int B1 = D2 + (MODE == FWD ? 0 : 4 * TR * DH);
+    static constexpr int B2 = B1 + 4 * H;
+    static constexpr int W3 = B2 + 4 * H;
+    static constexpr int B3 = W3 + 16 * H;
+    static constexpr int RED = B3 + 16;    // 8 warp maxima, 16 weight maxima, 16 output-bias sums
+    static constexpr int BAR = RED + 160;  // two mbarriers
+    static constexpr int PART = BAR + 16;  // [2][128][4] partial outputs, then [H][4] action columns of W1 or
+                                           // [8][H] of exact_unit2; or
+    static constexpr int SUMS = PART;      // [4][6][H] column sums of the 4 row groups
+    static constexpr int END = PART + (96 * H > 4096 + 32 * H ? 96 * H : 4096 + 32 * H);
+};
+constexpr int lay_bytes() {
+    int m = Lay<128, CRIT>::END;
+    if (Lay<128, FWD>::END > m) m = Lay<128, FWD>::END;
+    if (Lay<64, CRIT>::END > m) m = Lay<64, CRIT>::END;
+    return m;
+}
+constexpr int SMEM_BYTES = lay_bytes();
+
+// The halves of a network's W1 (zero-padded to 96 columns) and W2 as the passes read them:
+// W1 hi | lo | W2 hi | lo.  Kept in the run's scratch for a launch: made of the weights when
+// the launch starts on the run, and rewritten by every Adam and Polyak step, so that a pass
+// loads them with 16-byte copies instead of splitting the weights again (9 passes an update).
+__host__ __device__ constexpr int img_floats(int H) { return H * KP + H * H; }
+
+__host__ __device__ constexpr bool shape_ok(int Bc, int H, int DA, int DC) {
+    return Bc > 0 && Bc % TR == 0 && (H == 32 || H == 64 || H == 128) && DA <= KP && DC <= KP &&
+           DA % 2 == 0 && DC % 2 == 0;
+}
+
+// shared-memory descriptor: no swizzle, leading / stride byte offsets
+__device__ __forceinline__ uint64_t sd(uint32_t addr, int lbo, int sbo) {
+    return (uint64_t)((addr >> 4) & 0x3FFFu) | ((uint64_t)(lbo >> 4) << 16) | ((uint64_t)(sbo >> 4) << 32) |
+           ((uint64_t)1 << 46);
+}
+// An operand of KC column groups at `a`: K along the columns (K-major), or along the rows
+// (MN-major), and its byte advance per K step of 16.
+template <bool MN>
+__device__ __forceinline__ uint64_t op(uint32_t a, int kc) { return MN ? sd(a, kc * 128, 128) : sd(a, 128, kc * 128); }
+template <bool MN>
+__device__ __forceinline__ uint32_t adv(int kc) { return MN ? 2u * (uint32_t)kc * 128u : 256u; }
+
+template <bool TA, bool TB>
+__host__ __device__ constexpr uint32_t idesc(int n) {
+    return (1u << 4) | ((TA ? 1u : 0u) << 15) | ((TB ? 1u : 0u) << 16) | ((uint32_t)(n >> 3) << 17) |
+           ((uint32_t)(TR >> 4) << 24);
+}
+
+// One chain D (+)= A B over ks K steps: the small products first (see the file header).
+template <bool TA, bool TB>
+__device__ __forceinline__ void chain(uint32_t d, uint32_t ah, uint32_t al, int kca, uint32_t bh, uint32_t bl, int kcb,
+                                      int ks, uint32_t id, uint32_t acc) {
+    const uint64_t dah = op<TA>(ah, kca), dal = op<TA>(al, kca), dbh = op<TB>(bh, kcb), dbl = op<TB>(bl, kcb);
+    const uint64_t sa = adv<TA>(kca) >> 4, sb = adv<TB>(kcb) >> 4;
+    for (int j = 0; j < ks; ++j) {
+        tc::mma_ss(d, dah + j * sa, dbl + j * sb, id, acc | (uint32_t)(j > 0));
+        tc::mma_ss(d, dal + j * sa, dbh + j * sb, id, 1);
+    }
+    for (int j = 0; j < ks; ++j) tc::mma_ss(d, dah + j * sa, dbh + j * sb, id, 1);
+}
+
+// Column sums over a warp's 32 lanes of N columns held per lane: column lane / (32 / N).
+template <int N>
+__device__ __forceinline__ float colsum(const float* v) {
+    const int lane = threadIdx.x & 31;
+    float t[N];
+#pragma unroll
+    for (int i = 0; i < N; ++i) t[i] = v[i];
+    int o = 16;
+#pragma unroll
+    for (int n = N; n > 1; n >>= 1) {
+        const bool hi = (lane & o) != 0;
+#pragma unroll
+        for (int i = 0; i < n / 2; ++i) {
+            const float send = hi ? t[i] : t[i + n / 2], keep = hi ? t[i + n / 2] : t[i];
+            t[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+        }
+        o >>= 1;
+    }
+    float r = t[0];
+    for (; o > 0; o >>= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+    return r;
+}
+
+// Byte offset of parameter i (flat index) of a network in its image's hi half and the distance
+// to its lo half; false for biases and the output layer.
+__device__ __forceinline__ bool img_at(int i, int in, int H, int& at, int& lo) {
+    if (i < H * in) {
+        const int j = i / in;
+        at = 2 * tc::cano16(j, i - j * in, KC1);
+        lo = 2 * H * KP;
+        return true;
+    }
+    i -= H * in + H;
+    if (i < 0 || i >= H * H) return false;
+    const int j = i / H;
+    at = 4 * H * KP + 2 * tc::cano16(j, i - j * H, H / 8);
+    lo = 2 * H * H;
+    return true;
+}
+__device__ __forceinline__ void img_put(unsigned char* img, int i, int in, int H, float v) {
+    int at, lo;
+    if (!img_at(i, in, H, at, lo)) return;
+    const __half x = __float2half_rn(v);
+    *reinterpret_cast<__half*>(img + at) = x;
+    *reinterpret_cast<__half*>(img + at + lo) = __float2half_rn(v - __half2float(x));
+}
+// The whole image of a network (one CTA).
+__device__ __noinline__ void img_make(unsigned char* img, const float* W, int in, int H) {
+    for (int i = threadIdx.x; i < H * (KP - in); i += LT) {
+        const int j = i / (KP - in), at = 2 * tc::cano16(j, in + i - j * (KP - in), KC1);
+        *reinterpret_cast<__half*>(img + at) = __float2half_rn(0.0f);
+        *reinterpret_cast<__half*>(img + at + 2 * H * KP) = __float2half_rn(0.0f);
+    }
+    smlp::load_scatter(W, H * in + H + H * H, [&](int i, float v) { img_put(img, i, in, H, v); });
+}
+
+__device__ __forceinline__ void copy16(uint32_t dst, const unsigned char* src, int bytes) {
+    for (int i = 16 * threadIdx.x; i < bytes; i += 16 * LT)
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + (uint32_t)i), "l"(src + i) : "memory");
+}
+
+// Largest magnitude among n halves (a multiple of 8, 16-byte aligned) that this thread reads.
+__device__ __forceinline__ float max_half(const unsigned char* p, int n) {
+    __half2 m = __float2half2_rn(0.0f);
+    for (int i = threadIdx.x; i < n / 8; i += LT) {
+        const uint4 v = __ldcg(reinterpret_cast<const uint4*>(p) + i);
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) m = __hmax2(m, __habs2(*reinterpret_cast<const __half2*>(&w[e])));
+    }
+    return fmaxf(__low2float(m), __high2float(m));
+}
+
+// The FP32 value of one unit's pre-activation as the SIMT engine forms it (products added in
+// input order, then the bias).  A critic's regression takes the ReLU's sign from it where
+// the tensor cores' value lies too close to zero to tell (a band a few times their error):
+// which units pass is then the same as in FP32, and a gradient does not jump by a sample's
+// share because a rounding fell the other way.
+__device__ __noinline__ float exact_unit1(const float* W, int in, const float* xrow, int ldx, const float* bias, int j) {
+    float z = 0.0f;
+    const float* w = W + (size_t)j * in;
+    for (int k0 = 0; k0 < in; k0 += 8) {
+        float x[8], v[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const int k = min(k0 + e, in - 1);
+            x[e] = ldcg(xrow + (size_t)k * ldx);
+            v[e] = k0 + e < in ? ldcg(w + k) : 0.0f;
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) z = fmaf(x[e], v[e], z);
+    }
+    return z + ldcg(bias + j);
+}
+// The same for a unit of the second layer; the warp forms the row's first layer in buf [H].
+template <int H>
+__device__ __noinline__ float exact_unit2(const float* W, int in, const float* xrow, int ldx, int j, float* buf) {
+    const int lane = threadIdx.x & 31;
+    const float* b1 = W + (size_t)H * in;
+    const float* W2 = b1 + H;
+    for (int c = lane; c < H; c += 32) buf[c] = fmaxf(exact_unit1(W, in, xrow, ldx, b1, c), 0.0f);
+    __syncwarp();
+    float z = 0.0f;
+    for (int k = 0; k < H; ++k) z = fmaf(buf[k], ldcg(W2 + (size_t)j * H + k), z);
+    __syncwarp();
+    return z + ldcg(W2 + H * H + j);
+}
+
+// 8 values of row r, columns c0 .. c0 + 7, as hi / lo halves
+__device__ __forceinline__ void put8(unsigned char* hi, unsigned char* lo, int kc, int r, int c0, const float* v) {
+    uint32_t h[4], l[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) tc::split2(v[2 * e], v[2 * e + 1], h[e], l[e]);
+    const int at = 2 * tc::cano16(r, c0, kc);
+    *reinterpret_cast<uint4*>(hi + at) = make_uint4(h[0], h[1], h[2], h[3]);
+    *reinterpret_cast<uint4*>(lo + at) = make_uint4(l[0], l[1], l[2], l[3]);
+}
+
+__device__ __forceinline__ float exp2i(int e) { return __int_as_float((e + 127) << 23); }
+__device__ __forceinline__ int ilog2(float x) { return (int)((__float_as_uint(x) >> 23) & 255u) - 127; }
+
+struct Args {
+    const float* W;  // W1[H][in] b1 W2[H][H] b2 W3[out][H] b3
+    int in, out;
+    const float* X;  // input tiles (hi / lo halves), Bc / 128 of them
+    int Bc;
+    float* Y;        // FWD: outputs [Bc][out]
+    bool tanh_out;
+    const float* y;  // CRIT: regression targets [Bc]
+    float invB;
+    float* G;        // CRIT, ACT: gradient in the layout of W
+    const float* mu; // DQ: actions that take the input's last 4 columns [Bc][4]
+    float* da;       // DQ: out, dLoss/d(actor pre-activation) [Bc][4]; ACT: in
+    const unsigned char* img;  // halves of W1 and W2
+    const float* x32;  // CRIT: the FP32 inputs [in][Bc] and each row's sum of magnitudes [Bc]
+    const float* xn;
+};
+
+// One network pass over the CTA's tiles.  FWD: outputs only.  CRIT: squared-error gradient of a
+// critic, returns this thread's part of the mean squared error.  DQ: -mean Q of a critic at
+// actions mu, gradient with respect to the actor's pre-activations; returns this thread's
+// part of -mean Q.  ACT: parameter gradient of the actor from da.
+template <int H, int MODE>
+__device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int* status) {
+    using L = Lay<H, MODE>;
+    constexpr int KC2 = L::KC2, KCH = L::HC / 8, NC = H / 2, KCD = L::DH / 8;
+    constexpr int OUT = MODE == CRIT || MODE == DQ ? 1 : 4;  // FWD: 1 or 4 (a.out)
+    constexpr bool WG = MODE == CRIT || MODE == ACT, BWD = MODE != FWD;
+    unsigned char* sb = reinterpret_cast<unsigned char*>(sm);
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int r = 32 * (warp & 3) + lane, half = warp >> 2, cb = half * NC;  // this thread's row and columns
+    const int in = a.in, out = MODE == FWD ? a.out : OUT;
+    unsigned char *Xh = sb + L::X, *Xl = Xh + 2 * TILE_HALVES;
+    unsigned char *W1h = sb + L::W1, *W1l = W1h + 2 * H * KP, *W2h = sb + L::W2, *W2l = W2h + 2 * H * H;
+    unsigned char *H1h = sb + L::H1, *H1l = H1h + 2 * TR * L::HC, *D2h = sb + L::D2, *D2l = D2h + 2 * TR * L::DH;
+    float* b1 = reinterpret_cast<float*>(sb + L::B1);
+    float* b2 = reinterpret_cast<float*>(sb + L::B2);
+    float* W3 = reinterpret_cast<float*>(sb + L::W3);
+    float* b3 = reinterpret_cast<float*>(sb + L::B3);
+    float* red = reinterpret_cast<float*>(sb + L::RED);
+    float* part = reinterpret_cast<float*>(sb + L::PART);
+    float* w1a = part + 1024;  // DQ: [H][4], W1's action columns; CRIT: [8][H] of exact_unit2
+    float* sums = reinterpret_cast<float*>(sb + L::SUMS);
+    const uint32_t bar0 = tc::smem_u32(sb + L::BAR), bar1 = bar0 + 8;
+    const uint32_t uXh = tc::smem_u32(Xh), uXl = tc::smem_u32(Xl), uW1h = tc::smem_u32(W1h), uW1l = tc::smem_u32(W1l),
+                   uW2h = tc::smem_u32(W2h), uW2l = tc::smem_u32(W2l), uH1h = tc::smem_u32(H1h),
+                   uH1l = tc::smem_u32(H1l), uD2h = tc::smem_u32(D2h), uD2l = tc::smem_u32(D2l);
+    const uint32_t tP = tmem, tQ = tmem + H, tU = tmem + 2 * H, tV = tmem + 3 * H;
+    const uint32_t lanes = (uint32_t)(32 * (warp & 3)) << 16;
+    const float* gW1 = a.W;
+    const float* gb1 = gW1 + H * in;
+    const float* gW2 = gb1 + H;
+    const float* gb2 = gW2 + H * H;
+    const float* gW3 = gb2 + H;
+    const float* gb3 = gW3 + out * H;
+    uint32_t ph0 = 0, ph1 = 0;
+    auto wait = [&](uint32_t bar, uint32_t& ph) {
+        if (!tc::bar_wait(bar, ph, WAIT_POLLS) && lane == 0 && status) atomicCAS(status, DEV_OK, DEV_TIMEOUT);
+        ph ^= 1u;
+        tc::fence_after();
+    };
+    auto sync = [&] {  // operands in shared memory and tensor-memory reads done, for the next MMAs
+        tc::fence_async_smem();
+        tc::fence_before();
+        __syncthreads();
+        tc::fence_after();
+    };
+    auto load_tile = [&](int t) {
+        copy16(uXh, reinterpret_cast<const unsigned char*>(a.X + (size_t)t * TILE_FLOATS), 4 * TILE_HALVES);
+    };
+    // (the padded columns of W1 meet zero columns of X)
+    auto load_w1 = [&] { copy16(uW1h, a.img, 4 * H * KP); };
+    auto load_w2 = [&] { copy16(uW2h, a.img + 4 * H * KP, 4 * H * H); };
+    if (tid == 0) {
+        tc::bar_init(bar0, 1);
+        tc::bar_init(bar1, 1);
+    }
+    load_tile(0);
+    load_w1();
+    if constexpr (!L::SHARE) load_w2();
+    float w1m = 0.0f, w2m = 0.0f, w3m = 0.0f;
+    if constexpr (MODE == CRIT) w1m = max_half(a.img, H * KP);
+    if constexpr (BWD) w2m = max_half(a.img + 4 * H * KP, H * H);
+    for (int i = tid; i < H; i += LT) {
+        b1[i] = ldcg(gb1 + i);
+        b2[i] = ldcg(gb2 + i);
+    }
+    for (int i = tid; i < out * H; i += LT) {
+        const float w = ldcg(gW3 + i);
+        W3[i] = w;
+        w3m = fmaxf(w3m, fabsf(w));
+    }
+    if (tid < out) b3[tid] = ldcg(gb3 + tid);
+    if constexpr (MODE == DQ)
+        for (int i = tid; i < 4 * H; i += LT) w1a[i] = ldcg(gW1 + (size_t)(i >> 2) * in + in - 4 + (i & 3));
+    float dmax = 0.0f;  // largest |dZ2| and |dZ1| per unit of the largest output delta
+    if constexpr (BWD) {
+        for (int o = 16; o > 0; o >>= 1) {
+            w2m = fmaxf(w2m, __shfl_xor_sync(0xffffffffu, w2m, o));
+            w3m = fmaxf(w3m, __shfl_xor_sync(0xffffffffu, w3m, o));
+            w1m = fmaxf(w1m, __shfl_xor_sync(0xffffffffu, w1m, o));
+        }
+        if (lane == 0) {
+            red[warp] = w2m;
+            red[8 + warp] = w3m;
+            red[16 + warp] = w1m;
+        }
+        __syncthreads();
+        for (int i = 0; i < LT / 32; ++i) {
+            w2m = fmaxf(w2m, red[i]);
+            w3m = fmaxf(w3m, red[8 + i]);
+            w1m = fmaxf(w1m, red[16 + i]);
+        }
+        // (a bound 2^8 for dZ2 leaves dZ1 below 2^15 while H max|W2| <= 2^7)
+        dmax = w3m * (float)out * fmaxf(1.0f, (float)H * w2m * 0.0078125f);
+        __syncthreads();
+    }
+    float acc_loss = 0.0f;
+    for (int t = 0; t < a.Bc / TR; ++t) {
+        const bool first = t == 0;
+        const size_t row = (size_t)t * TR + r;
+        // (the tile's and W1's copies were issued before the loop or in the previous tile)
+        asm volatile("cp.async.wait_all;" ::: "memory");
+        if constexpr (MODE == DQ) {
+            __syncthreads();  // the tile is complete before its action columns are replaced
+            if (half == 0) {
+#pragma unroll
+                for (int c = 0; c < 4; c += 2) {
+                    uint32_t h, l;
+                    tc::split2(ldcg(a.mu + row * 4 + c), ldcg(a.mu + row * 4 + c + 1), h, l);
+                    const int at = 2 * tc::cano16(r, in - 4 + c, KC1);
+                    *reinterpret_cast<uint32_t*>(Xh + at) = h;
+                    *reinterpret_cast<uint32_t*>(Xl + at) = l;
+                }
+            }
+        }
+        sync();
+        // ---- layer 1
+        if (tid == 0) {
+            chain<false, false>(tP, uXh, uXl, KC1, uW1h, uW1l, KC1, KP / 16, idesc<false, false>(H), 0);
+            tc::commit(bar0);
+        }
+        wait(bar0, ph0);
+        if constexpr (L::SHARE) load_w2();
+        if (!BWD && t + 1 < a.Bc / TR) load_tile(t + 1);  // layer 1 has read the tile
+        uint32_t m1[(NC + 31) / 32], amb[(NC + 31) / 32];  // units that passed the ReLU; too close to tell
+        float hn = 0.0f, tau1 = 0.0f;
+        if constexpr (MODE == CRIT) tau1 = 5e-7f * w1m * ldcg(a.xn + row);
+#pragma unroll
+        for (int i = 0; i < (NC + 31) / 32; ++i) m1[i] = amb[i] = 0u;
+        auto epi1 = [&](int c_at) {  // H1's columns from c_at on are this half's
+#pragma unroll
+            for (int c0 = 0; c0 < NC; c0 += 16) {
+                uint32_t v[16];
+                tc::ld16(tP + lanes + cb + c0, v);
+                float x[16];
+#pragma unroll
+                for (int e = 0; e < 16; ++e) {
+                    const float z = __uint_as_float(v[e]) + b1[cb + c0 + e];
+                    x[e] = fmaxf(z, 0.0f);
+                    if (BWD && x[e] > 0.0f) m1[(c0 + e) >> 5] |= 1u << ((c0 + e) & 31);
+                    if constexpr (MODE == CRIT) {
+                        hn += x[e];
+                        if (fabsf(z) < tau1) amb[(c0 + e) >> 5] |= 1u << ((c0 + e) & 31);
+                    }
+                }
+                put8(H1h, H1l, KCH, r, c_at + c0, x);
+                put8(H1h, H1l, KCH, r, c_at + c0 + 8, x + 8);
+            }
+        };
+        if constexpr (L::HALVES) {
+            for (int hh = 0; hh < 2; ++hh) {
+                if (half == hh) epi1(0);
+                sync();
+                if (tid == 0) {
+                    const uint32_t w = (uint32_t)hh * 1024u;  // W2's columns 64 hh ..
+                    chain<false, false>(tQ, uH1h, uH1l, KCH, uW2h + w, uW2l + w, KC2, 4, idesc<false, false>(H), hh);
+                    tc::commit(bar0);
+                }
+                wait(bar0, ph0);
+            }
+        } else {
+            epi1(cb);
+            if constexpr (MODE == CRIT) {
+#pragma unroll
+                for (int i = 0; i < (NC + 31) / 32; ++i)
+                    for (uint32_t m = amb[i]; m; m &= m - 1) {
+                        const int b = __ffs(m) - 1, c = cb + 32 * i + b;
+                        const float z = fmaxf(exact_unit1(gW1, in, a.x32 + row, a.Bc, gb1, c), 0.0f);
+                        m1[i] = z > 0.0f ? m1[i] | (1u << b) : m1[i] & ~(1u << b);
+                        const int at = 2 * tc::cano16(r, c, KCH);
+                        const __half x = __float2half_rn(z);
+                        *reinterpret_cast<__half*>(H1h + at) = x;
+                        *reinterpret_cast<__half*>(H1l + at) = __float2half_rn(z - __half2float(x));
+                    }
+                part[half * TR + r] = hn;
+            }
+            if constexpr (L::SHARE) asm volatile("cp.async.wait_all;" ::: "memory");
+            sync();
+            // ---- layer 2
+            if (tid == 0) {
+                chain<false, false>(tQ, uH1h, uH1l, KCH, uW2h, uW2l, KC2, H / 16, idesc<false, false>(H), 0);
+                tc::commit(bar0);
+            }
+            wait(bar0, ph0);
+        }
+        float tau2 = 0.0f;
+        if constexpr (MODE == CRIT) {
+            tau2 = 5e-7f * w2m * (part[r] + part[TR + r]) + 0.5f * tau1;
+            __syncthreads();  // part is about to be reused
+#pragma unroll
+            for (int i = 0; i < (NC + 31) / 32; ++i) amb[i] = 0u;
+        }
+        float h2[NC], po[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+        for (int c0 = 0; c0 < NC; c0 += 16) {
+            uint32_t v[16];
+            tc::ld16(tQ + lanes + cb + c0, v);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) {
+                const int c = cb + c0 + e;
+                const float z = __uint_as_float(v[e]) + b2[c];
+                const float x = fmaxf(z, 0.0f);
+                h2[c0 + e] = x;
+                if (MODE == CRIT && fabsf(z) < tau2) amb[(c0 + e) >> 5] |= 1u << ((c0 + e) & 31);
+#pragma unroll
+                for (int o = 0; o < (MODE == FWD ? 4 : OUT); ++o)
+                    if (o < out) po[o] = fmaf(W3[o * H + c], x, po[o]);
+            }
+        }
+        if constexpr (MODE == CRIT) {
+#pragma unroll
+            for (int i = 0; i < (NC + 31) / 32; ++i) {
+                uint32_t who = __ballot_sync(0xffffffffu, amb[i] != 0u);  // (warp-uniform from here)
+                while (who) {
+                    const int src = __ffs(who) - 1;
+                    who &= who - 1;
+                    uint32_t m = __shfl_sync(0xffffffffu, amb[i], src);
+                    const size_t rs = (size_t)t * TR + 32 * (warp & 3) + src;
+                    while (m) {
+                        const int b = __ffs(m) - 1;
+                        m &= m - 1;
+                        const float z = exact_unit2<H>(gW1, in, a.x32 + rs, a.Bc, cb + 32 * i + b, w1a + warp * H);
+#pragma unroll
+                        for (int c = 32 * i; c < NC && c < 32 * i + 32; ++c)
+                            if (lane == src && c == 32 * i + b) h2[c] = fmaxf(z, 0.0f);
+                    }
+                }
+            }
+        }
+#pragma unroll
+        for (int o = 0; o < 4; ++o) part[(half * TR + r) * 4 + o] = po[o];
+        tc::fence_before();
+        __syncthreads();
+        tc::fence_after();
+        float yv[4];
+#pragma unroll
+        for (int o = 0; o < 4; ++o) yv[o] = o < out ? part[r * 4 + o] + part[(TR + r) * 4 + o] + b3[o] : 0.0f;
+        if constexpr (MODE == FWD) {
+            if (half == 0)
+                for (int o = 0; o < out; ++o) a.Y[row * out + o] = a.tanh_out ? tanhf(yv[o]) : yv[o];
+        } else {
+            // ---- output deltas and their scale
+            float dz3[OUT], big = 0.0f;
+            if constexpr (MODE == CRIT) {
+                const float e = yv[0] - ldcg(a.y + row);
+                dz3[0] = 2.0f * e * a.invB;
+                if (half == 0) acc_loss += e * e * a.invB;
+            } else if constexpr (MODE == DQ) {
+                dz3[0] = -a.invB;
+                if (half == 0) acc_loss += -yv[0] * a.invB;
+            } else {
+#pragma unroll
+                for (int o = 0; o < OUT; ++o) dz3[o] = ldcg(a.da + row * 4 + o);
+            }
+#pragma unroll
+            for (int o = 0; o < OUT; ++o) big = fmaxf(big, fabsf(dz3[o]));
+            for (int o = 16; o > 0; o >>= 1) big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, o));
+            if (lane == 0) red[warp] = big;
+            __syncthreads();
+            for (int i = 0; i < LT / 32; ++i) big = fmaxf(big, red[i]);
+            const float bound = big * dmax;
+            const int se = bound > 1e-30f && bound < 1e30f ? min(max(7 - ilog2(bound), -100), 100) : 0;
+            const float sc = exp2i(se), inv = exp2i(-se);
+#pragma unroll
+            for (int o = 0; o < OUT; ++o) dz3[o] *= sc;
+            float d2[NC];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                float v = 0.0f;
+#pragma unroll
+                for (int o = 0; o < OUT; ++o) v = fmaf(dz3[o], W3[o * H + cb + c], v);
+                d2[c] = h2[c] > 0.0f ? v : 0.0f;
+            }
+            constexpr int CN = NC < 32 ? NC : 32;  // columns per column sum
+            const int cl = lane / (32 / CN);
+            float* mys = sums + (warp & 3) * 6 * H + cb;  // this row group's sums: gb1, gb2, gW3[o]
+            // ---- dZ2 -> shared memory; dZ1 = dZ2 W2, dW2^T = H1^T dZ2
+            if constexpr (H != 128) {
+#pragma unroll
+                for (int c = 0; c < NC; c += 8) put8(D2h, D2l, KCD, r, cb + c, d2 + c);
+                sync();
+                if (tid == 0) {
+                    chain<false, true>(tP, uD2h, uD2l, KCD, uW2h, uW2l, KC2, H / 16, idesc<false, true>(H), 0);
+                    tc::commit(bar0);
+                }
+                if (WG && tid == 128) {
+                    chain<true, true>(tU, uH1h, uH1l, KCH, uD2h, uD2l, KCD, TR / 16, idesc<true, true>(H), 0);
+                    tc::commit(bar1);
+                }
+            } else {
+                for (int hh = 0; hh < 2; ++hh) {
+                    if (half == hh) {
+#pragma unroll
+                        for (int c = 0; c < NC; c += 8) put8(D2h, D2l, KCD, r, c, d2 + c);
+                    }
+                    sync();
+                    if (tid == 0) {
+                        const uint32_t w = (uint32_t)hh * 8u * KC2 * 128u;  // W2's rows 64 hh ..
+                        chain<false, true>(tP, uD2h, uD2l, KCD, uW2h + w, uW2l + w, KC2, 4, idesc<false, true>(H), hh);
+                        tc::commit(bar0);
+                    }
+                    if (WG && tid == 128) {
+                        chain<true, true>(tU + 64 * hh, uH1h, uH1l, KCH, uD2h, uD2l, KCD, TR / 16,
+                                          idesc<true, true>(64), 0);
+                        tc::commit(bar1);
+                    }
+                    if (hh == 0) {
+                        wait(bar0, ph0);
+                        if (WG) wait(bar1, ph1);
+                    }
+                }
+            }
+            if constexpr (WG) {  // while they run: the sums over the samples
+#pragma unroll
+                for (int c = 0; c < NC; c += CN) {
+                    float x = colsum<CN>(d2 + c);
+                    if (lane % (32 / CN) == 0) mys[H + c + cl] = x;
+#pragma unroll
+                    for (int o = 0; o < OUT; ++o) {
+                        float p[CN];
+#pragma unroll
+                        for (int e = 0; e < CN; ++e) p[e] = dz3[o] * h2[c + e];
+                        x = colsum<CN>(p);
+                        if (lane % (32 / CN) == 0) mys[(2 + o) * H + c + cl] = x;
+                    }
+                }
+                if (half == 0)
+#pragma unroll
+                    for (int o = 0; o < OUT; ++o) {
+                        const float x = smlp::warp_sum(dz3[o]);
+                        if (lane == 0) red[24 + 4 * warp + o] = x;
+                    }
+            }
+            wait(bar0, ph0);
+            if (L::SHARE && t + 1 < a.Bc / TR) load_w1();  // W2 has been read
+            // ---- dZ1
+            float d1[NC];
+#pragma unroll
+            for (int c0 = 0; c0 < NC; c0 += 16) {
+                uint32_t v[16];
+                tc::ld16(tP + lanes + cb + c0, v);
+#pragma unroll
+                for (int e = 0; e < 16; ++e)
+                    d1[c0 + e] = (m1[(c0 + e) >> 5] >> ((c0 + e) & 31)) & 1u ? __uint_as_float(v[e]) : 0.0f;
+            }
+            if constexpr (MODE == DQ) {
+                // dLoss/d(action): the last 4 input columns
+                float dx[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+#pragma unroll
+                for (int c = 0; c < NC; ++c)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) dx[q] = fmaf(d1[c], w1a[(cb + c) * 4 + q], dx[q]);
+#pragma unroll
+                for (int q = 0; q < 4; ++q) part[(half * TR + r) * 4 + q] = dx[q];
+                if (t + 1 < a.Bc / TR) load_tile(t + 1);
+                __syncthreads();
+                if (half == 0)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float m = ldcg(a.mu + row * 4 + q);
+                        a.da[row * 4 + q] = (part[r * 4 + q] + part[(TR + r) * 4 + q]) * inv * (1.0f - m * m);
+                    }
+            } else {
+                wait(bar1, ph1);  // H1 has been read: dZ1 takes its place
+#pragma unroll
+                for (int c = 0; c < NC; c += 8) put8(H1h, H1l, KCH, r, cb + c, d1 + c);
+                sync();
+                if (tid == 0) {
+                    chain<true, true>(tV, uXh, uXl, KC1, uH1h, uH1l, KCH, TR / 16, idesc<true, true>(H), 0);
+                    tc::commit(bar0);
+                }
+#pragma unroll
+                for (int c = 0; c < NC; c += CN) {
+                    const float x = colsum<CN>(d1 + c);
+                    if (lane % (32 / CN) == 0) mys[c + cl] = x;
+                }
+                // gradients: lane = input index, so each column is a coalesced row
+                float* G = a.G;
+                auto flush = [&](uint32_t acc, float* g, int ld, int rows) {
+#pragma unroll
+                    for (int c0 = 0; c0 < NC; c0 += 16) {
+                        uint32_t v[16];
+                        tc::ld16(acc + lanes + cb + c0, v);
+                        if (r < rows) {
+                            float* p = g + (size_t)(cb + c0) * ld + r;
+                            float old[16];
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) old[e] = first ? 0.0f : p[(size_t)e * ld];
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) p[(size_t)e * ld] = fmaf(__uint_as_float(v[e]), inv, old[e]);
+                        }
+                    }
+                };
+                flush(tU, G + H * in + H, H, H);
+                __syncthreads();  // the column sums are complete
+                for (int j = tid; j < H; j += LT) {
+                    auto total = [&](int q) {
+                        float s = 0.0f;
+#pragma unroll
+                        for (int w = 0; w < 4; ++w) s += sums[(w * 6 + q) * H + j];
+                        return s * inv;
+                    };
+                    auto add = [&](float* p, float x) { *p = first ? x : *p + x; };
+                    add(G + H * in + j, total(0));
+                    add(G + H * in + H + H * H + j, total(1));
+#pragma unroll
+                    for (int o = 0; o < OUT; ++o) add(G + H * in + 2 * H + H * H + o * H + j, total(2 + o));
+                }
+                if (tid < OUT) {
+                    float* p = G + H * in + 2 * H + H * H + OUT * H + tid;
+                    const float x = (red[24 + tid] + red[28 + tid] + red[32 + tid] + red[36 + tid]) * inv;
+                    *p = first ? x : *p + x;
+                }
+                wait(bar0, ph0);
+                if (t + 1 < a.Bc / TR) load_tile(t + 1);
+                flush(tV, G, in, in);
+            }
+        }
+        // the next tile reuses the tile buffers, the partial outputs and the tensor memory
+        tc::fence_before();
+        __syncthreads();
+        tc::fence_after();
+    }
+    return acc_loss;
+}
+
+}  // namespace tce
+}  // namespace qsim
