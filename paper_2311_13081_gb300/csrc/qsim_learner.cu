@@ -160,7 +160,7 @@ struct Scr {
     float *oa, *oa2, *oc, *oc2, *r, *term, *y, *q1, *q2, *mu, *da, *dz3, *X1, *X2, *H1a, *H2a,
         *H1b, *H2b, *dZ2, *dZ1, *ga, *g1, *g2, *loss, *env_obs, *env_h1, *env_h2, *env_mu;
     // tensor-core passes (in the place of X1 .. dZ1): this CTA's share of the six networks'
-    // halves (net_img), and o_c in FP32 [critic input][Bc] with its rows' sums of magnitudes [Bc]
+    // halves (net_img), and o_c in FP32 rows [Bc][critic input] with their sums of magnitudes [Bc]
     float *img, *x32, *xn;
 };
 enum Net { N_ACTOR, N_ACTOR_T, N_C1, N_C1_T, N_C2, N_C2_T };
@@ -668,7 +668,8 @@ __device__ __forceinline__ int64_t ring(int64_t a, int64_t m) {
 // formed and written out as coalesced rows.  256 samples on one CTA, values alone: 107 us
 // with the ring in DRAM and every SM at it, 27 us from L2 (two cycles a sector, the rate of
 // the load path); with the rows 140 and 57 us, against 177 and 72 us for one group of 32
-// samples after another through registers.
+// samples after another through registers.  Prefetching the same sectors into L2 first, as
+// tensor-map boxes or line by line, did not shorten it (102 and 119 us for the values).
 namespace gat {
 constexpr int GS = 256, GP = GS + 1;  // samples a pass; row stride (odd: lanes along rows are conflict-free)
 // rows of the shared tile [row][sample]: s, s', a_t, the lags, privileged values, reward,
@@ -681,13 +682,13 @@ static_assert(ROWS * GP + 3 * GS + 4 * MAPS / 2 <= SMEM_MAIN, "gather tile");
 // 4 bytes global -> shared, zero when !ok (nothing is read then)
 __device__ __forceinline__ void cp4(float* dst, const float* src, bool ok) {
     asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;"
-                 :: "r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 4 : 0) : "memory");
+                 :: "r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "r"(ok ? 4 : 0));
 }
 }  // namespace gat
 
 template <bool TILES>
 __device__ __noinline__ void gather_pass(const RunDesc& R, int j0, int Bc, int g0, int G, uint32_t u, int64_t head,
-                                         int64_t size, int64_t t_now, const Scr& S, float* sm) {
+                                         int64_t size, int64_t t_now, const Scr& S, float* sm, bool need_oa) {
     using namespace gat;
     const EnvCfg& C = R.C;
     const int ld = C.ld, F = C.F, NE = R.n_env, DA = R.DA, DC = R.DC, nh = C.n_hist;
@@ -698,8 +699,11 @@ __device__ __noinline__ void gather_pass(const RunDesc& R, int j0, int Bc, int g
     uint32_t* m_slot = reinterpret_cast<uint32_t*>(m_env + GS);          // slot,
     uint32_t* m_flag = m_slot + GS;                                      // and flags
     int16_t* map = reinterpret_cast<int16_t*>(m_flag + GS);              // tile row of o_a, o_a', o_c, o_c' column k
+    // (out of the descriptor once: it lies in global memory)
     int* const bst = R.E.status;
+    const float *const ring_rec = R.E.rec, *const ring_side = R.E.side;
     const int64_t rows = R.E.rows;
+    const int n_priv = C.n_priv;
     const int64_t lost = size == CAP ? nh : 0;
     const int64_t first = head - size + lost;  // ring position of sample index 0 (before wrapping)
     // ---- column maps
@@ -739,7 +743,7 @@ __device__ __noinline__ void gather_pass(const RunDesc& R, int j0, int Bc, int g
         const bool ok = in_bounds(bst, slot, rows, SITE_RING_READ) && in_bounds(bst, env, ld, SITE_SOA);
         m_env[jl] = ok ? env : -1;
         m_slot[jl] = (uint32_t)slot;
-        const uint32_t fl = ok ? __float_as_uint(ldcg(R.E.rec + ((size_t)slot * F + 22) * ld + env)) : 0u;
+        const uint32_t fl = ok ? __float_as_uint(ldcg(ring_rec + ((size_t)slot * F + 22) * ld + env)) : 0u;
         m_flag[jl] = fl;
         S.term[g0 + jl] = (fl & 1u) ? 1.0f : 0.0f;
     }
@@ -756,9 +760,9 @@ __device__ __noinline__ void gather_pass(const RunDesc& R, int j0, int Bc, int g
         const int64_t nslot = ring(slot + 1, CAP);
         const bool nxt_ok = done || in_bounds(bst, nslot, rows, SITE_RING_READ);
         float* T = tile + jl;
-        const float* rec = R.E.rec + (size_t)slot * F * ld + env;
+        const float* rec = ring_rec + (size_t)slot * F * ld + env;
         // the side slot is env-major (an env's 17 values contiguous), the records field-major
-        const float* src2 = done ? R.E.side + ((size_t)slot * ld + env) * NS : R.E.rec + (size_t)nslot * F * ld + env;
+        const float* src2 = done ? ring_side + ((size_t)slot * ld + env) * NS : ring_rec + (size_t)nslot * F * ld + env;
         const size_t st2 = done ? 1 : (size_t)ld;
         for (int i = sub; i < NS; i += tps) {
             cp4(T + (R_S + i) * GP, rec + (size_t)i * ld, true);
@@ -768,13 +772,13 @@ __device__ __noinline__ void gather_pass(const RunDesc& R, int j0, int Bc, int g
         for (int i = sub; i <= nh; i += tps) {
             const int64_t sl = ring(slot - i, CAP);
             const bool ok = i == 0 || ((uint32_t)i <= ep && in_bounds(bst, sl, rows, SITE_RING_READ));
-            const float* ap = ok ? R.E.rec + ((size_t)sl * F + 17) * ld + env : rec;
+            const float* ap = ok ? ring_rec + ((size_t)sl * F + 17) * ld + env : rec;
 #pragma unroll
             for (int c = 0; c < 4; ++c) cp4(T + (R_A + 4 * i + c) * GP, ap + (ok ? c * ld : 0), ok);
         }
         if (sub == tps - 1) {
             cp4(T + R_R * GP, rec + (size_t)21 * ld, true);
-            for (int k = 0; k < C.n_priv; ++k) cp4(T + (R_PV + k) * GP, rec + (size_t)(23 + k) * ld, true);
+            for (int k = 0; k < n_priv; ++k) cp4(T + (R_PV + k) * GP, rec + (size_t)(23 + k) * ld, true);
         }
     }
     asm volatile("cp.async.wait_all;" ::: "memory");
@@ -820,31 +824,48 @@ __device__ __noinline__ void gather_pass(const RunDesc& R, int j0, int Bc, int g
     if constexpr (TILES) {
         // input tiles of the tensor-core passes: lane = sample, 8 columns of one matrix at a
         // time as hi / lo halves (zero past the input width; a core matrix row is 16 bytes,
-        // 8 samples make 128); o_c' gets the target action later
-        float* const dst[4] = {S.oa, S.oa2, S.oc, S.oc2};
-        for (int js = tid; js < G; js += LT) {
+        // 8 samples make 128); o_c' gets the target action later.  A warp keeps a column
+        // group's tile rows for all of its samples.
+        constexpr int KC = tce::KC1;
+        for (int js = tid; R.H == 128 && js < G; js += LT) {
             float n = 0.0f;
-            if (m_env[js] >= 0)
+            if (m_env[js] >= 0) {
+#pragma unroll 8
                 for (int k = 0; k < DC; ++k) n += fabsf(tile[map[2 * MAPS + k] * GP + js]);
+            }
             S.xn[g0 + js] = n;
         }
-        constexpr int KC = tce::KC1;
-        for (int i = warp; i < 4 * KC * (G / 32); i += LT / 32) {
-            const int js = 32 * (i / (4 * KC)) + lane, q = i % (4 * KC), mat = q / KC, kc = q - mat * KC;
+        // o_c in FP32 rows for the critics' regression, a warp per sample
+        float* const x32 = S.x32;
+        for (int js = warp; js < G; js += LT / 32) {
+            if (m_env[js] < 0) continue;
+            float v[3];
+#pragma unroll
+            for (int e = 0; e < 3; ++e) v[e] = lane + 32 * e < DC ? tile[map[2 * MAPS + lane + 32 * e] * GP + js] : 0.0f;
+#pragma unroll
+            for (int e = 0; e < 3; ++e)
+                if (lane + 32 * e < DC) x32[(size_t)(g0 + js) * DC + lane + 32 * e] = v[e];
+        }
+        float *const t_oa = S.oa, *const t_oa2 = S.oa2, *const t_oc = S.oc, *const t_oc2 = S.oc2;
+        const bool need_oc = need_oa || R.H == 128;  // hidden <= 64: o_c's tile is read on the actor's step only
+        for (int q = (need_oa ? 0 : KC) + warp; q < 4 * KC; q += LT / 32) {
+            if (!need_oc && q / KC == 2) continue;
+            const int mat = q / KC, kc = q - mat * KC;
             const int w = mat < 2 ? DA : (mat == 2 ? DC : DC - 4);
-            float v[8];
+            float* const d = mat == 0 ? t_oa : (mat == 1 ? t_oa2 : (mat == 2 ? t_oc : t_oc2));
+            int row8[8];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) {
-                const int k = 8 * kc + e;
-                v[e] = k < w ? tile[map[mat * MAPS + k] * GP + js] : 0.0f;
+            for (int e = 0; e < 8; ++e) row8[e] = 8 * kc + e < w ? map[mat * MAPS + 8 * kc + e] * GP : -1;
+#pragma unroll 2
+            for (int s0 = 0; s0 < G; s0 += 32) {
+                const int js = s0 + lane, j = g0 + js;
+                float v[8];
+#pragma unroll
+                for (int e = 0; e < 8; ++e) v[e] = row8[e] >= 0 ? tile[row8[e] + js] : 0.0f;
+                if (m_env[js] < 0) continue;
+                unsigned char* t = reinterpret_cast<unsigned char*>(d + (size_t)(j / tce::TR) * tce::TILE_FLOATS);
+                tce::put8(t, t + 2 * tce::TILE_HALVES, KC, j % tce::TR, 8 * kc, v);
             }
-            const int j = g0 + js;
-            if (mat == 2 && m_env[js] >= 0)
-#pragma unroll
-                for (int e = 0; e < 8; ++e) S.x32[(size_t)(8 * kc + e) * Bc + j] = v[e];
-            unsigned char* t = reinterpret_cast<unsigned char*>((mat < 2 ? (mat ? dst[1] : dst[0]) : (mat == 2 ? dst[2] : dst[3])) +
-                                                                (size_t)(j / tce::TR) * tce::TILE_FLOATS);
-            if (m_env[js] >= 0) tce::put8(t, t + 2 * tce::TILE_HALVES, KC, j % tce::TR, 8 * kc, v);
         }
     } else {
         // FP32 rows, a warp per sample, 4 columns per lane and matrix in flight
@@ -868,35 +889,42 @@ __device__ __noinline__ void gather_pass(const RunDesc& R, int j0, int Bc, int g
     __syncthreads();
 }
 
-// Gather of this CTA's Bc samples (sm: shared memory, free at this point).
+// Gather of this CTA's Bc samples (sm: shared memory, free at this point); need_oa: whether this
+// update reads o_a (the actor's step).
 template <bool TILES>
 __device__ __forceinline__ void gather_all(const RunDesc& R, int j0, int Bc, uint32_t u,
                                            int64_t head, int64_t size, int64_t t_now,
-                                           const Scr& S, float* sm) {
+                                           const Scr& S, float* sm, bool need_oa = true) {
     for (int g0 = 0; g0 < Bc; g0 += gat::GS)
-        gather_pass<TILES>(R, j0, Bc, g0, min(gat::GS, Bc - g0), u, head, size, t_now, S, sm);
+        gather_pass<TILES>(R, j0, Bc, g0, min(gat::GS, Bc - g0), u, head, size, t_now, S, sm, need_oa);
 }
 
 // Adam on parameters [lo, hi) from the sum of S gradient partials (partial s at
 // gpart_base + s * part_stride + goff, summed in the order s = 0..S-1); with tg != nullptr
 // the target copy also takes its Polyak step tg = tau th + (1 - tau) tg from the new th
 // (the fused form of polyak_slice, for steps that update the targets).  img / timg: halves
-// of the network and its target for the tensor-core passes, kept in step (in, H: its shape).
+// of the network and its target for the tensor-core passes, kept in step.
+// The hyper-parameters are copied out of the run descriptor first: they lie in global memory,
+// and every store of the loop could have changed them for all the compiler knows, so each
+// element read them again behind the previous element's stores (20,000 parameters of two
+// critics on one CTA, with the halves: 52 us that way, 53 now; in isolation 10,500 parameters take 20,000 cycles
+// without the halves, 13,000 of them without the divisions and the root).
 __device__ void adam_slice(float* th, const float* gpart_base, size_t part_stride, int S,
                            int goff, float* m, float* v, int lo, int hi, int64_t t,
-                           const LearnHyper& hp, float gscale, float* tg = nullptr, unsigned char* img = nullptr,
-                           unsigned char* timg = nullptr, int in = 0, int H = 0) {
-    const float bc1 = 1.0f - powf(hp.beta1, (float)t);
-    const float bc2 = 1.0f - powf(hp.beta2, (float)t);
-    const float tau = hp.tau;
+                           const LearnHyper& hp, float gscale, float* tg = nullptr,
+                           const tce::Img img = tce::Img(), const tce::Img timg = tce::Img()) {
+    const float beta1 = hp.beta1, beta2 = hp.beta2, lr = hp.lr, eps = hp.eps, tau = hp.tau;
+    const float bc1 = 1.0f - powf(beta1, (float)t);
+    const float bc2 = 1.0f - powf(beta2, (float)t);
     // U elements per thread per pass, all their loads issued before the arithmetic (8 was
-    // measured no faster on the batched runs and 2.4 % slower on the single run)
+    // measured no faster on the batched runs and 2.4 % slower on the single run).  The loop is
+    // the same for every thread of the CTA: put_lanes needs whole warps.
     constexpr int U = 4;
-    for (int i0 = lo + threadIdx.x; i0 < hi; i0 += U * LT) {
+    for (int b = lo; b < hi; b += U * LT) {
         float g[U], mo[U], vo[U], to[U], tt[U];
 #pragma unroll
         for (int k = 0; k < U; ++k) {
-            const int i = i0 + k * LT;
+            const int i = b + (int)threadIdx.x + k * LT;
             g[k] = 0.0f; mo[k] = 0.0f; vo[k] = 0.0f; to[k] = 0.0f; tt[k] = 0.0f;
             if (i < hi) {
                 mo[k] = m[i]; vo[k] = v[i]; to[k] = th[i];
@@ -910,8 +938,10 @@ __device__ void adam_slice(float* th, const float* gpart_base, size_t part_strid
             for (int q = 0; q < 4; ++q) {
                 const float* gp = gpart_base + (size_t)(s0 + q) * part_stride + goff;
 #pragma unroll
-                for (int k = 0; k < U; ++k)
-                    x[q][k] = s0 + q < S && i0 + k * LT < hi ? ldcg(gp + i0 + k * LT) : 0.0f;
+                for (int k = 0; k < U; ++k) {
+                    const int i = b + (int)threadIdx.x + k * LT;
+                    x[q][k] = s0 + q < S && i < hi ? ldcg(gp + i) : 0.0f;
+                }
             }
 #pragma unroll
             for (int q = 0; q < 4; ++q)
@@ -921,21 +951,25 @@ __device__ void adam_slice(float* th, const float* gpart_base, size_t part_strid
         }
 #pragma unroll
         for (int k = 0; k < U; ++k) {
-            const int i = i0 + k * LT;
-            if (i >= hi) continue;
             const float gk = g[k] * gscale;
-            const float mi = fmaf(hp.beta1, mo[k], (1.0f - hp.beta1) * gk);
-            const float vi = fmaf(hp.beta2, vo[k], (1.0f - hp.beta2) * gk * gk);
-            m[i] = mi;
-            v[i] = vi;
-            const float ti = to[k] - hp.lr * (mi / bc1) / (sqrtf(vi / bc2) + hp.eps);
-            th[i] = ti;
-            if (img) tce::img_put(img, i, in, H, ti);
-            if (tg) {
-                const float gi = fmaf(tau, ti, (1.0f - tau) * tt[k]);
-                tg[i] = gi;
-                if (timg) tce::img_put(timg, i, in, H, gi);
+            const float mi = fmaf(beta1, mo[k], (1.0f - beta1) * gk);
+            const float vi = fmaf(beta2, vo[k], (1.0f - beta2) * gk * gk);
+            mo[k] = mi;
+            vo[k] = vi;
+            to[k] = to[k] - lr * (mi / bc1) / (sqrtf(vi / bc2) + eps);
+            tt[k] = fmaf(tau, to[k], (1.0f - tau) * tt[k]);
+        }
+#pragma unroll
+        for (int k = 0; k < U; ++k) {
+            const int i = b + (int)threadIdx.x + k * LT;
+            if (i < hi) {
+                m[i] = mo[k];
+                v[i] = vo[k];
+                th[i] = to[k];
+                if (tg) tg[i] = tt[k];
             }
+            if (img.p) img.put_lanes(i, hi, to[k]);
+            if (tg && timg.p) timg.put_lanes(i, hi, tt[k]);
         }
     }
 }
@@ -1261,11 +1295,46 @@ __device__ __noinline__ void td3_update_smem(RunDesc& R, int64_t head, int64_t s
     cluster_sync_all(nS);
 }
 
-// One TD3 update with every network pass on the tensor cores (tce::pass): a CTA holds whole
+// Critic regression of a CTA's rows on the shared-memory engine (hidden <= 64), forward and
+// backward chunk by chunk; IN: the critic's input width (0: in).  Returns this thread's part of
+// the loss.
+template <int H, int IN>
+__device__ __noinline__ float critics_smem(const RunDesc& R, const Scr& S, int Bc, int in, float* sm) {
+    using namespace smlp;
+    const int DC = IN ? IN : in, B = R.B;
+    const Buf b = carve(sm);
+    float lsum = 0.0f;
+    for (int c = 0; c < 2; ++c) {
+        float* q = c ? S.q2 : S.q1;
+        stage(c ? R.c2 : R.c1, DC, H, 1, b);
+        for (int r0 = 0; r0 < Bc; r0 += MC) {
+            const int mc = min(MC, Bc - r0);
+            forward(DC, H, 1, S.x32, DC, r0, mc, b, q, 1, false);
+            for (int r = threadIdx.x; r < mc; r += LT) {
+                const float e = q[r0 + r] - S.y[r0 + r];
+                b.dZ3s[r * 4] = 2.0f * e / (float)B;
+                lsum += e * e / (float)B;
+            }
+            __syncthreads();
+            backward(DC, H, 1, r0, mc, b, r0 == 0, true, nullptr, 0, 0);
+        }
+        store_grads(c ? S.g2 : S.g1, DC, H, 1, b);
+    }
+    return lsum;
+}
+
+// One TD3 update with its network passes on the tensor cores (tce::pass): a CTA holds whole
 // 128-sample tiles, at most 96 inputs.  Same phases, random streams and cluster reduction as
-// td3_update.  One CTA, 256 samples at hidden 64, us (SIMT engine -> here): target actor 20
-// -> 13, target critics 34 -> 19, critic regression 156 -> 54, mu 18 -> 11, dQ/da 55 -> 15,
-// actor gradient 105 -> 26; at hidden 128 regression 404 -> 114, actor gradient 234 -> 44.
+// td3_update.  The critics' regression runs there at hidden 128 only; at 32 and 64 it keeps the
+// shared-memory engine's FP32 sums in their order (and the target passes the order of their
+// MMAs), so that a critic's weights over many updates are bit for bit what they were: a unit
+// that passes the ReLU on one side of a rounding and not on the other moves a weight by a
+// sample's whole share, and over 16 updates of 128 runs one such unit was enough to be a
+// thousandth of the weights' size.  At hidden 128 a unit's share is smaller, exact_unit1/2
+// settle the doubtful ones, and the regression was a third of the whole step.
+// One CTA, 256 samples, us (SIMT engine -> here): hidden 64: target actor 20 -> 13, target
+// critics 34 -> 19, mu 18 -> 11, dQ/da 55 -> 15, actor gradient 105 -> 26; hidden 128:
+// regression 404 -> 108, actor gradient 234 -> 43.
 template <int H>
 __device__ __noinline__ void td3_update_tc(RunDesc& R, int64_t head, int64_t size, int64_t t_now, uint32_t u,
                                            int64_t& t_a, int64_t& t_c, const Scr& S, float* scr_base,
@@ -1277,7 +1346,8 @@ __device__ __noinline__ void td3_update_tc(RunDesc& R, int64_t head, int64_t siz
     int* const st = R.E.status;
     float* red = sm + SMEM_MAIN;
     const float invB = 1.0f / (float)B;
-    gather_all<true>(R, j0, Bc, u, head, size, t_now, S, sm);
+    const bool pol = (int64_t)(u % (uint32_t)hp.policy_delay) == (int64_t)(hp.policy_delay - 1);
+    gather_all<true>(R, j0, Bc, u, head, size, t_now, S, sm, pol);
     // target actor + smoothing; the target action goes into o_c' tiles' last columns
     const float* cl0 = scr_base - (size_t)rk * scr_stride;  // scratch of cluster rank 0
     auto img = [&](Net n) { return net_img(S, scr_base, scr_stride, rk, nS, H, n); };
@@ -1321,23 +1391,32 @@ __device__ __noinline__ void td3_update_tc(RunDesc& R, int64_t head, int64_t siz
     }
     __syncthreads();
     // critic regression
-    f.X = S.oc; f.y = S.y;
-    f.W = R.c1; f.img = img(N_C1); f.G = S.g1;
-    float lsum = pass<H, CRIT>(f, sm, tmem, st);
-    f.W = R.c2; f.img = img(N_C2); f.G = S.g2;
-    lsum += pass<H, CRIT>(f, sm, tmem, st);
+    float lsum;
+    if constexpr (H == 128) {
+        f.X = S.oc; f.y = S.y;
+        f.W = R.c1; f.img = img(N_C1); f.G = S.g1;
+        lsum = pass<H, CRIT>(f, sm, tmem, st);
+        f.W = R.c2; f.img = img(N_C2); f.G = S.g2;
+        lsum += pass<H, CRIT>(f, sm, tmem, st);
+    } else if (DC == 90) {
+        lsum = critics_smem<H, 90>(R, S, Bc, DC, sm);
+    } else if (H == 64 && DC == 96) {
+        lsum = critics_smem<H, H == 64 ? 96 : 0>(R, S, Bc, DC, sm);
+    } else {
+        lsum = critics_smem<H, 0>(R, S, Bc, DC, sm);
+    }
     lsum = block_sum(lsum, red);
     if (threadIdx.x == 0) S.loss[0] = lsum;
     cluster_sync_all(nS);
     t_c += 1;
-    const bool pol = (int64_t)(u % (uint32_t)hp.policy_delay) == (int64_t)(hp.policy_delay - 1);
     {
         const int lo = (int)((int64_t)PC * rk / nS), hi = (int)((int64_t)PC * (rk + 1) / nS);
         // on steps that update the actor, the critics' targets take their Polyak step here
+        // (at hidden <= 64 only those steps read critic 1's halves, and none critic 2's)
         adam_slice(R.c1, cl0, scr_stride, nS, (int)(S.g1 - scr_base), R.m_c1, R.v_c1, lo, hi, t_c, hp, 1.0f,
-                   pol ? R.c1_t : nullptr, img(N_C1), img(N_C1_T), DC, H);
+                   pol ? R.c1_t : nullptr, H == 128 || pol ? Img(img(N_C1), DC, H) : Img(), Img(img(N_C1_T), DC, H));
         adam_slice(R.c2, cl0, scr_stride, nS, (int)(S.g2 - scr_base), R.m_c2, R.v_c2, lo, hi, t_c, hp, 1.0f,
-                   pol ? R.c2_t : nullptr, img(N_C2), img(N_C2_T), DC, H);
+                   pol ? R.c2_t : nullptr, H == 128 ? Img(img(N_C2), DC, H) : Img(), Img(img(N_C2_T), DC, H));
         if (rk == 0 && threadIdx.x == 0) {
             float l = 0.0f;
             for (int s2 = 0; s2 < nS; ++s2) l += ldcg(cl0 + (size_t)s2 * scr_stride + (S.loss - scr_base));
@@ -1360,7 +1439,7 @@ __device__ __noinline__ void td3_update_tc(RunDesc& R, int64_t head, int64_t siz
     {
         const int lo = (int)((int64_t)PA * rk / nS), hi = (int)((int64_t)PA * (rk + 1) / nS);
         adam_slice(R.actor, cl0, scr_stride, nS, (int)(S.ga - scr_base), R.m_a, R.v_a, lo, hi, t_a, hp, 1.0f, R.actor_t,
-                   img(N_ACTOR), img(N_ACTOR_T), DA, H);
+                   Img(img(N_ACTOR), DA, H), Img(img(N_ACTOR_T), DA, H));
         if (rk == 0 && threadIdx.x == 0) {
             float l = 0.0f;
             for (int s2 = 0; s2 < nS; ++s2) l += ldcg(cl0 + (size_t)s2 * scr_stride + (S.loss - scr_base) + 1);
@@ -1736,13 +1815,19 @@ static qsim_status learner_run(ac_handle* a, qsim_handle* env, int64_t n_iters, 
 // parameters, barriers, weight staging; and a part per sample on a CTA: gather, the
 // networks' passes).  Only its ratios matter: it balances the longest-processing-time-first
 // assignment of runs to clusters, where a pure FLOP count left the small runs' fixed costs
-// out and piled them onto the same clusters.
+// out and piled them onto the same clusters.  The tensor-core passes have their own fit
+// (256 samples, hidden 32 / 64 / 128: 45 / 81 / 190 us fixed and 90 / 113 / 175 us a tile).
 static double run_cost(const ac_handle* a, const qsim_handle* e, int nS) {
     const double h = a->hidden, b = (double)a->batch / std::max(1, nS);
     // the small-run env step (<= 8 envs, one env per lane group) or the CTA-wide one
     const double env = e->n <= 8 && a->hidden <= 128 ? 13.0 + 0.1 * h : 16.0 + 0.34 * h;
-    const double per_sample = 1.042 + 3.98e-5 * (h * (a->obs_dim + a->critic_in) + 3.0 * h * h);
-    const double upd = 32.3 + 0.71 * h + 0.0109 * h * h + b * per_sample;
+    double upd;
+    if (tce::shape_ok(a->batch / std::max(1, nS), a->hidden, a->obs_dim, a->critic_in)) {
+        upd = 20.0 + 0.6 * h + 0.0057 * h * h + b / tce::TR * (66.0 + 0.68 * h + 0.0013 * h * h);
+    } else {
+        const double per_sample = 1.042 + 3.98e-5 * (h * (a->obs_dim + a->critic_in) + 3.0 * h * h);
+        upd = 32.3 + 0.71 * h + 0.0109 * h * h + b * per_sample;
+    }
     return env + std::max(1, (int)a->cfg.updates_per_step) * upd;
 }
 

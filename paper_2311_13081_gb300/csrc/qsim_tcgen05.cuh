@@ -1,6 +1,6 @@
 // qsim_tcgen05.cuh -- small building blocks for tcgen05 (5th-generation tensor core) MMAs with
 // fp16 operands in shared memory and FP32 accumulators in tensor memory, used by the
-// learner's tensor-core forward pass.
+// learner's tensor-core passes (qsim_tcmlp.cuh).
 //
 // Operand layout: the canonical no-swizzle K-major layout -- 8-row x 16-byte core matrices
 // (8 halves along K), K-adjacent core matrices 128 B apart (leading byte offset), 8-row
@@ -72,6 +72,18 @@ __device__ __forceinline__ void ld16(uint32_t ta, uint32_t* r) {
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
                    "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
                  : "r"(ta) : "memory");
+}
+
+// Two such loads in flight, one wait.
+__device__ __forceinline__ void ld16x2(uint32_t ta, uint32_t* r, uint32_t tb, uint32_t* q) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%32];\n"
+                 "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%16,%17,%18,%19,%20,%21,%22,%23,%24,%25,%26,%27,%28,%29,%30,%31}, [%33];\n"
+                 "tcgen05.wait::ld.sync.aligned;"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),
+                   "=r"(q[0]), "=r"(q[1]), "=r"(q[2]), "=r"(q[3]), "=r"(q[4]), "=r"(q[5]), "=r"(q[6]), "=r"(q[7]),
+                   "=r"(q[8]), "=r"(q[9]), "=r"(q[10]), "=r"(q[11]), "=r"(q[12]), "=r"(q[13]), "=r"(q[14]), "=r"(q[15])
+                 : "r"(ta), "r"(tb) : "memory");
 }
 
 __device__ __forceinline__ uint32_t h2u(__half2 h) { return *reinterpret_cast<uint32_t*>(&h); }

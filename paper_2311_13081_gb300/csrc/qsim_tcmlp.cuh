@@ -3,8 +3,8 @@
 // 128}, out <= 4.
 //
 // Every product runs as tcgen05.mma (M 128, kind::f16) on fp16 hi / lo halves of both
-// operands (qsim_tcgen05.cuh), three products per K step of 16, the two small ones of a
-// chain first: they meet an accumulator that is still small, so the tensor core's
+// operands (qsim_tcgen05.cuh), three products per K step of 16, in the passes with gradients
+// the two small ones of a chain first: they meet an accumulator that is still small, so the tensor core's
 // truncation of each partial sum costs next to nothing, and only the hi x hi steps
 // truncate at full size (relative error of a 128-row reduction 1.9e-7, 5.1e-7 with the
 // three products of each K step in a row, 1.3e-7 for the sequential FP32 sum; measured
@@ -25,7 +25,7 @@
 //
 // Bound: latency of the chain MMA -> tensor-memory read -> split -> shared memory -> MMA with
 // one CTA per SM (a chain of MMAs from one thread completes one every ~65 cycles).  256
-// samples at H 64 through one critic, forward and backward: 27 us, the SIMT engine 78.
+// samples at H 128 through one critic, forward and backward: 54 us, the SIMT engine 202.
 #pragma once
 #include "qsim_smlp.cuh"
 #include "qsim_tcgen05.cuh"
@@ -62,10 +62,9 @@ struct Lay {
     static constexpr int B3 = W3 + 16 * H;
     static constexpr int RED = B3 + 16;    // 8 warp maxima, 16 weight maxima, 16 output-bias sums
     static constexpr int BAR = RED + 160;  // two mbarriers
-    static constexpr int PART = BAR + 16;  // [2][128][4] partial outputs, then [H][4] action columns of W1 or
-                                           // [8][H] of exact_unit2; or
+    static constexpr int PART = BAR + 16;  // [2][128][4] partial outputs, then [H][4] action columns of W1; or
     static constexpr int SUMS = PART;      // [4][6][H] column sums of the 4 row groups
-    static constexpr int END = PART + (96 * H > 4096 + 32 * H ? 96 * H : 4096 + 32 * H);
+    static constexpr int END = PART + (96 * H > 4096 + 16 * H ? 96 * H : 4096 + 16 * H);
 };
 constexpr int lay_bytes() {
     int m = Lay<128, CRIT>::END;
@@ -92,29 +91,66 @@ __device__ __forceinline__ uint64_t sd(uint32_t addr, int lbo, int sbo) {
            ((uint64_t)1 << 46);
 }
 // An operand of KC column groups at `a`: K along the columns (K-major), or along the rows
-// (MN-major), and its byte advance per K step of 16.
+// (MN-major).
 template <bool MN>
 __device__ __forceinline__ uint64_t op(uint32_t a, int kc) { return MN ? sd(a, kc * 128, 128) : sd(a, 128, kc * 128); }
-template <bool MN>
-__device__ __forceinline__ uint32_t adv(int kc) { return MN ? 2u * (uint32_t)kc * 128u : 256u; }
-
 template <bool TA, bool TB>
 __host__ __device__ constexpr uint32_t idesc(int n) {
     return (1u << 4) | ((TA ? 1u : 0u) << 15) | ((TB ? 1u : 0u) << 16) | ((uint32_t)(n >> 3) << 17) |
            ((uint32_t)(TR >> 4) << 24);
 }
 
-// One chain D (+)= A B over ks K steps: the small products first (see the file header).
-template <bool TA, bool TB>
-__device__ __forceinline__ void chain(uint32_t d, uint32_t ah, uint32_t al, int kca, uint32_t bh, uint32_t bl, int kcb,
-                                      int ks, uint32_t id, uint32_t acc) {
-    const uint64_t dah = op<TA>(ah, kca), dal = op<TA>(al, kca), dbh = op<TB>(bh, kcb), dbl = op<TB>(bl, kcb);
-    const uint64_t sa = adv<TA>(kca) >> 4, sb = adv<TB>(kcb) >> 4;
-    for (int j = 0; j < ks; ++j) {
-        tc::mma_ss(d, dah + j * sa, dbl + j * sb, id, acc | (uint32_t)(j > 0));
-        tc::mma_ss(d, dal + j * sa, dbh + j * sb, id, 1);
+// One chain D (+)= A B over KS K steps of operands with KCA and KCB column groups: the small
+// products first (see the file header), or in FWD order, the three of a K step in a row.  Everything but the base addresses is a constant, so
+// that the issuing lane does little more than issue.
+template <bool TA, bool TB, int KCA, int KCB, int KS, bool ROW = false>
+__device__ __forceinline__ void chain(uint32_t d, uint32_t ah, uint32_t al, uint32_t bh, uint32_t bl, uint32_t id,
+                                      uint32_t acc) {
+    const uint64_t dah = op<TA>(ah, KCA), dal = op<TA>(al, KCA), dbh = op<TB>(bh, KCB), dbl = op<TB>(bl, KCB);
+    constexpr uint64_t sa = (TA ? 2 * KCA * 128 : 256) / 16, sb = (TB ? 2 * KCB * 128 : 256) / 16;
+    if constexpr (ROW) {
+#pragma unroll
+        for (int j = 0; j < KS; ++j) {
+            tc::mma_ss(d, dah + j * sa, dbh + j * sb, id, j ? 1u : acc);
+            tc::mma_ss(d, dah + j * sa, dbl + j * sb, id, 1);
+            tc::mma_ss(d, dal + j * sa, dbh + j * sb, id, 1);
+        }
+    } else {
+#pragma unroll
+        for (int j = 0; j < KS; ++j) {
+            tc::mma_ss(d, dah + j * sa, dbl + j * sb, id, j ? 1u : acc);
+            tc::mma_ss(d, dal + j * sa, dbh + j * sb, id, 1);
+        }
+#pragma unroll
+        for (int j = 0; j < KS; ++j) tc::mma_ss(d, dah + j * sa, dbh + j * sb, id, 1);
     }
-    for (int j = 0; j < ks; ++j) tc::mma_ss(d, dah + j * sa, dbh + j * sb, id, 1);
+}
+
+// A product's K steps as one chain, or (two accumulators, dcols columns apart) as two halves
+// that two warps issue side by side: a chain completes one MMA per ~65 cycles, two of them
+// one per ~33.  Part w of PARTS = 2 (the first or second half of the K steps) or the whole.
+template <bool TA, bool TB, int PARTS, int KCA, int KCB, int KS, bool ROW = false>
+__device__ __forceinline__ void chain_part(int w, uint32_t d, int dcols, uint32_t ah, uint32_t al, uint32_t bh, uint32_t bl,
+                                           uint32_t id, uint32_t acc) {
+    constexpr uint32_t sa = (KS / PARTS) * (TA ? 2 * KCA * 128 : 256), sb = (KS / PARTS) * (TB ? 2 * KCB * 128 : 256);
+    const uint32_t oa = (uint32_t)w * sa, ob = (uint32_t)w * sb;
+    chain<TA, TB, KCA, KCB, KS / PARTS, ROW>(d + (uint32_t)(w * dcols), ah + oa, al + oa, bh + ob, bl + ob, id, acc);
+}
+
+// 16 columns of an accumulator, or the sum of the two halves' accumulators.
+template <int PARTS>
+__device__ __forceinline__ void ld_acc(uint32_t t, int dcols, float* x) {
+    uint32_t v[16];
+    if constexpr (PARTS == 1) {
+        tc::ld16(t, v);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) x[e] = __uint_as_float(v[e]);
+    } else {
+        uint32_t w[16];
+        tc::ld16x2(t, v, t + (uint32_t)dcols, w);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) x[e] = __uint_as_float(v[e]) + __uint_as_float(w[e]);
+    }
 }
 
 // Column sums over a warp's 32 lanes of N columns held per lane: column lane / (32 / N).
@@ -140,37 +176,74 @@ __device__ __forceinline__ float colsum(const float* v) {
     return r;
 }
 
-// Byte offset of parameter i (flat index) of a network in its image's hi half and the distance
-// to its lo half; false for biases and the output layer.
-__device__ __forceinline__ bool img_at(int i, int in, int H, int& at, int& lo) {
-    if (i < H * in) {
-        const int j = i / in;
-        at = 2 * tc::cano16(j, i - j * in, KC1);
-        lo = 2 * H * KP;
+// A network's image and the exact divisions by its shape (indices below 2^24).
+struct Img {
+    unsigned char* p = nullptr;
+    int in = 0, H = 0;
+    uint32_t mi = 0, mh = 0;
+    __device__ __forceinline__ Img() {}
+    __device__ __forceinline__ Img(unsigned char* q, int in_, int H_)
+        : p(q), in(in_), H(H_), mi(0xffffffffu / (uint32_t)in_ + 1u), mh(0xffffffffu / (uint32_t)H_ + 1u) {}
+    // Byte offset of parameter i (flat index) in the hi half and the distance to its lo half;
+    // false for biases and the output layer.
+    __device__ __forceinline__ bool at(int i, int& o, int& lo) const {
+        if (i < H * in) {
+            const int j = (int)__umulhi((uint32_t)i, mi);
+            o = 2 * tc::cano16(j, i - j * in, KC1);
+            lo = 2 * H * KP;
+            return true;
+        }
+        i -= H * in + H;
+        if (i < 0 || i >= H * H) return false;
+        const int j = (int)__umulhi((uint32_t)i, mh);
+        o = 4 * H * KP + 2 * tc::cano16(j, i - j * H, H / 8);
+        lo = 2 * H * H;
         return true;
     }
-    i -= H * in + H;
-    if (i < 0 || i >= H * H) return false;
-    const int j = i / H;
-    at = 4 * H * KP + 2 * tc::cano16(j, i - j * H, H / 8);
-    lo = 2 * H * H;
-    return true;
-}
-__device__ __forceinline__ void img_put(unsigned char* img, int i, int in, int H, float v) {
-    int at, lo;
-    if (!img_at(i, in, H, at, lo)) return;
-    const __half x = __float2half_rn(v);
-    *reinterpret_cast<__half*>(img + at) = x;
-    *reinterpret_cast<__half*>(img + at + lo) = __float2half_rn(v - __half2float(x));
-}
-// The whole image of a network (one CTA).
-__device__ __noinline__ void img_make(unsigned char* img, const float* W, int in, int H) {
-    for (int i = threadIdx.x; i < H * (KP - in); i += LT) {
-        const int j = i / (KP - in), at = 2 * tc::cano16(j, in + i - j * (KP - in), KC1);
-        *reinterpret_cast<__half*>(img + at) = __float2half_rn(0.0f);
-        *reinterpret_cast<__half*>(img + at + 2 * H * KP) = __float2half_rn(0.0f);
+    // Parameters i (and i + 1 when two; i even then, so both lie in one row).
+    __device__ __forceinline__ void put(int i, float v, float w, bool two) const {
+        int o, lo;
+        if (!at(i, o, lo)) return;
+        uint32_t h, l;
+        tc::split2(v, w, h, l);
+        if (two) {
+            *reinterpret_cast<uint32_t*>(p + o) = h;
+            *reinterpret_cast<uint32_t*>(p + o + lo) = l;
+        } else {
+            *reinterpret_cast<uint16_t*>(p + o) = (uint16_t)h;
+            *reinterpret_cast<uint16_t*>(p + o + lo) = (uint16_t)l;
+        }
     }
-    smlp::load_scatter(W, H * in + H + H * H, [&](int i, float v) { img_put(img, i, in, H, v); });
+    // One value per lane, consecutive lanes consecutive parameters (all lanes call; the ones
+    // with i >= hi store nothing): pairs leave as 4 bytes.
+    __device__ __forceinline__ void put_lanes(int i, int hi, float v) const {
+        const int lane = threadIdx.x & 31;
+        const float w = __shfl_down_sync(0xffffffffu, v, 1);
+        if (i >= hi) return;
+        const bool two = lane < 31 && i + 1 < hi;
+        if ((i & 1) == 0) put(i, v, w, two);
+        else if (lane == 0) put(i, v, 0.0f, false);
+    }
+};
+
+// The whole image of a network (one CTA), 8 columns of a row per thread.
+__device__ __noinline__ void img_make(unsigned char* img, const float* W, int in, int H) {
+    auto rows = [&](const float* src, int cols, int kc, unsigned char* hi, unsigned char* lo) {
+        for (int i = threadIdx.x; i < H * kc; i += LT) {
+            const int j = i / kc, k0 = 8 * (i - j * kc);
+            float v[8];
+#pragma unroll
+            for (int e = 0; e < 8; ++e) v[e] = k0 + e < cols ? ldcg(src + (size_t)j * cols + k0 + e) : 0.0f;
+            uint32_t h[4], l[4];
+#pragma unroll
+            for (int e = 0; e < 4; ++e) tc::split2(v[2 * e], v[2 * e + 1], h[e], l[e]);
+            const int o = 2 * tc::cano16(j, k0, kc);
+            *reinterpret_cast<uint4*>(hi + o) = make_uint4(h[0], h[1], h[2], h[3]);
+            *reinterpret_cast<uint4*>(lo + o) = make_uint4(l[0], l[1], l[2], l[3]);
+        }
+    };
+    rows(W, in, KC1, img, img + 2 * H * KP);
+    rows(W + H * in + H, H, H / 8, img + 4 * H * KP, img + 4 * H * KP + 2 * H * H);
 }
 
 __device__ __forceinline__ void copy16(uint32_t dst, const unsigned char* src, int bytes) {
@@ -192,37 +265,60 @@ __device__ __forceinline__ float max_half(const unsigned char* p, int n) {
 
 // The FP32 value of one unit's pre-activation as the SIMT engine forms it (products added in
 // input order, then the bias).  A critic's regression takes the ReLU's sign from it where
-// the tensor cores' value lies too close to zero to tell (a band a few times their error):
-// which units pass is then the same as in FP32, and a gradient does not jump by a sample's
-// share because a rounding fell the other way.
-__device__ __noinline__ float exact_unit1(const float* W, int in, const float* xrow, int ldx, const float* bias, int j) {
+// the tensor cores' value lies too close to zero to tell: which units pass is then the same
+// as in FP32, and a gradient does not jump by a sample's share because a rounding fell the
+// other way.  The band is kBand x (largest weight) x (sum of the inputs' magnitudes): about
+// 5 times the difference of the two roundings at the learner's inputs (2.4e-7 of the sum of
+// the products' magnitudes), which some 3 units in 10^6 fall into.
+constexpr float kBand = 1.5e-7f;
+__device__ __noinline__ float exact_unit1(const float* W, int in, const float* xrow, const float* bias, int j) {
     float z = 0.0f;
     const float* w = W + (size_t)j * in;
-    for (int k0 = 0; k0 < in; k0 += 8) {
+#pragma unroll 1
+    for (int k0 = 0; k0 < in; k0 += 8) {  // 16 loads in flight
         float x[8], v[8];
 #pragma unroll
         for (int e = 0; e < 8; ++e) {
             const int k = min(k0 + e, in - 1);
-            x[e] = ldcg(xrow + (size_t)k * ldx);
-            v[e] = k0 + e < in ? ldcg(w + k) : 0.0f;
+            x[e] = ldcg(xrow + k);
+            v[e] = ldcg(w + k);
         }
 #pragma unroll
-        for (int e = 0; e < 8; ++e) z = fmaf(x[e], v[e], z);
+        for (int e = 0; e < 8; ++e)
+            if (k0 + e < in) z = fmaf(x[e], v[e], z);
     }
     return z + ldcg(bias + j);
 }
-// The same for a unit of the second layer; the warp forms the row's first layer in buf [H].
+// The same for a unit of the second layer, by a whole warp: its lanes form the row's first
+// layer, then its units' products are added in order.
 template <int H>
-__device__ __noinline__ float exact_unit2(const float* W, int in, const float* xrow, int ldx, int j, float* buf) {
+__device__ __noinline__ float exact_unit2(const float* W, int in, const float* xrow, int j) {
     const int lane = threadIdx.x & 31;
     const float* b1 = W + (size_t)H * in;
     const float* W2 = b1 + H;
-    for (int c = lane; c < H; c += 32) buf[c] = fmaxf(exact_unit1(W, in, xrow, ldx, b1, c), 0.0f);
-    __syncwarp();
-    float z = 0.0f;
-    for (int k = 0; k < H; ++k) z = fmaf(buf[k], ldcg(W2 + (size_t)j * H + k), z);
-    __syncwarp();
-    return z + ldcg(W2 + H * H + j);
+    float z2 = 0.0f;
+#pragma unroll 1
+    for (int u = 0; u < H; u += 32) {  // this lane's unit u + lane of the first layer
+        const float* w = W + (size_t)(u + lane) * in;
+        const float w2 = ldcg(W2 + (size_t)j * H + u + lane);
+        float z = 0.0f;
+#pragma unroll 1
+        for (int k0 = 0; k0 < in; k0 += 16) {
+            float v[16];
+            const float x = ldcg(xrow + min(k0 + (lane & 15), in - 1));
+#pragma unroll
+            for (int k = 0; k < 16; ++k) v[k] = ldcg(w + min(k0 + k, in - 1));
+#pragma unroll
+            for (int k = 0; k < 16; ++k) {
+                const float xk = __shfl_sync(0xffffffffu, x, k);
+                if (k0 + k < in) z = fmaf(xk, v[k], z);
+            }
+        }
+        z = fmaxf(z + ldcg(b1 + u + lane), 0.0f);
+        for (int k = 0; k < 32; ++k)
+            z2 = fmaf(__shfl_sync(0xffffffffu, z, k), __shfl_sync(0xffffffffu, w2, k), z2);
+    }
+    return z2 + ldcg(W2 + H * H + j);
 }
 
 // 8 values of row r, columns c0 .. c0 + 7, as hi / lo halves
@@ -251,7 +347,7 @@ struct Args {
     const float* mu; // DQ: actions that take the input's last 4 columns [Bc][4]
     float* da;       // DQ: out, dLoss/d(actor pre-activation) [Bc][4]; ACT: in
     const unsigned char* img;  // halves of W1 and W2
-    const float* x32;  // CRIT: the FP32 inputs [in][Bc] and each row's sum of magnitudes [Bc]
+    const float* x32;  // CRIT: the FP32 inputs [Bc][in] and each row's sum of magnitudes [Bc]
     const float* xn;
 };
 
@@ -263,6 +359,9 @@ template <int H, int MODE>
 __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int* status) {
     using L = Lay<H, MODE>;
     constexpr int KC2 = L::KC2, KCH = L::HC / 8, NC = H / 2, KCD = L::DH / 8;
+    constexpr bool ROW = MODE == FWD;  // the order of the forward-only passes' products
+    // MMA chains per product (hidden 128 has no tensor-memory columns for two)
+    constexpr int PT = H == 128 || MODE == FWD ? 1 : 2;
     constexpr int OUT = MODE == CRIT || MODE == DQ ? 1 : 4;  // FWD: 1 or 4 (a.out)
     constexpr bool WG = MODE == CRIT || MODE == ACT, BWD = MODE != FWD;
     unsigned char* sb = reinterpret_cast<unsigned char*>(sm);
@@ -278,13 +377,14 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
     float* b3 = reinterpret_cast<float*>(sb + L::B3);
     float* red = reinterpret_cast<float*>(sb + L::RED);
     float* part = reinterpret_cast<float*>(sb + L::PART);
-    float* w1a = part + 1024;  // DQ: [H][4], W1's action columns; CRIT: [8][H] of exact_unit2
+    float* w1a = part + 1024;  // DQ: [H][4], W1's action columns
     float* sums = reinterpret_cast<float*>(sb + L::SUMS);
     const uint32_t bar0 = tc::smem_u32(sb + L::BAR), bar1 = bar0 + 8;
     const uint32_t uXh = tc::smem_u32(Xh), uXl = tc::smem_u32(Xl), uW1h = tc::smem_u32(W1h), uW1l = tc::smem_u32(W1l),
                    uW2h = tc::smem_u32(W2h), uW2l = tc::smem_u32(W2l), uH1h = tc::smem_u32(H1h),
                    uH1l = tc::smem_u32(H1l), uD2h = tc::smem_u32(D2h), uD2l = tc::smem_u32(D2l);
-    const uint32_t tP = tmem, tQ = tmem + H, tU = tmem + 2 * H, tV = tmem + 3 * H;
+    const uint32_t tP = tmem, tQ = tP + PT * H, tU = tQ + PT * H, tV = tU + PT * H;
+    static_assert(4 * PT * H <= TMEM_COLS, "tensor memory");
     const uint32_t lanes = (uint32_t)(32 * (warp & 3)) << 16;
     const float* gW1 = a.W;
     const float* gb1 = gW1 + H * in;
@@ -311,8 +411,8 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
     auto load_w1 = [&] { copy16(uW1h, a.img, 4 * H * KP); };
     auto load_w2 = [&] { copy16(uW2h, a.img + 4 * H * KP, 4 * H * H); };
     if (tid == 0) {
-        tc::bar_init(bar0, 1);
-        tc::bar_init(bar1, 1);
+        tc::bar_init(bar0, PT);
+        tc::bar_init(bar1, PT);
     }
     load_tile(0);
     load_w1();
@@ -375,8 +475,8 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
         }
         sync();
         // ---- layer 1
-        if (tid == 0) {
-            chain<false, false>(tP, uXh, uXl, KC1, uW1h, uW1l, KC1, KP / 16, idesc<false, false>(H), 0);
+        if (lane == 0 && warp < PT) {
+            chain_part<false, false, PT, KC1, KC1, KP / 16, ROW>(warp, tP, H, uXh, uXl, uW1h, uW1l, idesc<false, false>(H), 0);
             tc::commit(bar0);
         }
         wait(bar0, ph0);
@@ -384,18 +484,17 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
         if (!BWD && t + 1 < a.Bc / TR) load_tile(t + 1);  // layer 1 has read the tile
         uint32_t m1[(NC + 31) / 32], amb[(NC + 31) / 32];  // units that passed the ReLU; too close to tell
         float hn = 0.0f, tau1 = 0.0f;
-        if constexpr (MODE == CRIT) tau1 = 5e-7f * w1m * ldcg(a.xn + row);
+        if constexpr (MODE == CRIT) tau1 = kBand * w1m * ldcg(a.xn + row);
 #pragma unroll
         for (int i = 0; i < (NC + 31) / 32; ++i) m1[i] = amb[i] = 0u;
         auto epi1 = [&](int c_at) {  // H1's columns from c_at on are this half's
 #pragma unroll
             for (int c0 = 0; c0 < NC; c0 += 16) {
-                uint32_t v[16];
-                tc::ld16(tP + lanes + cb + c0, v);
-                float x[16];
+                float v[16], x[16];
+                ld_acc<PT>(tP + lanes + cb + c0, H, v);
 #pragma unroll
                 for (int e = 0; e < 16; ++e) {
-                    const float z = __uint_as_float(v[e]) + b1[cb + c0 + e];
+                    const float z = v[e] + b1[cb + c0 + e];
                     x[e] = fmaxf(z, 0.0f);
                     if (BWD && x[e] > 0.0f) m1[(c0 + e) >> 5] |= 1u << ((c0 + e) & 31);
                     if constexpr (MODE == CRIT) {
@@ -413,7 +512,7 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
                 sync();
                 if (tid == 0) {
                     const uint32_t w = (uint32_t)hh * 1024u;  // W2's columns 64 hh ..
-                    chain<false, false>(tQ, uH1h, uH1l, KCH, uW2h + w, uW2l + w, KC2, 4, idesc<false, false>(H), hh);
+                    chain<false, false, KCH, KC2, 4, ROW>(tQ, uH1h, uH1l, uW2h + w, uW2l + w, idesc<false, false>(H), hh);
                     tc::commit(bar0);
                 }
                 wait(bar0, ph0);
@@ -425,7 +524,7 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
                 for (int i = 0; i < (NC + 31) / 32; ++i)
                     for (uint32_t m = amb[i]; m; m &= m - 1) {
                         const int b = __ffs(m) - 1, c = cb + 32 * i + b;
-                        const float z = fmaxf(exact_unit1(gW1, in, a.x32 + row, a.Bc, gb1, c), 0.0f);
+                        const float z = fmaxf(exact_unit1(gW1, in, a.x32 + row * in, gb1, c), 0.0f);
                         m1[i] = z > 0.0f ? m1[i] | (1u << b) : m1[i] & ~(1u << b);
                         const int at = 2 * tc::cano16(r, c, KCH);
                         const __half x = __float2half_rn(z);
@@ -437,15 +536,16 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
             if constexpr (L::SHARE) asm volatile("cp.async.wait_all;" ::: "memory");
             sync();
             // ---- layer 2
-            if (tid == 0) {
-                chain<false, false>(tQ, uH1h, uH1l, KCH, uW2h, uW2l, KC2, H / 16, idesc<false, false>(H), 0);
+            if (lane == 0 && warp < PT) {
+                chain_part<false, false, PT, KCH, KC2, H / 16, ROW>(warp, tQ, H, uH1h, uH1l, uW2h, uW2l,
+                                                               idesc<false, false>(H), 0);
                 tc::commit(bar0);
             }
             wait(bar0, ph0);
         }
         float tau2 = 0.0f;
         if constexpr (MODE == CRIT) {
-            tau2 = 5e-7f * w2m * (part[r] + part[TR + r]) + 0.5f * tau1;
+            tau2 = kBand * w2m * (part[r] + part[TR + r]) + 0.25f * tau1;
             __syncthreads();  // part is about to be reused
 #pragma unroll
             for (int i = 0; i < (NC + 31) / 32; ++i) amb[i] = 0u;
@@ -453,12 +553,12 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
         float h2[NC], po[4] = {0.0f, 0.0f, 0.0f, 0.0f};
 #pragma unroll
         for (int c0 = 0; c0 < NC; c0 += 16) {
-            uint32_t v[16];
-            tc::ld16(tQ + lanes + cb + c0, v);
+            float v[16];
+            ld_acc<PT>(tQ + lanes + cb + c0, H, v);
 #pragma unroll
             for (int e = 0; e < 16; ++e) {
                 const int c = cb + c0 + e;
-                const float z = __uint_as_float(v[e]) + b2[c];
+                const float z = v[e] + b2[c];
                 const float x = fmaxf(z, 0.0f);
                 h2[c0 + e] = x;
                 if (MODE == CRIT && fabsf(z) < tau2) amb[(c0 + e) >> 5] |= 1u << ((c0 + e) & 31);
@@ -479,7 +579,7 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
                     while (m) {
                         const int b = __ffs(m) - 1;
                         m &= m - 1;
-                        const float z = exact_unit2<H>(gW1, in, a.x32 + rs, a.Bc, cb + 32 * i + b, w1a + warp * H);
+                        const float z = exact_unit2<H>(gW1, in, a.x32 + rs * in, cb + 32 * i + b);
 #pragma unroll
                         for (int c = 32 * i; c < NC && c < 32 * i + 32; ++c)
                             if (lane == src && c == 32 * i + b) h2[c] = fmaxf(z, 0.0f);
@@ -539,12 +639,14 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
 #pragma unroll
                 for (int c = 0; c < NC; c += 8) put8(D2h, D2l, KCD, r, cb + c, d2 + c);
                 sync();
-                if (tid == 0) {
-                    chain<false, true>(tP, uD2h, uD2l, KCD, uW2h, uW2l, KC2, H / 16, idesc<false, true>(H), 0);
+                if (lane == 0 && warp < PT) {
+                    chain_part<false, true, PT, KCD, KC2, H / 16>(warp, tP, H, uD2h, uD2l, uW2h, uW2l,
+                                                                  idesc<false, true>(H), 0);
                     tc::commit(bar0);
                 }
-                if (WG && tid == 128) {
-                    chain<true, true>(tU, uH1h, uH1l, KCH, uD2h, uD2l, KCD, TR / 16, idesc<true, true>(H), 0);
+                if (WG && lane == 0 && warp >= 4 && warp < 4 + PT) {
+                    chain_part<true, true, PT, KCH, KCD, TR / 16>(warp - 4, tU, H, uH1h, uH1l, uD2h, uD2l,
+                                                                  idesc<true, true>(H), 0);
                     tc::commit(bar1);
                 }
             } else {
@@ -556,12 +658,12 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
                     sync();
                     if (tid == 0) {
                         const uint32_t w = (uint32_t)hh * 8u * KC2 * 128u;  // W2's rows 64 hh ..
-                        chain<false, true>(tP, uD2h, uD2l, KCD, uW2h + w, uW2l + w, KC2, 4, idesc<false, true>(H), hh);
+                        chain<false, true, KCD, KC2, 4>(tP, uD2h, uD2l, uW2h + w, uW2l + w, idesc<false, true>(H), hh);
                         tc::commit(bar0);
                     }
                     if (WG && tid == 128) {
-                        chain<true, true>(tU + 64 * hh, uH1h, uH1l, KCH, uD2h, uD2l, KCD, TR / 16,
-                                          idesc<true, true>(64), 0);
+                        chain<true, true, KCH, KCD, TR / 16>(tU + 64 * hh, uH1h, uH1l, uD2h, uD2l,
+                                                             idesc<true, true>(64), 0);
                         tc::commit(bar1);
                     }
                     if (hh == 0) {
@@ -597,11 +699,10 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
             float d1[NC];
 #pragma unroll
             for (int c0 = 0; c0 < NC; c0 += 16) {
-                uint32_t v[16];
-                tc::ld16(tP + lanes + cb + c0, v);
+                float v[16];
+                ld_acc<PT>(tP + lanes + cb + c0, H, v);
 #pragma unroll
-                for (int e = 0; e < 16; ++e)
-                    d1[c0 + e] = (m1[(c0 + e) >> 5] >> ((c0 + e) & 31)) & 1u ? __uint_as_float(v[e]) : 0.0f;
+                for (int e = 0; e < 16; ++e) d1[c0 + e] = (m1[(c0 + e) >> 5] >> ((c0 + e) & 31)) & 1u ? v[e] : 0.0f;
             }
             if constexpr (MODE == DQ) {
                 // dLoss/d(action): the last 4 input columns
@@ -625,8 +726,9 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
 #pragma unroll
                 for (int c = 0; c < NC; c += 8) put8(H1h, H1l, KCH, r, cb + c, d1 + c);
                 sync();
-                if (tid == 0) {
-                    chain<true, true>(tV, uXh, uXl, KC1, uH1h, uH1l, KCH, TR / 16, idesc<true, true>(H), 0);
+                if (lane == 0 && warp < PT) {
+                    chain_part<true, true, PT, KC1, KCH, TR / 16>(warp, tV, H, uXh, uXl, uH1h, uH1l,
+                                                                  idesc<true, true>(H), 0);
                     tc::commit(bar0);
                 }
 #pragma unroll
@@ -639,15 +741,15 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
                 auto flush = [&](uint32_t acc, float* g, int ld, int rows) {
 #pragma unroll
                     for (int c0 = 0; c0 < NC; c0 += 16) {
-                        uint32_t v[16];
-                        tc::ld16(acc + lanes + cb + c0, v);
+                        float v[16];
+                        ld_acc<PT>(acc + lanes + cb + c0, H, v);
                         if (r < rows) {
                             float* p = g + (size_t)(cb + c0) * ld + r;
                             float old[16];
 #pragma unroll
                             for (int e = 0; e < 16; ++e) old[e] = first ? 0.0f : p[(size_t)e * ld];
 #pragma unroll
-                            for (int e = 0; e < 16; ++e) p[(size_t)e * ld] = fmaf(__uint_as_float(v[e]), inv, old[e]);
+                            for (int e = 0; e < 16; ++e) p[(size_t)e * ld] = fmaf(v[e], inv, old[e]);
                         }
                     }
                 };
