@@ -1831,6 +1831,62 @@ static double run_cost(const ac_handle* a, const qsim_handle* e, int nS) {
     return env + std::max(1, (int)a->cfg.updates_per_step) * upd;
 }
 
+// The calling thread's pinned staging for the batched launch's descriptors.  From pageable
+// memory the upload waited for everything before it on the stream (the previous launch), so
+// consecutive calls left the GPU idle for the whole of their host work.  Two slots in turn: a
+// call waits only if the copy of the call before the last has not run yet.  At most two
+// buffers of the largest call's descriptors (~1 KB a run), freed when the thread ends.
+struct Staging {
+    void* p[2] = {nullptr, nullptr};
+    size_t cap[2] = {0, 0};
+    cudaEvent_t ev[2] = {nullptr, nullptr};
+    int dev = -1, turn = 0;
+    void release() {
+        for (int i = 0; i < 2; ++i) {
+            if (ev[i]) {
+                cudaEventSynchronize(ev[i]);
+                cudaEventDestroy(ev[i]);
+            }
+            if (p[i]) cudaFreeHost(p[i]);
+            p[i] = nullptr;
+            ev[i] = nullptr;
+            cap[i] = 0;
+        }
+        cudaGetLastError();
+    }
+    ~Staging() { release(); }
+    // Space for `bytes`, or null (the caller then copies from pageable memory).
+    void* take(size_t bytes) {
+        int d = -1;
+        if (cudaGetDevice(&d) != cudaSuccess) return nullptr;
+        if (d != dev) {  // events belong to a device
+            release();
+            dev = d;
+        }
+        const int i = turn;
+        bool ok = ev[i] || cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming) == cudaSuccess;
+        ok = ok && cudaEventSynchronize(ev[i]) == cudaSuccess;
+        if (ok && cap[i] < bytes) {
+            if (p[i]) cudaFreeHost(p[i]);
+            p[i] = nullptr;
+            cap[i] = 0;
+            ok = cudaHostAlloc(&p[i], bytes, cudaHostAllocDefault) == cudaSuccess;
+            if (ok) cap[i] = bytes;
+            else p[i] = nullptr;
+        }
+        if (!ok) {
+            cudaGetLastError();
+            return nullptr;
+        }
+        return p[i];
+    }
+    // The space taken last is read by the work submitted to st so far.
+    void used(cudaStream_t st) {
+        cudaEventRecord(ev[turn], st);
+        turn ^= 1;
+    }
+};
+
 static qsim_status launch_train(std::vector<ac_handle*>& A, std::vector<qsim_handle*>& E,
                                 int64_t n_iters, int do_env, int nS, cudaStream_t st,
                                 int n_clusters_in) {
@@ -1868,26 +1924,39 @@ static qsim_status launch_train(std::vector<ac_handle*>& A, std::vector<qsim_han
         }
         off[n_clusters] = k;
     }
-    // device copies (stream-ordered; freed in stream order after the launch)
-    RunDesc* d_runs;
-    int *d_order, *d_off;
-    float* scratch;
-    const size_t scr_bytes = sizeof(float) * stride * (size_t)n_clusters * nS;
-    QCHECK_CUDA(cudaMallocAsync((void**)&d_runs, sizeof(RunDesc) * n, st));
-    QCHECK_CUDA(cudaMallocAsync((void**)&d_order, sizeof(int) * n, st));
-    QCHECK_CUDA(cudaMallocAsync((void**)&d_off, sizeof(int) * (n_clusters + 1), st));
-    QCHECK_CUDA(cudaMallocAsync((void**)&scratch, scr_bytes, st));
-    QCHECK_CUDA(cudaMemcpyAsync(d_runs, D.data(), sizeof(RunDesc) * n, cudaMemcpyHostToDevice, st));
-    QCHECK_CUDA(cudaMemcpyAsync(d_order, order.data(), sizeof(int) * n, cudaMemcpyHostToDevice, st));
-    QCHECK_CUDA(cudaMemcpyAsync(d_off, off.data(), sizeof(int) * (n_clusters + 1), cudaMemcpyHostToDevice, st));
+    // device copies and scratch: one stream-ordered allocation, freed in stream order after
+    // the launch
+    auto up = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const size_t o_order = up(sizeof(RunDesc) * n), o_off = o_order + up(sizeof(int) * n),
+                 o_scr = o_off + up(sizeof(int) * (n_clusters + 1));
+    unsigned char* dev;
+    QCHECK_CUDA(cudaMallocAsync((void**)&dev, o_scr + sizeof(float) * stride * (size_t)n_clusters * nS, st));
+    static thread_local Staging staging;
+    // (a captured copy keeps its source's address: not the staging's, which is reused)
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaStreamIsCapturing(st, &cap);
+    std::vector<unsigned char> pageable;
+    unsigned char* host = cap == cudaStreamCaptureStatusNone ? (unsigned char*)staging.take(o_scr) : nullptr;
+    const bool pinned = host != nullptr;
+    if (!pinned) {
+        pageable.resize(o_scr);
+        host = pageable.data();
+    }
+    memcpy(host, D.data(), sizeof(RunDesc) * n);
+    memcpy(host + o_order, order.data(), sizeof(int) * n);
+    memcpy(host + o_off, off.data(), sizeof(int) * (n_clusters + 1));
+    const cudaError_t ce = cudaMemcpyAsync(dev, host, o_scr, cudaMemcpyHostToDevice, st);
+    if (pinned) staging.used(st);
+    if (ce != cudaSuccess) {
+        cudaFreeAsync(dev, st);
+        return cuda_fail(ce, "ac_train: descriptors");
+    }
     int use_tc = 0;
     for (int i = 0; i < n; ++i) use_tc |= tc_wanted(D[i], nS) ? 1 : 0;
-    qsim_status s = launch_k_train(n_clusters * nS, nS, st, d_runs, d_order, d_off, n_iters, do_env,
-                                   scratch, stride, use_tc);
-    cudaFreeAsync(scratch, st);
-    cudaFreeAsync(d_off, st);
-    cudaFreeAsync(d_order, st);
-    cudaFreeAsync(d_runs, st);
+    qsim_status s = launch_k_train(n_clusters * nS, nS, st, reinterpret_cast<RunDesc*>(dev),
+                                   reinterpret_cast<int*>(dev + o_order), reinterpret_cast<int*>(dev + o_off), n_iters,
+                                   do_env, reinterpret_cast<float*>(dev + o_scr), stride, use_tc);
+    cudaFreeAsync(dev, st);
     if (s != QSIM_OK) return s;
     for (int i = 0; i < n; ++i) {
         advance_desc(D[i], n_iters, do_env);
