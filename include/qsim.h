@@ -523,6 +523,14 @@ qsim_status qsim_rollout_vjp(const qsim_vjp_desc* d, const qsim_params* veh, con
                              const float* params, const float* actions, const float* actor,
                              const float* seed, float* loss, float* g_actions, float* g_actor,
                              float* g_params, float* actions_out, void* workspace, void* stream);
+/* The reverse sweep alone, on a workspace that an earlier qsim_rollout_vjp call with the same
+ * descriptor, vehicle and inputs filled and that nothing has written since (a forward-only
+ * call, or one whose gradients were already taken: the sweep leaves the rollout's part of
+ * the workspace as it is, so it can be repeated).  Same gradients as qsim_rollout_vjp. */
+qsim_status qsim_rollout_vjp_reverse(const qsim_vjp_desc* d, const qsim_params* veh, const float* s0,
+                                     const float* params, const float* actions, const float* actor,
+                                     const float* seed, float* g_actions, float* g_actor,
+                                     float* g_params, void* workspace, void* stream);
 
 #ifdef __cplusplus
 }

@@ -152,6 +152,8 @@ _SIGS = {
     "qsim_vjp_workspace": (C.c_size_t, [C.POINTER(QsimVjpDesc)]),
     "qsim_rollout_vjp": (C.c_int, [C.POINTER(QsimVjpDesc), C.POINTER(QsimParams), P, P, P, P,
                                    P, P, P, P, P, P, P, P]),
+    "qsim_rollout_vjp_reverse": (C.c_int, [C.POINTER(QsimVjpDesc), C.POINTER(QsimParams), P, P, P,
+                                           P, P, P, P, P, P, P]),
 }
 
 
@@ -563,6 +565,16 @@ def qsim_rollout_vjp(desc: QsimVjpDesc, veh: QsimParams, s0, params, actions, ac
                                _ptr(actions), _ptr(actor), _ptr(seed), _ptr(loss),
                                _ptr(g_actions), _ptr(g_actor), _ptr(g_params),
                                _ptr(actions_out), _ptr(workspace), _stream(stream)))
+
+
+def qsim_rollout_vjp_reverse(desc: QsimVjpDesc, veh: QsimParams, s0, params, actions, actor, seed,
+                             g_actions, g_actor, g_params, workspace, stream=None):
+    """The reverse sweep on a workspace that qsim_rollout_vjp filled for the same inputs."""
+    load()
+    _chk(_lib.qsim_rollout_vjp_reverse(C.byref(desc), C.byref(veh), _ptr(s0), _ptr(params),
+                                       _ptr(actions), _ptr(actor), _ptr(seed), _ptr(g_actions),
+                                       _ptr(g_actor), _ptr(g_params), _ptr(workspace),
+                                       _stream(stream)))
 
 
 def param_count(inp: int, hid: int, out: int) -> int:

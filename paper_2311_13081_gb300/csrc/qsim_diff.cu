@@ -1296,11 +1296,12 @@ extern "C" size_t qsim_vjp_workspace(const qsim_vjp_desc* d) {
     return ws_layout(*d, DA, PA, nchunk).total * sizeof(float);
 }
 
-extern "C" qsim_status qsim_rollout_vjp(const qsim_vjp_desc* d, const qsim_params* veh,
-                                        const float* s0, const float* params, const float* actions,
-                                        const float* actor, const float* seed, float* loss,
-                                        float* g_actions, float* g_actor, float* g_params,
-                                        float* actions_out, void* workspace, void* stream) {
+// The rollout (unless `workspace` already holds this very rollout's: forward = false) and the
+// reverse sweep.
+static qsim_status vjp_run(const qsim_vjp_desc* d, const qsim_params* veh, const float* s0, const float* params,
+                           const float* actions, const float* actor, const float* seed, float* loss,
+                           float* g_actions, float* g_actor, float* g_params, float* actions_out, void* workspace,
+                           void* stream, bool forward) {
     qsim_status st = check_desc(d);
     if (st != QSIM_OK) return st;
     if (!veh || !s0 || !params || !workspace) return fail(QSIM_EINVAL, "qsim_rollout_vjp: null pointer");
@@ -1359,8 +1360,8 @@ extern "C" qsim_status qsim_rollout_vjp(const qsim_vjp_desc* d, const qsim_param
             QCHECK_CUDA(cudaFuncSetAttribute(gk.bw, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024));
             configured[hi][ci] = true;
         }
-        gk.fw<<<gridw, 32 * WV, smem_fw, cs>>>(a);
-    } else {
+        if (forward) gk.fw<<<gridw, 32 * WV, smem_fw, cs>>>(a);
+    } else if (forward) {
         k_vjp_forward<<<grid, VT, smem, cs>>>(a);
     }
     QCHECK_LAUNCH("k_vjp_forward");
@@ -1446,4 +1447,20 @@ extern "C" qsim_status qsim_rollout_vjp(const qsim_vjp_desc* d, const qsim_param
         }
     }
     return QSIM_OK;
+}
+
+extern "C" qsim_status qsim_rollout_vjp(const qsim_vjp_desc* d, const qsim_params* veh, const float* s0,
+                                        const float* params, const float* actions, const float* actor,
+                                        const float* seed, float* loss, float* g_actions, float* g_actor,
+                                        float* g_params, float* actions_out, void* workspace, void* stream) {
+    return vjp_run(d, veh, s0, params, actions, actor, seed, loss, g_actions, g_actor, g_params, actions_out, workspace,
+                   stream, true);
+}
+
+extern "C" qsim_status qsim_rollout_vjp_reverse(const qsim_vjp_desc* d, const qsim_params* veh, const float* s0,
+                                                const float* params, const float* actions, const float* actor,
+                                                const float* seed, float* g_actions, float* g_actor, float* g_params,
+                                                void* workspace, void* stream) {
+    return vjp_run(d, veh, s0, params, actions, actor, seed, nullptr, g_actions, g_actor, g_params, nullptr, workspace,
+                   stream, false);
 }

@@ -1,0 +1,43 @@
+"""The reverse sweep on a workspace that a forward-only call filled gives the gradients of the
+call that runs both, bit for bit, and can be repeated."""
+import numpy as np
+import pytest
+import torch
+
+import workloads as W
+from helpers import cpu
+from paper_2311_13081_gb300 import diff
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("mode,hidden,n,H,ckpt", [(0, 64, 64, 23, 10), (0, 64, 4, 1, 5), (1, 64, 68, 23, 10),
+                                                  (1, 32, 4, 7, 20), (1, 16, 32, 9, 4)])
+def test_reverse_alone_equals_both(gpu, mode, hidden, n, H, ckpt):
+    q = gpu
+    g = torch.Generator("cuda").manual_seed(n + H)
+    veh = q.make_params(W.VEHICLE)
+    s0 = torch.tensor(W.random_states(3, n).T.copy(), dtype=torch.float32, device="cuda")
+    prm = torch.tensor(W.random_params(4, n).T.copy(), dtype=torch.float32, device="cuda")
+    acts = torch.rand(H, 4, n, device="cuda", generator=g) * 2 - 1
+    actor = torch.randn(q.param_count(82, hidden, 4), device="cuda", generator=g) * 0.1
+    seed = torch.rand(n, device="cuda", generator=g)
+    desc = diff.make_desc(n, n, H, ckpt, mode, (1.0, 0.5, 0.2, 0.05), hidden=hidden)
+    a, p = (acts, None) if mode == 0 else (None, actor)
+
+    def grads():
+        return (torch.zeros_like(acts) if mode == 0 else None, torch.zeros_like(actor) if mode else None,
+                torch.zeros(4, n, device="cuda"))
+
+    ws = [torch.empty(q.qsim_vjp_workspace(desc) // 4 + 4, device="cuda") for _ in range(2)]
+    loss = torch.zeros(n, device="cuda")
+    want = grads()
+    q.qsim_rollout_vjp(desc, veh, s0, prm, a, p, seed, loss, *want, None, ws[0])
+    q.qsim_rollout_vjp(desc, veh, s0, prm, a, p, None, loss, None, None, None, None, ws[1])
+    for _ in range(2):
+        got = grads()
+        q.qsim_rollout_vjp_reverse(desc, veh, s0, prm, a, p, seed, *got, ws[1])
+        torch.cuda.synchronize()
+        for x, y in zip(got, want):
+            if x is not None:
+                assert np.array_equal(cpu(x).view(np.uint32), cpu(y).view(np.uint32))
