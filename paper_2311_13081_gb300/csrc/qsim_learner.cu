@@ -3,8 +3,10 @@
 //
 // One run is processed by a thread-block cluster of S CTAs.  Each CTA owns B/S samples of
 // the minibatch: it gathers them from the replay ring, rebuilds the actor and privileged
-// critic observations, and runs every forward / backward GEMM of its slice with
-// activations in its own scratch (L2-resident).  Weight gradients are reduced across the
+// critic observations, and runs every forward / backward GEMM of its slice: on the tensor
+// cores when it holds whole 128-sample tiles (td3_update_tc, qsim_tcmlp.cuh), else in shared
+// memory (td3_update_smem, qsim_smlp.cuh) or, for odd shapes, with activations in its own
+// L2-resident scratch (td3_update).  Weight gradients are reduced across the
 // cluster in a fixed order (deterministic, no float atomics): each CTA sums one slice of
 // the parameter vector over the S partials and applies Adam (and Polyak) to that slice,
 // with hardware cluster barriers between phases.  A persistent grid of clusters walks a
@@ -904,11 +906,10 @@ __device__ __forceinline__ void gather_all(const RunDesc& R, int j0, int Bc, uin
 // the target copy also takes its Polyak step tg = tau th + (1 - tau) tg from the new th
 // (the fused form of polyak_slice, for steps that update the targets).  img / timg: halves
 // of the network and its target for the tensor-core passes, kept in step.
-// The hyper-parameters are copied out of the run descriptor first: they lie in global memory,
-// and every store of the loop could have changed them for all the compiler knows, so each
-// element read them again behind the previous element's stores (20,000 parameters of two
-// critics on one CTA, with the halves: 52 us that way, 53 now; in isolation 10,500 parameters take 20,000 cycles
-// without the halves, 13,000 of them without the divisions and the root).
+// Bound by issue and the latency of its loads: 10,500 parameters on one CTA take 20,000 cycles
+// (9.7 us), 12,500 without the two divisions by the bias corrections, the quotient and the
+// root, whose roundings the weights keep; the halves add 8,000.  Loads of the next block
+// ahead of this block's arithmetic were slower (61 against 52 us for two critics).
 __device__ void adam_slice(float* th, const float* gpart_base, size_t part_stride, int S,
                            int goff, float* m, float* v, int lo, int hi, int64_t t,
                            const LearnHyper& hp, float gscale, float* tg = nullptr,
@@ -1472,7 +1473,7 @@ __global__ void __launch_bounds__(LT) k_train(RunDesc* runs, const int* order, c
                                               int n_iters, int do_env, float* scratch,
                                               size_t scr_stride, int nS, int use_tc) {
     extern __shared__ __align__(16) float sm[];
-    // tensor memory for the tensor-core forward passes, when some run of the launch has them
+    // tensor memory for the tensor-core passes, when some run of the launch has them
     __shared__ uint32_t tmem_slot;
     if (use_tc) {
         if ((threadIdx.x >> 5) == 0) {
