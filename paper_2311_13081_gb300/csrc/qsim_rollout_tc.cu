@@ -886,7 +886,10 @@ qsim_status launch_rollout_tc_range(qsim_handle* h, const float* actor, int T, u
         int sms = 152;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
         chunk = std::min(chunk, T);
-        const int ct = tiles_per_cta((w1 - w0 + 3) / 4, (T + chunk - 1) / chunk, sms);
+        // (a lowered wait limit keeps full groups: their hand-overs take as long as they did
+        // when the limit was chosen, a lone tile's MMAs can be done within one poll)
+        const int ct = h->dc.wait_limit < DEFAULT_WAIT_LIMIT ? TILES
+                                                             : tiles_per_cta((w1 - w0 + 3) / 4, (T + chunk - 1) / chunk, sms);
         const int groups = (w1 - w0 + 4 * ct - 1) / (4 * ct);
         QCHECK_CUDA(cudaMemsetAsync(sched, 0, sizeof(int) * (size_t)(1 + groups), st));
         const int grid = std::min(sms, groups);
