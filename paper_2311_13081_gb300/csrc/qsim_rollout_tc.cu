@@ -146,8 +146,14 @@ __device__ __forceinline__ bool warp_wait(uint32_t bar, uint32_t parity, volatil
                                           int limit) {
     for (int i = 0; i < limit; ++i) {
         uint32_t done;
-        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-                     "selp.u32 %0, 1, 0, p;\n}" : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+        // the first poll only looks (a try_wait may sleep longer than a lone tile's MMAs take,
+        // and a limit of one poll would then not run out)
+        if (i == 0)
+            asm volatile("{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+                         "selp.u32 %0, 1, 0, p;\n}" : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+        else
+            asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+                         "selp.u32 %0, 1, 0, p;\n}" : "=r"(done) : "r"(bar), "r"(parity) : "memory");
         if (__any_sync(0xffffffffu, done)) return true;
         if ((i & 255) == 255 && *abort_flag) return false;
     }
@@ -886,10 +892,7 @@ qsim_status launch_rollout_tc_range(qsim_handle* h, const float* actor, int T, u
         int sms = 152;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
         chunk = std::min(chunk, T);
-        // (a lowered wait limit keeps full groups: their hand-overs take as long as they did
-        // when the limit was chosen, a lone tile's MMAs can be done within one poll)
-        const int ct = h->dc.wait_limit < DEFAULT_WAIT_LIMIT ? TILES
-                                                             : tiles_per_cta((w1 - w0 + 3) / 4, (T + chunk - 1) / chunk, sms);
+        const int ct = tiles_per_cta((w1 - w0 + 3) / 4, (T + chunk - 1) / chunk, sms);
         const int groups = (w1 - w0 + 4 * ct - 1) / (4 * ct);
         QCHECK_CUDA(cudaMemsetAsync(sched, 0, sizeof(int) * (size_t)(1 + groups), st));
         const int grid = std::min(sms, groups);

@@ -70,6 +70,56 @@ def test_tc_wait_that_runs_out_is_reported_and_the_next_call_runs(gpu, sched):
         q.qsim_destroy(h)
 
 
+@pytest.mark.parametrize("n", [129, 152 * 128 + 1, 2 * 152 * 128 + 1])
+def test_tc_wait_runs_out_at_every_group_size(gpu, n):
+    """One, two and three tiles per block (chosen by the env count alone): a one-poll limit
+    runs out, and the call after it matches the oracle."""
+    q = gpu
+    d, h, actor = _env(q, n)
+    try:
+        A = torch.tensor(actor, device="cuda")
+        q.qsim_set_wait_limit(h, 1)
+        q.qsim_rollout(h, A, 64, 4, 0.1)
+        with pytest.raises(q.QsimError) as ei:
+            q.qsim_sync(h)
+        assert ei.value.status == QSIM_ETIMEOUT
+        q.qsim_set_wait_limit(h, 0)
+        e = oracle_envs(q.qsim_info_get(h), np.arange(0, n, max(1, n // 50)))
+        assert np.isfinite(e["s"]).all()
+        q.qsim_destroy(h)
+        d, h, actor = _env(q, n)  # (every block of the next launch allocates all tensor memory)
+        if n < 1000:
+            _one_step_parity(q, d, h, actor, n, "after timeout")
+        else:
+            q.qsim_rollout(h, A, 64, 2, 0.1)
+        q.qsim_sync(h)
+    finally:
+        q.qsim_destroy(h)
+
+
+def test_wait_limit_leaves_the_launch_shape_alone(gpu):
+    """A lowered but ample limit takes the same time as the default one: three tiles per block
+    instead of one are 1.4 times slower at 1,000 envs."""
+    q = gpu
+    d, h, actor = _env(q, 1000)
+    try:
+        A = torch.tensor(actor, device="cuda")
+        best = {}
+        for rep in range(6):
+            for limit in (0, 1 << 21):
+                q.qsim_set_wait_limit(h, limit)
+                e0, e1 = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+                e0.record()
+                q.qsim_rollout(h, A, 64, 200, 0.1)
+                e1.record()
+                torch.cuda.synchronize()
+                best[limit] = min(best.get(limit, 1e9), e0.elapsed_time(e1))
+        q.qsim_sync(h)
+        assert best[1 << 21] < 1.2 * best[0], best
+    finally:
+        q.qsim_destroy(h)
+
+
 @pytest.mark.parametrize("scale", [3e5, 1e6])
 def test_tc_half_precision_overflow_is_reported(gpu, scale):
     """First-layer weights scaled by 3e5 (at most 3.3e4, still inside the fp16 range)
