@@ -38,6 +38,8 @@ class RolloutLoss(torch.autograd.Function):
     @staticmethod
     def forward(ctx, params, x, s0, veh: QsimParams, desc: QsimVjpDesc):
         load()
+        # copies: the structs are the caller's, who may change them before the backward pass
+        desc, veh = QsimVjpDesc.from_buffer_copy(desc), QsimParams.from_buffer_copy(veh)
         ld, n = desc.ld, desc.n
         loss = torch.zeros(ld, device="cuda")
         ws = _workspace(desc)

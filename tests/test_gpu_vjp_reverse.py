@@ -41,3 +41,28 @@ def test_reverse_alone_equals_both(gpu, mode, hidden, n, H, ckpt):
         for x, y in zip(got, want):
             if x is not None:
                 assert np.array_equal(cpu(x).view(np.uint32), cpu(y).view(np.uint32))
+
+
+def _autograd_inputs(q, n, H, closed, hidden=64):
+    g = torch.Generator("cuda").manual_seed(n + H)
+    veh = q.make_params(W.VEHICLE)
+    s0 = torch.tensor(W.random_states(3, n).T.copy(), dtype=torch.float32, device="cuda")
+    prm = torch.tensor(W.random_params(4, n).T.copy(), dtype=torch.float32, device="cuda").requires_grad_()
+    x = (torch.randn(q.param_count(82, hidden, 4), device="cuda", generator=g) * 0.1 if closed
+         else torch.rand(H, 4, n, device="cuda", generator=g) * 2 - 1).requires_grad_()
+    desc = diff.make_desc(n, n, H, 10, int(closed), (1.0, 0.5, 0.2, 0.05), hidden=hidden)
+    return veh, s0, prm, x, desc
+
+
+@pytest.mark.parametrize("closed", [False, True])
+def test_structs_changed_after_the_forward_pass(gpu, closed):
+    """The backward pass belongs to the loss that was computed: the caller's descriptor and
+    vehicle may be reused for something else in between."""
+    q = gpu
+    veh, s0, prm, x, desc = _autograd_inputs(q, 68, 23, closed)
+    want = torch.autograd.grad(diff.RolloutLoss.apply(prm, x, s0, veh, desc).sum(), (prm, x))
+    loss = diff.RolloutLoss.apply(prm, x, s0, veh, desc)
+    desc.w_p, desc.w_q, veh.kf = 7.0, 0.0, 2.0 * veh.kf
+    got = torch.autograd.grad(loss.sum(), (prm, x))
+    for a, b in zip(got, want):
+        assert torch.equal(a, b)
