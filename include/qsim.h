@@ -526,11 +526,27 @@ qsim_status qsim_rollout_vjp(const qsim_vjp_desc* d, const qsim_params* veh, con
 /* The reverse sweep alone, on a workspace that an earlier qsim_rollout_vjp call with the same
  * descriptor, vehicle and inputs filled and that nothing has written since (a forward-only
  * call, or one whose gradients were already taken: the sweep leaves the rollout's part of
- * the workspace as it is, so it can be repeated).  Same gradients as qsim_rollout_vjp. */
+ * the workspace as it is, so it can be repeated).  Same gradients as qsim_rollout_vjp.
+ * Nothing in the workspace says which descriptor filled it: that is the caller's to know. */
 qsim_status qsim_rollout_vjp_reverse(const qsim_vjp_desc* d, const qsim_params* veh, const float* s0,
                                      const float* params, const float* actions, const float* actor,
                                      const float* seed, float* g_actions, float* g_actor,
                                      float* g_params, void* workspace, void* stream);
+/* The same two halves with the workspace in two parts, for a caller who keeps many rollouts
+ * until their gradients are due: `kept` (checkpoints and actions, its first
+ * qsim_vjp_kept() bytes) is written by the rollout and only read by the sweep, and `scratch`
+ * (the other qsim_vjp_workspace() - qsim_vjp_kept() bytes) holds nothing between the calls.
+ * Parts smaller than the descriptor needs are refused (QSIM_EINVAL). */
+size_t qsim_vjp_kept(const qsim_vjp_desc* d);
+qsim_status qsim_rollout_vjp_keep(const qsim_vjp_desc* d, const qsim_params* veh, const float* s0,
+                                  const float* params, const float* actions, const float* actor,
+                                  float* loss, float* actions_out, void* kept, size_t kept_bytes,
+                                  void* scratch, size_t scratch_bytes, void* stream);
+qsim_status qsim_rollout_vjp_from(const qsim_vjp_desc* d, const qsim_params* veh, const float* s0,
+                                  const float* params, const float* actions, const float* actor,
+                                  const float* seed, float* g_actions, float* g_actor, float* g_params,
+                                  const void* kept, size_t kept_bytes, void* scratch,
+                                  size_t scratch_bytes, void* stream);
 
 #ifdef __cplusplus
 }

@@ -154,6 +154,11 @@ _SIGS = {
                                    P, P, P, P, P, P, P, P]),
     "qsim_rollout_vjp_reverse": (C.c_int, [C.POINTER(QsimVjpDesc), C.POINTER(QsimParams), P, P, P,
                                            P, P, P, P, P, P, P]),
+    "qsim_vjp_kept": (C.c_size_t, [C.POINTER(QsimVjpDesc)]),
+    "qsim_rollout_vjp_keep": (C.c_int, [C.POINTER(QsimVjpDesc), C.POINTER(QsimParams), P, P, P, P,
+                                        P, P, P, C.c_size_t, P, C.c_size_t, P]),
+    "qsim_rollout_vjp_from": (C.c_int, [C.POINTER(QsimVjpDesc), C.POINTER(QsimParams), P, P, P, P,
+                                        P, P, P, P, P, C.c_size_t, P, C.c_size_t, P]),
 }
 
 
@@ -575,6 +580,33 @@ def qsim_rollout_vjp_reverse(desc: QsimVjpDesc, veh: QsimParams, s0, params, act
                                        _ptr(actions), _ptr(actor), _ptr(seed), _ptr(g_actions),
                                        _ptr(g_actor), _ptr(g_params), _ptr(workspace),
                                        _stream(stream)))
+
+
+def qsim_vjp_kept(desc: QsimVjpDesc) -> int:
+    load()
+    return int(_lib.qsim_vjp_kept(C.byref(desc)))
+
+
+def _bytes(t) -> int:
+    return t.numel() * t.element_size()
+
+
+def qsim_rollout_vjp_keep(desc: QsimVjpDesc, veh: QsimParams, s0, params, actions, actor, loss,
+                          actions_out, kept, scratch, stream=None):
+    """The rollout alone; ``kept`` holds what qsim_rollout_vjp_from starts from."""
+    load()
+    _chk(_lib.qsim_rollout_vjp_keep(C.byref(desc), C.byref(veh), _ptr(s0), _ptr(params), _ptr(actions),
+                                    _ptr(actor), _ptr(loss), _ptr(actions_out), _ptr(kept), _bytes(kept),
+                                    _ptr(scratch), _bytes(scratch), _stream(stream)))
+
+
+def qsim_rollout_vjp_from(desc: QsimVjpDesc, veh: QsimParams, s0, params, actions, actor, seed,
+                          g_actions, g_actor, g_params, kept, scratch, stream=None):
+    """The reverse sweep from the ``kept`` of qsim_rollout_vjp_keep for the same inputs."""
+    load()
+    _chk(_lib.qsim_rollout_vjp_from(C.byref(desc), C.byref(veh), _ptr(s0), _ptr(params), _ptr(actions),
+                                    _ptr(actor), _ptr(seed), _ptr(g_actions), _ptr(g_actor), _ptr(g_params),
+                                    _ptr(kept), _bytes(kept), _ptr(scratch), _bytes(scratch), _stream(stream)))
 
 
 def param_count(inp: int, hid: int, out: int) -> int:

@@ -1168,6 +1168,8 @@ __global__ void __launch_bounds__(256) k_vjp_wreduce(VjpArgs a) {
 
 static size_t align_up(size_t x) { return (x + 63) & ~(size_t)63; }
 
+// The rollout's part (checkpoints and actions: what the reverse sweep starts from) comes first,
+// then the sweep's scratch, from `la` on.
 struct WsLayout {
     size_t ck, A, la, segs, lam, gp, rec, fo, part, total;
 };
@@ -1288,26 +1290,32 @@ static qsim_status check_desc(const qsim_vjp_desc* d) {
     return QSIM_OK;
 }
 
-extern "C" size_t qsim_vjp_workspace(const qsim_vjp_desc* d) {
-    if (check_desc(d) != QSIM_OK) return 0;
-    const int DA = 18 + 4 * d->n_hist;
-    const int PA = d->hidden * DA + d->hidden + d->hidden * d->hidden + d->hidden + 4 * d->hidden + 4;
-    const int nchunk = (d->n + kChunk - 1) / kChunk;
-    return ws_layout(*d, DA, PA, nchunk).total * sizeof(float);
+static WsLayout desc_layout(const qsim_vjp_desc& d) {
+    const int DA = 18 + 4 * d.n_hist;
+    const int PA = d.hidden * DA + d.hidden + d.hidden * d.hidden + d.hidden + 4 * d.hidden + 4;
+    return ws_layout(d, DA, PA, (d.n + kChunk - 1) / kChunk);
 }
 
-// The rollout (unless `workspace` already holds this very rollout's: forward = false) and the
+extern "C" size_t qsim_vjp_workspace(const qsim_vjp_desc* d) {
+    return check_desc(d) == QSIM_OK ? desc_layout(*d).total * sizeof(float) : 0;
+}
+
+extern "C" size_t qsim_vjp_kept(const qsim_vjp_desc* d) {
+    return check_desc(d) == QSIM_OK ? desc_layout(*d).la * sizeof(float) : 0;
+}
+
+// The rollout (unless `kept` already holds this very rollout's: forward = false) and the
 // reverse sweep.
 static qsim_status vjp_run(const qsim_vjp_desc* d, const qsim_params* veh, const float* s0, const float* params,
                            const float* actions, const float* actor, const float* seed, float* loss,
-                           float* g_actions, float* g_actor, float* g_params, float* actions_out, void* workspace,
-                           void* stream, bool forward) {
+                           float* g_actions, float* g_actor, float* g_params, float* actions_out, void* kept,
+                           void* scratch, void* stream, bool forward) {
     qsim_status st = check_desc(d);
     if (st != QSIM_OK) return st;
-    if (!veh || !s0 || !params || !workspace) return fail(QSIM_EINVAL, "qsim_rollout_vjp: null pointer");
+    if (!veh || !s0 || !params || !kept || !scratch) return fail(QSIM_EINVAL, "qsim_rollout_vjp: null pointer");
     if (d->mode == 0 && !actions) return fail(QSIM_EINVAL, "qsim_rollout_vjp: open loop needs actions");
     if (d->mode == 1 && !actor) return fail(QSIM_EINVAL, "qsim_rollout_vjp: closed loop needs actor");
-    if (!aligned16(s0) || !aligned16(params) || !aligned16(workspace))
+    if (!aligned16(s0) || !aligned16(params) || !aligned16(kept) || !aligned16(scratch))
         return fail(QSIM_EINVAL, "qsim_rollout_vjp: pointers must be 16-byte aligned");
     VjpArgs a;
     memset(&a, 0, sizeof(a));
@@ -1329,10 +1337,11 @@ static qsim_status vjp_run(const qsim_vjp_desc* d, const qsim_params* veh, const
     qsim_vjp_desc dd = *d;
     dd.n_hist = a.nh;
     const WsLayout w = ws_layout(dd, a.DA, a.PA, a.nchunk);
-    float* base = static_cast<float*>(workspace);
-    a.ck = base + w.ck; a.A = base + w.A; a.la = base + w.la; a.segs = base + w.segs;
-    a.lam = base + w.lam; a.gp = base + w.gp; a.rec = base + w.rec; a.fo = base + w.fo;
-    a.part = base + w.part;
+    float *const keep = static_cast<float*>(kept), *const scr = static_cast<float*>(scratch);
+    a.ck = keep + w.ck; a.A = keep + w.A;
+    a.la = scr; a.segs = scr + (w.segs - w.la);
+    a.lam = scr + (w.lam - w.la); a.gp = scr + (w.gp - w.la); a.rec = scr + (w.rec - w.la); a.fo = scr + (w.fo - w.la);
+    a.part = scr + (w.part - w.la);
     cudaStream_t cs = (cudaStream_t)stream;
     const size_t smem = d->mode == 1 ? sizeof(float) * (size_t)a.PA : 0;
     if (smem > 48 * 1024) {
@@ -1449,12 +1458,17 @@ static qsim_status vjp_run(const qsim_vjp_desc* d, const qsim_params* veh, const
     return QSIM_OK;
 }
 
+// One workspace: the kept part, then the scratch.
+static void* ws_scratch(const qsim_vjp_desc* d, void* workspace) {
+    return workspace && d ? static_cast<char*>(workspace) + qsim_vjp_kept(d) : nullptr;
+}
+
 extern "C" qsim_status qsim_rollout_vjp(const qsim_vjp_desc* d, const qsim_params* veh, const float* s0,
                                         const float* params, const float* actions, const float* actor,
                                         const float* seed, float* loss, float* g_actions, float* g_actor,
                                         float* g_params, float* actions_out, void* workspace, void* stream) {
     return vjp_run(d, veh, s0, params, actions, actor, seed, loss, g_actions, g_actor, g_params, actions_out, workspace,
-                   stream, true);
+                   ws_scratch(d, workspace), stream, true);
 }
 
 extern "C" qsim_status qsim_rollout_vjp_reverse(const qsim_vjp_desc* d, const qsim_params* veh, const float* s0,
@@ -1462,5 +1476,37 @@ extern "C" qsim_status qsim_rollout_vjp_reverse(const qsim_vjp_desc* d, const qs
                                                 const float* seed, float* g_actions, float* g_actor, float* g_params,
                                                 void* workspace, void* stream) {
     return vjp_run(d, veh, s0, params, actions, actor, seed, nullptr, g_actions, g_actor, g_params, nullptr, workspace,
-                   stream, false);
+                   ws_scratch(d, workspace), stream, false);
+}
+
+// Sizes of the two parts as the caller has them: none may be smaller than the descriptor's.
+static qsim_status check_parts(const qsim_vjp_desc* d, size_t kept_bytes, size_t scratch_bytes) {
+    const qsim_status st = check_desc(d);
+    if (st != QSIM_OK) return st;
+    const size_t k = qsim_vjp_kept(d), s = qsim_vjp_workspace(d) - k;
+    if (kept_bytes < k || scratch_bytes < s)
+        return fail(QSIM_EINVAL, "qsim_rollout_vjp: workspace parts of %zu and %zu bytes, the descriptor needs %zu and %zu",
+                    kept_bytes, scratch_bytes, k, s);
+    return QSIM_OK;
+}
+
+extern "C" qsim_status qsim_rollout_vjp_keep(const qsim_vjp_desc* d, const qsim_params* veh, const float* s0,
+                                             const float* params, const float* actions, const float* actor, float* loss,
+                                             float* actions_out, void* kept, size_t kept_bytes, void* scratch,
+                                             size_t scratch_bytes, void* stream) {
+    const qsim_status st = check_parts(d, kept_bytes, scratch_bytes);
+    if (st != QSIM_OK) return st;
+    return vjp_run(d, veh, s0, params, actions, actor, nullptr, loss, nullptr, nullptr, nullptr, actions_out, kept, scratch,
+                   stream, true);
+}
+
+extern "C" qsim_status qsim_rollout_vjp_from(const qsim_vjp_desc* d, const qsim_params* veh, const float* s0,
+                                             const float* params, const float* actions, const float* actor,
+                                             const float* seed, float* g_actions, float* g_actor, float* g_params,
+                                             const void* kept, size_t kept_bytes, void* scratch, size_t scratch_bytes,
+                                             void* stream) {
+    const qsim_status st = check_parts(d, kept_bytes, scratch_bytes);
+    if (st != QSIM_OK) return st;
+    return vjp_run(d, veh, s0, params, actions, actor, seed, nullptr, g_actions, g_actor, g_params, nullptr,
+                   const_cast<void*>(kept), scratch, stream, false);
 }

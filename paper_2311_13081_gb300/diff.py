@@ -7,8 +7,8 @@ from __future__ import annotations
 
 import torch
 
-from . import (QsimParams, QsimVjpDesc, _lib, load, qsim_rollout_vjp, qsim_rollout_vjp_reverse,
-               qsim_vjp_workspace)
+from . import (QsimParams, QsimVjpDesc, _lib, load, qsim_rollout_vjp_from, qsim_rollout_vjp_keep,
+               qsim_vjp_kept, qsim_vjp_workspace)
 
 
 def make_desc(n, ld, H, ckpt, mode, weights, dt=0.01, renorm=1, n_hist=16, hidden=64,
@@ -22,18 +22,23 @@ def make_desc(n, ld, H, ckpt, mode, weights, dt=0.01, renorm=1, n_hist=16, hidde
     return d
 
 
-def _workspace(desc):
-    nbytes = qsim_vjp_workspace(desc)
+def _floats(nbytes):
     return torch.empty((nbytes + 3) // 4, dtype=torch.float32, device="cuda")
+
+
+def _scratch(desc):
+    return _floats(qsim_vjp_workspace(desc) - qsim_vjp_kept(desc))
 
 
 class RolloutLoss(torch.autograd.Function):
     """loss_e of an H-step rollout; differentiable w.r.t. ``params`` rows m, Jx, Jy, Jz
     and w.r.t. ``x`` = actions [H][4][ld] (open loop) or the flat actor (closed loop).
 
-    The forward pass's workspace (checkpoints and actions) goes to the backward pass as a
-    saved tensor, which then runs the reverse sweep alone (4,096 envs x 200 open-loop steps:
-    682 us for both passes when the rollout was run again, 546 us now)."""
+    The forward pass's checkpoints and actions go to the backward pass as a saved tensor,
+    which then runs the reverse sweep alone (4,096 envs x 200 open-loop steps: 682 us for
+    both passes when the rollout was run again, 546 us now).  The rest of the workspace is
+    scratch of either pass and not held in between (closed loop, 4,096 envs x 200 steps,
+    checkpoint 20, hidden 64: 16 MB a pending loss, 272 MB with it)."""
 
     @staticmethod
     def forward(ctx, params, x, s0, veh: QsimParams, desc: QsimVjpDesc):
@@ -42,18 +47,17 @@ class RolloutLoss(torch.autograd.Function):
         desc, veh = QsimVjpDesc.from_buffer_copy(desc), QsimParams.from_buffer_copy(veh)
         ld, n = desc.ld, desc.n
         loss = torch.zeros(ld, device="cuda")
-        ws = _workspace(desc)
+        kept = _floats(qsim_vjp_kept(desc))
         acts = x if desc.mode == 0 else None
         actor = x if desc.mode == 1 else None
-        qsim_rollout_vjp(desc, veh, s0, params, acts, actor, None, loss, None, None, None, None,
-                         ws)
-        ctx.save_for_backward(params, x, s0, ws)
+        qsim_rollout_vjp_keep(desc, veh, s0, params, acts, actor, loss, None, kept, _scratch(desc))
+        ctx.save_for_backward(params, x, s0, kept)
         ctx.veh, ctx.desc = veh, desc
         return loss[:n]
 
     @staticmethod
     def backward(ctx, g_loss):
-        params, x, s0, ws = ctx.saved_tensors
+        params, x, s0, kept = ctx.saved_tensors
         desc, veh = ctx.desc, ctx.veh
         ld, n = desc.ld, desc.n
         seed = torch.zeros(ld, device="cuda")
@@ -61,9 +65,9 @@ class RolloutLoss(torch.autograd.Function):
         gp = torch.zeros(4, ld, device="cuda")
         gx = torch.zeros_like(x)
         if desc.mode == 0:
-            qsim_rollout_vjp_reverse(desc, veh, s0, params, x, None, seed, gx, None, gp, ws)
+            qsim_rollout_vjp_from(desc, veh, s0, params, x, None, seed, gx, None, gp, kept, _scratch(desc))
         else:
-            qsim_rollout_vjp_reverse(desc, veh, s0, params, None, x, seed, None, gx, gp, ws)
+            qsim_rollout_vjp_from(desc, veh, s0, params, None, x, seed, None, gx, gp, kept, _scratch(desc))
         g_params = torch.zeros_like(params)
         g_params[0:4] = gp
         return g_params, gx, None, None, None

@@ -66,3 +66,35 @@ def test_structs_changed_after_the_forward_pass(gpu, closed):
     got = torch.autograd.grad(loss.sum(), (prm, x))
     for a, b in zip(got, want):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("closed,hidden", [(False, 64), (True, 64), (True, 16)])
+def test_pending_losses_hold_their_rollouts_only(gpu, closed, hidden):
+    """Two pending losses and a retained graph give the gradients of one loss at a time, bit
+    for bit, and a pending loss holds its checkpoints, actions and loss row, no scratch."""
+    q = gpu
+    veh, s0, prm, x, desc = _autograd_inputs(q, 132, 23, closed, hidden)
+    x2 = (x.detach() * 0.5).requires_grad_()
+    want = [torch.autograd.grad(diff.RolloutLoss.apply(prm, v, s0, veh, desc).sum(), (prm, v)) for v in (x, x2)]
+    torch.cuda.synchronize()
+    before = torch.cuda.memory_allocated()
+    losses = [diff.RolloutLoss.apply(prm, v, s0, veh, desc) for v in (x, x2)]
+    held = (torch.cuda.memory_allocated() - before) // 2
+    rollout = 4 * desc.ld * (-(-desc.H // desc.ckpt) * 17 + 4 * desc.H)  # checkpoints and actions
+    assert held <= rollout + 4 * desc.ld + 4 * 512, (held, rollout, q.qsim_vjp_workspace(desc))
+    for loss, v, w in ((losses[1], x2, want[1]), (losses[0], x, want[0]), (losses[1], x2, want[1])):
+        for a, b in zip(torch.autograd.grad(loss.sum(), (prm, v), retain_graph=True), w):
+            assert torch.equal(a, b)
+
+
+def test_workspace_parts_too_small_are_refused(gpu):
+    q = gpu
+    veh, s0, prm, x, desc = _autograd_inputs(q, 64, 23, True)
+    kept = torch.empty(q.qsim_vjp_kept(desc) // 4, device="cuda")
+    scratch = torch.empty((q.qsim_vjp_workspace(desc) - q.qsim_vjp_kept(desc)) // 4, device="cuda")
+    loss, gx = torch.zeros(64, device="cuda"), torch.zeros_like(x)
+    q.qsim_rollout_vjp_keep(desc, veh, s0, prm, None, x, loss, None, kept, scratch)
+    desc.H += 40
+    for k, s in ((kept, torch.empty(1 << 24, device="cuda")), (torch.empty(1 << 22, device="cuda"), scratch[:100])):
+        with pytest.raises(q.QsimError, match="workspace parts"):
+            q.qsim_rollout_vjp_from(desc, veh, s0, prm, None, x, None, None, gx, None, k, s)
