@@ -576,6 +576,8 @@ def qsim_rollout_vjp_reverse(desc: QsimVjpDesc, veh: QsimParams, s0, params, act
                              g_actions, g_actor, g_params, workspace, stream=None):
     """The reverse sweep on a workspace that qsim_rollout_vjp filled for the same inputs."""
     load()
+    if not isinstance(workspace, int) and _bytes(workspace) < qsim_vjp_workspace(desc):
+        raise ValueError(f"workspace of {_bytes(workspace)} bytes, the descriptor needs {qsim_vjp_workspace(desc)}")
     _chk(_lib.qsim_rollout_vjp_reverse(C.byref(desc), C.byref(veh), _ptr(s0), _ptr(params),
                                        _ptr(actions), _ptr(actor), _ptr(seed), _ptr(g_actions),
                                        _ptr(g_actor), _ptr(g_params), _ptr(workspace),
