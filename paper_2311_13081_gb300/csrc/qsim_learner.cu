@@ -29,6 +29,7 @@
 #include "qsim_smlp.cuh"
 #include "qsim_internal.h"
 #include "qsim_recalc.cuh"
+#include "qsim_staging.h"
 #include "qsim_tcgen05.cuh"
 #include "qsim_tcmlp.cuh"
 
@@ -1832,62 +1833,6 @@ static double run_cost(const ac_handle* a, const qsim_handle* e, int nS) {
     return env + std::max(1, (int)a->cfg.updates_per_step) * upd;
 }
 
-// The calling thread's pinned staging for the batched launch's descriptors.  From pageable
-// memory the upload waited for everything before it on the stream (the previous launch), so
-// consecutive calls left the GPU idle for the whole of their host work.  Two slots in turn: a
-// call waits only if the copy of the call before the last has not run yet.  At most two
-// buffers of the largest call's descriptors (~1 KB a run), freed when the thread ends.
-struct Staging {
-    void* p[2] = {nullptr, nullptr};
-    size_t cap[2] = {0, 0};
-    cudaEvent_t ev[2] = {nullptr, nullptr};
-    int dev = -1, turn = 0;
-    void release() {
-        for (int i = 0; i < 2; ++i) {
-            if (ev[i]) {
-                cudaEventSynchronize(ev[i]);
-                cudaEventDestroy(ev[i]);
-            }
-            if (p[i]) cudaFreeHost(p[i]);
-            p[i] = nullptr;
-            ev[i] = nullptr;
-            cap[i] = 0;
-        }
-        cudaGetLastError();
-    }
-    ~Staging() { release(); }
-    // Space for `bytes`, or null (the caller then copies from pageable memory).
-    void* take(size_t bytes) {
-        int d = -1;
-        if (cudaGetDevice(&d) != cudaSuccess) return nullptr;
-        if (d != dev) {  // events belong to a device
-            release();
-            dev = d;
-        }
-        const int i = turn;
-        bool ok = ev[i] || cudaEventCreateWithFlags(&ev[i], cudaEventDisableTiming) == cudaSuccess;
-        ok = ok && cudaEventSynchronize(ev[i]) == cudaSuccess;
-        if (ok && cap[i] < bytes) {
-            if (p[i]) cudaFreeHost(p[i]);
-            p[i] = nullptr;
-            cap[i] = 0;
-            ok = cudaHostAlloc(&p[i], bytes, cudaHostAllocDefault) == cudaSuccess;
-            if (ok) cap[i] = bytes;
-            else p[i] = nullptr;
-        }
-        if (!ok) {
-            cudaGetLastError();
-            return nullptr;
-        }
-        return p[i];
-    }
-    // The space taken last is read by the work submitted to st so far.
-    void used(cudaStream_t st) {
-        cudaEventRecord(ev[turn], st);
-        turn ^= 1;
-    }
-};
-
 static qsim_status launch_train(std::vector<ac_handle*>& A, std::vector<qsim_handle*>& E,
                                 int64_t n_iters, int do_env, int nS, cudaStream_t st,
                                 int n_clusters_in) {
@@ -1932,12 +1877,12 @@ static qsim_status launch_train(std::vector<ac_handle*>& A, std::vector<qsim_han
                  o_scr = o_off + up(sizeof(int) * (n_clusters + 1));
     unsigned char* dev;
     QCHECK_CUDA(cudaMallocAsync((void**)&dev, o_scr + sizeof(float) * stride * (size_t)n_clusters * nS, st));
-    static thread_local Staging staging;
     // (a captured copy keeps its source's address: not the staging's, which is reused)
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaStreamIsCapturing(st, &cap);
     std::vector<unsigned char> pageable;
-    unsigned char* host = cap == cudaStreamCaptureStatusNone ? (unsigned char*)staging.take(o_scr) : nullptr;
+    Staging* const staging = cap == cudaStreamCaptureStatusNone ? staging_slot() : nullptr;
+    unsigned char* host = staging ? (unsigned char*)staging->take(o_scr) : nullptr;
     const bool pinned = host != nullptr;
     if (!pinned) {
         pageable.resize(o_scr);
@@ -1947,7 +1892,7 @@ static qsim_status launch_train(std::vector<ac_handle*>& A, std::vector<qsim_han
     memcpy(host + o_order, order.data(), sizeof(int) * n);
     memcpy(host + o_off, off.data(), sizeof(int) * (n_clusters + 1));
     const cudaError_t ce = cudaMemcpyAsync(dev, host, o_scr, cudaMemcpyHostToDevice, st);
-    if (pinned) staging.used(st);
+    if (pinned) staging->used(st);
     if (ce != cudaSuccess) {
         cudaFreeAsync(dev, st);
         return cuda_fail(ce, "ac_train: descriptors");
