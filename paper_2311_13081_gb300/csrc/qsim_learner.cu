@@ -1751,6 +1751,34 @@ static qsim_status launch_k_train(int grid, int nS, cudaStream_t st, RunDesc* d_
     return QSIM_OK;
 }
 
+// Host to device copy of pageable `src`, which may go when this returns.  Outside stream capture
+// the copy is staged by then; a captured copy reads its source at every replay, so that the
+// bytes then belong to the graph.
+static cudaError_t upload_pageable(void* dst, const void* src, size_t bytes, cudaStream_t st) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    cudaGraph_t graph = nullptr;
+    cudaError_t e = cudaStreamGetCaptureInfo(st, &status, nullptr, &graph);
+    if (e != cudaSuccess) return e;
+    if (status == cudaStreamCaptureStatusActive) {
+        void* own = malloc(bytes);
+        if (!own) return cudaErrorMemoryAllocation;
+        memcpy(own, src, bytes);
+        cudaUserObject_t obj;
+        e = cudaUserObjectCreate(&obj, own, free, 1, cudaUserObjectNoDestructorSync);
+        if (e != cudaSuccess) {
+            free(own);
+            return e;
+        }
+        e = cudaGraphRetainUserObject(graph, obj, 1, cudaGraphUserObjectMove);
+        if (e != cudaSuccess) {
+            cudaUserObjectRelease(obj, 1);
+            return e;
+        }
+        src = own;
+    }
+    return cudaMemcpyAsync(dst, src, bytes, cudaMemcpyHostToDevice, st);
+}
+
 // One run, one launch of n_iters iterations.  desc_dev holds a PackedRun; when `mirror`
 // is given it is the host copy of what desc_dev holds once the stream's earlier work has
 // run, and the descriptor is uploaded only if the handles' state differs from it.
@@ -1764,8 +1792,7 @@ static qsim_status run_single(ac_handle* a, qsim_handle* env, int64_t n_iters, i
     pk.off[1] = 1;
     PackedRun* d_pk = reinterpret_cast<PackedRun*>(desc_dev);
     if (!mirror || memcmp(&pk.run, mirror, sizeof(RunDesc)) != 0) {
-        // pageable source: the copy is staged before the call returns
-        QCHECK_CUDA(cudaMemcpyAsync(d_pk, &pk, sizeof(pk), cudaMemcpyHostToDevice, st));
+        QCHECK_CUDA(upload_pageable(d_pk, &pk, sizeof(pk), st));
     }
     s = launch_k_train(L.nS, L.nS, st, &d_pk->run, d_pk->order, d_pk->off, n_iters, do_env, scratch, L.stride,
                        tc_wanted(pk.run, L.nS) ? 1 : 0);
@@ -1877,7 +1904,7 @@ static qsim_status launch_train(std::vector<ac_handle*>& A, std::vector<qsim_han
                  o_scr = o_off + up(sizeof(int) * (n_clusters + 1));
     unsigned char* dev;
     QCHECK_CUDA(cudaMallocAsync((void**)&dev, o_scr + sizeof(float) * stride * (size_t)n_clusters * nS, st));
-    // (a captured copy keeps its source's address: not the staging's, which is reused)
+    // (not under capture: the staging is reused, and a replay reads the copy's source again)
     cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
     cudaStreamIsCapturing(st, &cap);
     std::vector<unsigned char> pageable;
@@ -1891,7 +1918,8 @@ static qsim_status launch_train(std::vector<ac_handle*>& A, std::vector<qsim_han
     memcpy(host, D.data(), sizeof(RunDesc) * n);
     memcpy(host + o_order, order.data(), sizeof(int) * n);
     memcpy(host + o_off, off.data(), sizeof(int) * (n_clusters + 1));
-    const cudaError_t ce = cudaMemcpyAsync(dev, host, o_scr, cudaMemcpyHostToDevice, st);
+    const cudaError_t ce = pinned ? cudaMemcpyAsync(dev, host, o_scr, cudaMemcpyHostToDevice, st)
+                                  : upload_pageable(dev, host, o_scr, st);
     if (pinned) staging->used(st);
     if (ce != cudaSuccess) {
         cudaFreeAsync(dev, st);
