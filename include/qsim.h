@@ -411,8 +411,9 @@ int32_t ac_set_cluster(ac_handle* a, int32_t cluster);
  * ac_update; the learner and env handles still supply every input and output.
  * Differences:
  *  - Scratch (activations, partial gradients, the run descriptor) lives in a static
- *    device array of QSIM_STATIC_SCRATCH_BYTES (+ QSIM_STATIC_DESC_BYTES) that every GPU
- *    which loads the library holds until the process exits.  Configurations needing more
+ *    device array of QSIM_STATIC_SCRATCH_BYTES (+ 1 MiB for the tensor-core form of a run that
+ *    fits otherwise, + QSIM_STATIC_DESC_BYTES) that every GPU which loads the library holds
+ *    until the process exits.  Configurations needing more
  *    scratch (large batch x hidden, see the error message) return QSIM_EINVAL.
  *  - The call makes no cudaMalloc / cudaFree and calls no allocating library routine.
  *  - The first call on each device looks up the array's device address

@@ -179,10 +179,11 @@ __device__ __forceinline__ unsigned char* net_img(const Scr& S, float* scr_base,
 // Networks' halves per CTA of a cluster of nS: network n lies in the scratch of rank n mod nS.
 __host__ __device__ constexpr int imgs_per_cta(int nS) { return (6 + nS - 1) / nS; }
 
+// (tiles: as the tensor-core passes lay it out, else in FP32 rows)
 __host__ __device__ inline size_t scratch_floats(int Bc, int H, int DA, int DC, int PA, int PC,
-                                                 int n_env, int nS) {
+                                                 int n_env, int nS, bool tiles) {
     size_t f = 0;
-    if (tce::shape_ok(Bc, H, DA, DC)) {
+    if (tiles) {
         f += 4 * (size_t)(Bc / tce::TR) * tce::TILE_FLOATS;              // oa oa2 oc oc2: input tiles
         f += (size_t)(tce::KP + 1) * Bc;                                 // x32 xn
         f += (size_t)imgs_per_cta(nS) * tce::img_floats(H);              // img
@@ -195,6 +196,10 @@ __host__ __device__ inline size_t scratch_floats(int Bc, int H, int DA, int DC, 
     f += (size_t)PA + 2 * (size_t)PC + 8;             // partial grads + loss
     f += (size_t)n_env * (DA + 2 * H + 4);            // env-step tile
     return (f + 31) & ~(size_t)31;
+}
+
+__host__ __device__ inline size_t scratch_floats(int Bc, int H, int DA, int DC, int PA, int PC, int n_env, int nS) {
+    return scratch_floats(Bc, H, DA, DC, PA, PC, n_env, nS, tce::shape_ok(Bc, H, DA, DC));
 }
 
 __device__ Scr carve(float* base, int Bc, int H, int DA, int DC, int PA, int PC, int n_env, int nS, bool tiles) {
@@ -2064,7 +2069,11 @@ extern "C" qsim_status ac_update(ac_handle* a, qsim_handle* env, int32_t n_updat
 // (held from library load until process exit), plus room for the run descriptor.
 // Host code must not pass the symbol itself to a kernel (in host code it names a host-side
 // stand-in); the device address comes from cudaGetSymbolAddress, looked up once per device.
-static __device__ __align__(256) float g_static_scratch[QSIM_STATIC_SCRATCH_BYTES / sizeof(float)];
+// A run fits if its scratch in FP32 rows does, or that in tiles: the tensor-core passes' tiles and
+// halves take up to 0.7 MiB more than the rows (181,248 floats at hidden 32, batch 1,024, no
+// history, cluster 4; all shapes ac_create takes), for which the array has room.
+constexpr size_t kStaticArea = QSIM_STATIC_SCRATCH_BYTES + (1u << 20);
+static __device__ __align__(256) float g_static_scratch[kStaticArea / sizeof(float)];
 static __device__ __align__(256) unsigned char g_static_desc[QSIM_STATIC_DESC_BYTES];
 
 namespace {
@@ -2103,8 +2112,10 @@ extern "C" qsim_status ac_update_static(ac_handle* a, qsim_handle* env, int32_t 
     SingleRun L;
     qsim_status st = prepare_single(a, env, 0, n_updates, "ac_update_static", &L);
     if (st != QSIM_OK || n_updates == 0) return st;
-    const size_t need = L.stride * sizeof(float) * (size_t)L.nS;
-    if (need > QSIM_STATIC_SCRATCH_BYTES)
+    const size_t per_cta = std::min(L.stride, scratch_floats(a->batch / L.nS, a->hidden, a->obs_dim, a->critic_in,
+                                                             a->n_actor, a->n_critic, env->n, L.nS, false));
+    const size_t need = per_cta * sizeof(float) * (size_t)L.nS;
+    if (need > QSIM_STATIC_SCRATCH_BYTES || L.stride * sizeof(float) * (size_t)L.nS > kStaticArea)
         return fail(QSIM_EINVAL,
                     "ac_update_static: needs %zu bytes of scratch (batch %d, hidden %d, cluster %d), "
                     "more than the static maximum of %d bytes; use ac_update",

@@ -77,3 +77,42 @@ def test_static_update_rejects_oversized_configuration(gpu):
     finally:
         q.ac_destroy(a)
         q.qsim_destroy(h)
+
+
+@pytest.mark.parametrize("hidden,batch,n_hist", [(32, 256, 0), (64, 128, 16), (128, 128, 16)])
+def test_static_update_takes_what_fits_in_rows(gpu, hidden, batch, n_hist):
+    """A run whose scratch fits the array in FP32 rows, by a few floats, but not in the tiles
+    of the tensor-core passes is taken and gives ac_update's results."""
+    q = gpu
+    made = []
+    try:
+        for _ in range(2):
+            d, cfg, veh = lib_config(q, "c1", n_envs=1, capacity=24, learning_starts=0, n_hist=n_hist)
+            h = q.qsim_create(cfg, veh)
+            info = q.qsim_info_get(h)
+            q.qsim_destroy(h)
+            DA, DC = info["obs_dim"], info["critic_obs_dim"] + 4
+            PA, PC = q.param_count(DA, hidden, 4), q.param_count(DC, hidden, 1)
+            fixed = 2 * batch * (DA + DC) + 8 * batch * hidden + 17 * batch + PA + 2 * PC + 8
+            n = ((8 << 20) // 4 - 32 - fixed) // (DA + 2 * hidden + 4)
+            d, cfg, veh = lib_config(q, "c1", n_envs=n, capacity=24, learning_starts=0, n_hist=n_hist, episode_len=12)
+            h = q.qsim_create(cfg, veh)
+            hp = dict(W.TD3)
+            hp.update(hidden=hidden, batch=batch)
+            a = q.ac_create(q.make_ac_config(hp, cluster=1), h)
+            made.append((h, a))
+            ld = q.qsim_info_get(h)["ld"]
+            for k in range(22):
+                q.qsim_step(h, torch.tensor(W.random_actions(70 + k, (4, ld)), dtype=torch.float32, device="cuda"))
+        (h1, a1), (h2, a2) = made
+        for _ in range(2):
+            q.ac_update(a1, h1, 1)
+            q.ac_update_static(a2, h2, 1)
+        torch.cuda.synchronize()
+        A1, A2 = q.ac_info_get(a1), q.ac_info_get(a2)
+        for k in NETS + ("stats",):
+            assert np.array_equal(cpu(A1[k]).view(np.uint32), cpu(A2[k]).view(np.uint32)), k
+    finally:
+        for h, a in made:
+            q.ac_destroy(a)
+            q.qsim_destroy(h)
