@@ -199,7 +199,10 @@ qsim_status qsim_sync(qsim_handle* h);
  * of the default length), tensor memory is released and the kernel returns, so later
  * calls run normally.  The env set's contents are then those of a partly completed call
  * (unspecified, finite if the inputs were), with the counters advanced as for a full
- * call.  A limit far below the
+ * call.  The learner's updates on this env set wait for the tensor cores under the same
+ * limit: when one runs out, the run's networks whose gradients are not complete keep their
+ * weights, targets and moments, the run's other updates of that call are left out, and the
+ * counters advance as for a full call.  A limit far below the
  * MMA latency (a few thousand cycles) makes the waits run out on purpose, which is how
  * the failure path is tested.  Returns the previous limit, or a negative qsim_status.
  * (No counterpart in the paper.) */

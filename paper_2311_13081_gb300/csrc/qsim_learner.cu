@@ -1342,10 +1342,12 @@ __device__ __noinline__ float critics_smem(const RunDesc& R, const Scr& S, int B
 // One CTA, 256 samples, us (SIMT engine -> here): hidden 64: target actor 20 -> 13, target
 // critics 34 -> 19, mu 18 -> 11, dQ/da 55 -> 15, actor gradient 105 -> 26; hidden 128:
 // regression 404 -> 108, actor gradient 234 -> 43.
+// False (on every CTA of the cluster) when a wait for the tensor cores ran out on one of them:
+// the networks whose gradients were not complete by then are left as they were.
 template <int H>
-__device__ __noinline__ void td3_update_tc(RunDesc& R, int64_t head, int64_t size, int64_t t_now, uint32_t u,
+__device__ __noinline__ bool td3_update_tc(RunDesc& R, int64_t head, int64_t size, int64_t t_now, uint32_t u,
                                            int64_t& t_a, int64_t& t_c, const Scr& S, float* scr_base,
-                                           size_t scr_stride, int rk, int nS, float* sm, uint32_t tmem) {
+                                           size_t scr_stride, int rk, int nS, float* sm, uint32_t tmem, int* dead) {
     using namespace tce;
     const int B = R.B, Bc = B / nS, PA = R.PA, PC = R.PC, DA = R.DA, DC = R.DC;
     const LearnHyper& hp = R.hp;
@@ -1360,6 +1362,19 @@ __device__ __noinline__ void td3_update_tc(RunDesc& R, int64_t head, int64_t siz
     auto img = [&](Net n) { return net_img(S, scr_base, scr_stride, rk, nS, H, n); };
     Args f{};
     f.Bc = Bc;
+    f.limit = R.C.wait_limit;
+    f.dead = dead;
+    // (a pass ends with a barrier of the CTA, so that all of its threads see the flag alike)
+    auto alive = [&] { return *reinterpret_cast<volatile int*>(dead) == 0; };
+    // Before a cluster barrier each CTA posts its flag; after it, whether all are alive.
+    auto post = [&](int k) {
+        if (nS > 1 && threadIdx.x == 0) S.loss[k] = alive() ? 0.0f : 1.0f;
+    };
+    auto all_alive = [&](int k) {
+        if (nS == 1) return alive();
+        const float* p = cl0 + (size_t)(threadIdx.x < (unsigned)nS ? threadIdx.x : 0) * scr_stride + (S.loss - scr_base);
+        return __syncthreads_or(ldcg(p + k) != 0.0f) == 0;
+    };
     f.x32 = S.x32;
     f.xn = S.xn;
     f.invB = invB;
@@ -1389,22 +1404,22 @@ __device__ __noinline__ void td3_update_tc(RunDesc& R, int64_t head, int64_t siz
     // twin target critics, clipped double-Q target
     f.in = DC; f.out = 1; f.X = S.oc2; f.tanh_out = false;
     f.W = R.c1_t; f.img = img(N_C1_T); f.Y = S.q1;
-    pass<H, FWD>(f, sm, tmem, st);
+    if (alive()) pass<H, FWD>(f, sm, tmem, st);
     f.W = R.c2_t; f.img = img(N_C2_T); f.Y = S.q2;
-    pass<H, FWD>(f, sm, tmem, st);
+    if (alive()) pass<H, FWD>(f, sm, tmem, st);
     for (int jl = threadIdx.x; jl < Bc; jl += LT) {
         const float qmin = fminf(ldcg(S.q1 + jl), ldcg(S.q2 + jl));
         S.y[jl] = S.r[jl] + (S.term[jl] != 0.0f ? 0.0f : hp.gamma * qmin);
     }
     __syncthreads();
     // critic regression
-    float lsum;
+    float lsum = 0.0f;
     if constexpr (H == 128) {
         f.X = S.oc; f.y = S.y;
         f.W = R.c1; f.img = img(N_C1); f.G = S.g1;
-        lsum = pass<H, CRIT>(f, sm, tmem, st);
+        if (alive()) lsum = pass<H, CRIT>(f, sm, tmem, st);
         f.W = R.c2; f.img = img(N_C2); f.G = S.g2;
-        lsum += pass<H, CRIT>(f, sm, tmem, st);
+        if (alive()) lsum += pass<H, CRIT>(f, sm, tmem, st);
     } else if (DC == 90) {
         lsum = critics_smem<H, 90>(R, S, Bc, DC, sm);
     } else if (H == 64 && DC == 96) {
@@ -1414,7 +1429,9 @@ __device__ __noinline__ void td3_update_tc(RunDesc& R, int64_t head, int64_t siz
     }
     lsum = block_sum(lsum, red);
     if (threadIdx.x == 0) S.loss[0] = lsum;
+    post(2);
     cluster_sync_all(nS);
+    if (!all_alive(2)) return false;
     t_c += 1;
     {
         const int lo = (int)((int64_t)PC * rk / nS), hi = (int)((int64_t)PC * (rk + 1) / nS);
@@ -1431,17 +1448,19 @@ __device__ __noinline__ void td3_update_tc(RunDesc& R, int64_t head, int64_t siz
         }
     }
     cluster_sync_all(nS);
-    if (!pol) return;
+    if (!pol) return true;
     // delayed actor update through the updated first critic
     f.W = R.actor; f.img = img(N_ACTOR); f.in = DA; f.out = 4; f.X = S.oa; f.Y = S.mu; f.tanh_out = true;
     pass<H, FWD>(f, sm, tmem, st);
     f.W = R.c1; f.img = img(N_C1); f.in = DC; f.out = 1; f.X = S.oc; f.mu = S.mu; f.da = S.da;
-    float qs = pass<H, DQ>(f, sm, tmem, st);
+    float qs = alive() ? pass<H, DQ>(f, sm, tmem, st) : 0.0f;
     f.W = R.actor; f.img = img(N_ACTOR); f.in = DA; f.out = 4; f.X = S.oa; f.G = S.ga;
-    pass<H, ACT>(f, sm, tmem, st);
+    if (alive()) pass<H, ACT>(f, sm, tmem, st);
     qs = block_sum(qs, red);
     if (threadIdx.x == 0) S.loss[1] = qs;
+    post(3);
     cluster_sync_all(nS);
+    if (!all_alive(3)) return false;
     t_a += 1;
     {
         const int lo = (int)((int64_t)PA * rk / nS), hi = (int)((int64_t)PA * (rk + 1) / nS);
@@ -1454,6 +1473,7 @@ __device__ __noinline__ void td3_update_tc(RunDesc& R, int64_t head, int64_t siz
         }
     }
     cluster_sync_all(nS);
+    return true;
 }
 
 // Curriculum change + reward recalculation over the run's buffer, split over the cluster.
@@ -1481,6 +1501,7 @@ __global__ void __launch_bounds__(LT) k_train(RunDesc* runs, const int* order, c
     extern __shared__ __align__(16) float sm[];
     // tensor memory for the tensor-core passes, when some run of the launch has them
     __shared__ uint32_t tmem_slot;
+    __shared__ int dead;  // a wait for the tensor cores ran out
     if (use_tc) {
         if ((threadIdx.x >> 5) == 0) {
             asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
@@ -1502,7 +1523,9 @@ __global__ void __launch_bounds__(LT) k_train(RunDesc* runs, const int* order, c
         const int Bc = R.B / nS;
         const bool tiles = use_tc && tce::shape_ok(Bc, R.H, R.DA, R.DC);  // tensor-core passes
         const Scr S = carve(my, Bc, R.H, R.DA, R.DC, R.PA, R.PC, R.n_env, nS, tiles);
+        bool updating = true;  // until a wait runs out: the launch's other updates of the run are then left out
         if (tiles) {
+            if (threadIdx.x == 0) dead = 0;
             // the networks' halves for the tensor-core passes, shared out over the cluster
             const float* nets[6] = {R.actor, R.actor_t, R.c1, R.c1_t, R.c2, R.c2_t};
             for (int n = rk; n < 6; n += nS)
@@ -1534,12 +1557,18 @@ __global__ void __launch_bounds__(LT) k_train(RunDesc* runs, const int* order, c
             const bool resident128 = R.H == 128 && R.DA == 82 && R.DC == 90;
             for (int k = 0; k < n_upd; ++k) {
                 if (tiles) {
-                    if (R.H == 64)
-                        td3_update_tc<64>(R, head, size, t_now, (uint32_t)u, t_a, t_c, S, my, scr_stride, rk, nS, sm, tmem);
-                    else if (R.H == 32)
-                        td3_update_tc<32>(R, head, size, t_now, (uint32_t)u, t_a, t_c, S, my, scr_stride, rk, nS, sm, tmem);
-                    else
-                        td3_update_tc<128>(R, head, size, t_now, (uint32_t)u, t_a, t_c, S, my, scr_stride, rk, nS, sm, tmem);
+                    // (the counters advance as the host expects, whatever became of the update)
+                    const int64_t a1 = t_a + ((uint32_t)u % (uint32_t)R.hp.policy_delay == (uint32_t)(R.hp.policy_delay - 1));
+                    const int64_t c1 = t_c + 1;
+                    if (updating)
+                        updating = R.H == 64   ? td3_update_tc<64>(R, head, size, t_now, (uint32_t)u, t_a, t_c, S, my,
+                                                                   scr_stride, rk, nS, sm, tmem, &dead)
+                                   : R.H == 32 ? td3_update_tc<32>(R, head, size, t_now, (uint32_t)u, t_a, t_c, S, my,
+                                                                   scr_stride, rk, nS, sm, tmem, &dead)
+                                               : td3_update_tc<128>(R, head, size, t_now, (uint32_t)u, t_a, t_c, S, my,
+                                                                    scr_stride, rk, nS, sm, tmem, &dead);
+                    t_a = a1;
+                    t_c = c1;
                 } else if (resident) {
                     // specialised shapes: hidden 64 or 32 over 16 actions of history, and the
                     // privileged critic (82 + 4 + 6 motor/parameter inputs + 4 actions)

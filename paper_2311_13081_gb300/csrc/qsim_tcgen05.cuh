@@ -42,12 +42,18 @@ __device__ __forceinline__ void bar_init(uint32_t bar, uint32_t count) {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 }
 
-// Waits (bounded) for the phase of `bar` with the given parity; false when it gave up.
+// Waits (bounded) for the phase of `bar` with the given parity; false when it gave up.  The first
+// poll only looks: a try_wait may sleep longer than a short chain of MMAs takes, and a limit
+// of one poll would then not run out.
 __device__ __forceinline__ bool bar_wait(uint32_t bar, uint32_t parity, int limit) {
     for (int i = 0; i < limit; ++i) {
         uint32_t done;
-        asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
-                     "selp.u32 %0, 1, 0, p;\n}" : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+        if (i == 0)
+            asm volatile("{\n.reg .pred p;\nmbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+                         "selp.u32 %0, 1, 0, p;\n}" : "=r"(done) : "r"(bar), "r"(parity) : "memory");
+        else
+            asm volatile("{\n.reg .pred p;\nmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+                         "selp.u32 %0, 1, 0, p;\n}" : "=r"(done) : "r"(bar), "r"(parity) : "memory");
         if (done) return true;
     }
     return false;

@@ -38,7 +38,7 @@ constexpr int TR = 128;               // rows of a tile
 constexpr int TILE_HALVES = TR * KP;  // one half (hi or lo) of an input tile
 constexpr int TILE_FLOATS = TILE_HALVES;  // a tile in scratch: hi then lo
 constexpr int TMEM_COLS = 512;
-constexpr int WAIT_POLLS = 1 << 24;
+constexpr int DRAIN_POLLS = 1 << 24;
 
 enum Mode { FWD, CRIT, DQ, ACT };
 
@@ -347,6 +347,8 @@ struct Args {
     const float* mu; // DQ: actions that take the input's last 4 columns [Bc][4]
     float* da;       // DQ: out, dLoss/d(actor pre-activation) [Bc][4]; ACT: in
     const unsigned char* img;  // halves of W1 and W2
+    int limit;    // polls of a wait before it gives up
+    int* dead;    // shared flag: a wait of this CTA gave up (what the passes left is not to be used)
     const float* x32;  // CRIT: the FP32 inputs [Bc][in] and each row's sum of magnitudes [Bc]
     const float* xn;
 };
@@ -393,8 +395,15 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
     const float* gW3 = gb2 + H;
     const float* gb3 = gW3 + out * H;
     uint32_t ph0 = 0, ph1 = 0;
+    // A wait that gives up marks the pass and then, once, waits on with a limit of its own: the
+    // MMAs in flight are over before the operands, accumulators and barriers are used again.
+    bool stuck = false;
     auto wait = [&](uint32_t bar, uint32_t& ph) {
-        if (!tc::bar_wait(bar, ph, WAIT_POLLS) && lane == 0 && status) atomicCAS(status, DEV_OK, DEV_TIMEOUT);
+        if (!stuck && !tc::bar_wait(bar, ph, a.limit)) {
+            *a.dead = 1;
+            if (lane == 0 && status) atomicCAS(status, DEV_OK, DEV_TIMEOUT);
+            stuck = !tc::bar_wait(bar, ph, DRAIN_POLLS);
+        }
         ph ^= 1u;
         tc::fence_after();
     };

@@ -1,12 +1,13 @@
 """The learner's tensor-core passes (CTAs of whole 128-sample tiles) at the edges of their range:
 one to four tiles, every hidden width, narrow and full inputs, clusters, every critic layout;
 against the FP64 oracle with the tolerances of the other update tests."""
+import numpy as np
 import pytest
 import torch
 
 import oracle as O
-from helpers import assert_close, f64
-from test_gpu_learner import check_update, make_run, oracle_buffer, oracle_learner
+from helpers import assert_close, cpu, f64
+from test_gpu_learner import NETS, check_update, make_run, oracle_buffer, oracle_learner
 
 pytestmark = pytest.mark.gpu
 
@@ -33,6 +34,39 @@ def test_tile_update_parity(gpu, hidden, batch, cluster, layout, n_hist):
             ai = q.ac_info_get(a)
             check_update(ai, L, dg, hp, f"update{call}")
             assert_close(f64(ai["stats"])[0], dg["critic_loss"], 1.0, what="critic loss")
+    finally:
+        q.ac_destroy(a)
+        q.qsim_destroy(h)
+
+
+@pytest.mark.parametrize("hidden,batch,cluster", [(32, 128, 1), (64, 256, 2), (128, 256, 1), (128, 512, 4)])
+def test_wait_that_runs_out_leaves_the_networks_alone(gpu, hidden, batch, cluster):
+    """A one-poll limit on the env set: qsim_sync reports QSIM_ETIMEOUT, no weight, target or
+    moment has changed, the counters stand where a full call leaves them, and with the
+    default limit the next updates match the oracle."""
+    q = gpu
+    d, h, a, hp = make_run(q, hidden=hidden, batch=batch, cluster=cluster)
+    try:
+        q.ac_update(a, h, 2)
+        q.qsim_sync(h)
+        before = {k: cpu(q.ac_info_get(a)[k]).view(np.uint32).copy() for k in NETS}
+        q.qsim_set_wait_limit(h, 1)
+        q.ac_update(a, h, 3)
+        with pytest.raises(q.QsimError) as ei:
+            q.qsim_sync(h)
+        assert ei.value.status == -4
+        ai = q.ac_info_get(a)
+        for k in NETS:
+            assert np.array_equal(cpu(ai[k]).view(np.uint32), before[k]), k
+        assert (ai["updates"], ai["t_critic"], ai["t_actor"]) == (5, 5, 2)
+        q.qsim_set_wait_limit(h, 0)
+        for call in range(2):
+            info = q.qsim_info_get(h)
+            L = oracle_learner(q.ac_info_get(a))
+            q.ac_update(a, h, 1)
+            q.qsim_sync(h)
+            dg = O.td3_update(d, hp, L, oracle_buffer(info, info["n_envs"]))
+            check_update(q.ac_info_get(a), L, dg, hp, f"update{call}")
     finally:
         q.ac_destroy(a)
         q.qsim_destroy(h)
