@@ -685,6 +685,8 @@ constexpr int GS = 256, GP = GS + 1;  // samples a pass; row stride (odd: lanes 
 constexpr int R_S = 0, R_S2 = NS, R_A = 2 * NS, R_L = R_A + 4, R_PV = R_L + 4 * HMAX, R_R = R_PV + NPRIV,
               R_O = R_R + 1, R_O2 = R_O + 18, R_ON = R_O2 + 18, R_ON2 = R_ON + 18, ROWS = R_ON2 + 18;
 constexpr int MAPS = 128;  // entries of a column map (input widths are below that)
+constexpr int XE = 4;      // passes of the largest batch
+static_assert(GS == tce::TILES_X * tce::TR, "an exponent a pass");
 static_assert(ROWS * GP + 3 * GS + 4 * MAPS / 2 <= SMEM_MAIN, "gather tile");
 
 // 4 bytes global -> shared, zero when !ok (nothing is read then)
@@ -696,7 +698,8 @@ __device__ __forceinline__ void cp4(float* dst, const float* src, bool ok) {
 
 template <bool TILES>
 __device__ __noinline__ void gather_pass(const RunDesc& R, int j0, int Bc, int g0, int G, uint32_t u, int64_t head,
-                                         int64_t size, int64_t t_now, const Scr& S, float* sm, bool need_oa) {
+                                         int64_t size, int64_t t_now, const Scr& S, float* sm, bool need_oa,
+                                         int* xe, bool plain_next) {
     using namespace gat;
     const EnvCfg& C = R.C;
     const int ld = C.ld, F = C.F, NE = R.n_env, DA = R.DA, DC = R.DC, nh = C.n_hist;
@@ -835,14 +838,57 @@ __device__ __noinline__ void gather_pass(const RunDesc& R, int j0, int Bc, int g
         // 8 samples make 128); o_c' gets the target action later.  A warp keeps a column
         // group's tile rows for all of its samples.
         constexpr int KC = tce::KC1;
-        for (int js = tid; R.H == 128 && js < G; js += LT) {
-            float n = 0.0f;
-            if (m_env[js] >= 0) {
+        const bool need_oc = need_oa || R.H == 128;  // hidden <= 64: o_c's tile is read on the actor's step only
+        // The power of two that this pass's samples are scaled by, one for o_a and o_c and one
+        // for o_a' and o_c' (none where the passes take them plain): their largest magnitude
+        // goes below 2^X_TOP.  Actions that are put in later are at most 1.
+        float mx = 1.0f, mx2 = 1.0f;
+        for (int js = tid; js < G; js += LT) {
+            if (m_env[js] < 0) continue;
+            const float* T = tile + js;
+            if (need_oc) {
+                float n = 0.0f;
 #pragma unroll 8
-                for (int k = 0; k < DC; ++k) n += fabsf(tile[map[2 * MAPS + k] * GP + js]);
+                for (int k = 0; k < DC; ++k) {
+                    const float v = fabsf(T[map[2 * MAPS + k] * GP]);
+                    n += v;
+                    mx = fmaxf(mx, v);
+                }
+                if (R.H == 128) S.xn[g0 + js] = n;
             }
-            S.xn[g0 + js] = n;
+            // (o_a has o_c's columns but for the noise, unless the critic sees no history)
+            if (need_oa)
+#pragma unroll 8
+                for (int k = 0; k < DA; ++k) mx = fmaxf(mx, fabsf(T[map[k] * GP]));
+            if (!plain_next) {
+#pragma unroll 8
+                for (int k = 0; k < DA; ++k) mx2 = fmaxf(mx2, fabsf(T[map[MAPS + k] * GP]));
+#pragma unroll 8
+                for (int k = 0; k < DC - 4; ++k) mx2 = fmaxf(mx2, fabsf(T[map[3 * MAPS + k] * GP]));
+            }
         }
+        {
+            float* red = sm + SMEM_MAIN;
+            for (int o = 16; o > 0; o >>= 1) {
+                mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+                mx2 = fmaxf(mx2, __shfl_xor_sync(0xffffffffu, mx2, o));
+            }
+            if (lane == 0) {
+                red[warp] = mx;
+                red[8 + warp] = mx2;
+            }
+            __syncthreads();
+            for (int i = 0; i < LT / 32; ++i) {
+                mx = fmaxf(mx, red[i]);
+                mx2 = fmaxf(mx2, red[8 + i]);
+            }
+        }
+        const int e_cur = tce::scale_max(tce::X_TOP, mx), e_next = plain_next ? 0 : tce::scale_max(tce::X_TOP, mx2);
+        if (tid == 0) {
+            xe[g0 / GS] = e_cur;
+            xe[XE + g0 / GS] = e_next;
+        }
+        const float x_cur = tce::exp2i(e_cur), x_next = tce::exp2i(e_next);
         // o_c in FP32 rows for the critics' regression, a warp per sample
         float* const x32 = S.x32;
         for (int js = warp; js < G; js += LT / 32) {
@@ -855,7 +901,6 @@ __device__ __noinline__ void gather_pass(const RunDesc& R, int j0, int Bc, int g
                 if (lane + 32 * e < DC) x32[(size_t)(g0 + js) * DC + lane + 32 * e] = v[e];
         }
         float *const t_oa = S.oa, *const t_oa2 = S.oa2, *const t_oc = S.oc, *const t_oc2 = S.oc2;
-        const bool need_oc = need_oa || R.H == 128;  // hidden <= 64: o_c's tile is read on the actor's step only
         for (int q = (need_oa ? 0 : KC) + warp; q < 4 * KC; q += LT / 32) {
             if (!need_oc && q / KC == 2) continue;
             const int mat = q / KC, kc = q - mat * KC;
@@ -869,7 +914,7 @@ __device__ __noinline__ void gather_pass(const RunDesc& R, int j0, int Bc, int g
                 const int js = s0 + lane, j = g0 + js;
                 float v[8];
 #pragma unroll
-                for (int e = 0; e < 8; ++e) v[e] = row8[e] >= 0 ? tile[row8[e] + js] : 0.0f;
+                for (int e = 0; e < 8; ++e) v[e] = row8[e] >= 0 ? tile[row8[e] + js] * (mat & 1 ? x_next : x_cur) : 0.0f;
                 if (m_env[js] < 0) continue;
                 unsigned char* t = reinterpret_cast<unsigned char*>(d + (size_t)(j / tce::TR) * tce::TILE_FLOATS);
                 tce::put8(t, t + 2 * tce::TILE_HALVES, KC, j % tce::TR, 8 * kc, v);
@@ -898,13 +943,15 @@ __device__ __noinline__ void gather_pass(const RunDesc& R, int j0, int Bc, int g
 }
 
 // Gather of this CTA's Bc samples (sm: shared memory, free at this point); need_oa: whether this
-// update reads o_a (the actor's step).
+// update reads o_a (the actor's step).  In tiles: xe gets the passes' exponents, plain_next
+// leaves those of s_{t+1} at zero.
 template <bool TILES>
 __device__ __forceinline__ void gather_all(const RunDesc& R, int j0, int Bc, uint32_t u,
                                            int64_t head, int64_t size, int64_t t_now,
-                                           const Scr& S, float* sm, bool need_oa = true) {
+                                           const Scr& S, float* sm, bool need_oa = true, int* xe = nullptr,
+                                           bool plain_next = true) {
     for (int g0 = 0; g0 < Bc; g0 += gat::GS)
-        gather_pass<TILES>(R, j0, Bc, g0, min(gat::GS, Bc - g0), u, head, size, t_now, S, sm, need_oa);
+        gather_pass<TILES>(R, j0, Bc, g0, min(gat::GS, Bc - g0), u, head, size, t_now, S, sm, need_oa, xe, plain_next);
 }
 
 // Adam on parameters [lo, hi) from the sum of S gradient partials (partial s at
@@ -1330,6 +1377,66 @@ __device__ __noinline__ float critics_smem(const RunDesc& R, const Scr& S, int B
     return lsum;
 }
 
+// What a CTA keeps about the tensor-core passes in shared memory, alike in a cluster: the
+// networks' exponents (of the images), the gathered samples', and whether a wait ran out.
+struct TcState {
+    tce::NetScale net[6];
+    int xe[2 * gat::XE];
+    int dead;
+};
+
+// Whether the passes of the target networks take their operands as they are and in one chain: at
+// hidden 32 and 64, where they feed the critics' FP32 regression and keep the bits they had.
+__host__ __device__ constexpr bool plain_targets(int H) { return H != 128; }
+
+__device__ __forceinline__ float2 block_max2(float a, float b, float* red) {
+    for (int o = 16; o > 0; o >>= 1) {
+        a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, o));
+        b = fmaxf(b, __shfl_xor_sync(0xffffffffu, b, o));
+    }
+    if ((threadIdx.x & 31) == 0) {
+        red[threadIdx.x >> 5] = a;
+        red[8 + (threadIdx.x >> 5)] = b;
+    }
+    __syncthreads();
+    for (int i = 0; i < LT / 32; ++i) {
+        a = fmaxf(a, red[i]);
+        b = fmaxf(b, red[8 + i]);
+    }
+    __syncthreads();
+    return make_float2(a, b);
+}
+
+// Largest magnitudes of a network's W1 and W2.
+__device__ __noinline__ float2 net_max(const float* W, int in, int H, float* red) {
+    float a = 0.0f, b = 0.0f;
+    for (int i = threadIdx.x; i < H * in; i += LT) a = fmaxf(a, fabsf(ldcg(W + i)));
+    for (int i = threadIdx.x; i < H * H; i += LT) b = fmaxf(b, fabsf(ldcg(W + H * in + H + i)));
+    return block_max2(a, b, red);
+}
+
+// Largest magnitudes of W1 and W2 of a network whose image a pass is about to read.  An image
+// whose halves have left their range since it was made (Adam and Polyak keep its exponents)
+// is made again, by its owner; every CTA of the cluster calls and finds the same.
+template <int H>
+__device__ __noinline__ float2 net_check(tce::NetScale& ns, unsigned char* img, const float* W, int in, bool owner, int nS,
+                                         float* red) {
+    using namespace tce;
+    const NetScale e = ns;
+    const float2 m = block_max2(max_half<H * KP>(img), max_half<H * H>(img + 4 * H * KP), red);
+    if (m.x >= kScaleLow && m.x < kScaleTop && m.y >= kScaleLow && m.y < kScaleTop)
+        return make_float2(m.x * exp2i(-e.e1), m.y * exp2i(-e.e2));
+    const float2 w = net_max(W, in, H, red);
+    const NetScale f{scale_max(W_TOP, w.x), scale_max(W_TOP, w.y)};
+    if (f.e1 != e.e1 || f.e2 != e.e2) {
+        if (threadIdx.x == 0) ns = f;
+        cluster_sync_all(nS);  // every CTA has read the image
+        if (owner) img_make(img, W, in, H, f);
+        cluster_sync_all(nS);
+    }
+    return w;
+}
+
 // One TD3 update with its network passes on the tensor cores (tce::pass): a CTA holds whole
 // 128-sample tiles, at most 96 inputs.  Same phases, random streams and cluster reduction as
 // td3_update.  The critics' regression runs there at hidden 128 only; at 32 and 64 it keeps the
@@ -1347,7 +1454,7 @@ __device__ __noinline__ float critics_smem(const RunDesc& R, const Scr& S, int B
 template <int H>
 __device__ __noinline__ bool td3_update_tc(RunDesc& R, int64_t head, int64_t size, int64_t t_now, uint32_t u,
                                            int64_t& t_a, int64_t& t_c, const Scr& S, float* scr_base,
-                                           size_t scr_stride, int rk, int nS, float* sm, uint32_t tmem, int* dead) {
+                                           size_t scr_stride, int rk, int nS, float* sm, uint32_t tmem, TcState& tcs) {
     using namespace tce;
     const int B = R.B, Bc = B / nS, PA = R.PA, PC = R.PC, DA = R.DA, DC = R.DC;
     const LearnHyper& hp = R.hp;
@@ -1356,16 +1463,17 @@ __device__ __noinline__ bool td3_update_tc(RunDesc& R, int64_t head, int64_t siz
     float* red = sm + SMEM_MAIN;
     const float invB = 1.0f / (float)B;
     const bool pol = (int64_t)(u % (uint32_t)hp.policy_delay) == (int64_t)(hp.policy_delay - 1);
-    gather_all<true>(R, j0, Bc, u, head, size, t_now, S, sm, pol);
+    constexpr bool plain = plain_targets(H);
+    gather_all<true>(R, j0, Bc, u, head, size, t_now, S, sm, pol, tcs.xe, plain);
     // target actor + smoothing; the target action goes into o_c' tiles' last columns
     const float* cl0 = scr_base - (size_t)rk * scr_stride;  // scratch of cluster rank 0
     auto img = [&](Net n) { return net_img(S, scr_base, scr_stride, rk, nS, H, n); };
     Args f{};
     f.Bc = Bc;
     f.limit = R.C.wait_limit;
-    f.dead = dead;
+    f.dead = &tcs.dead;
     // (a pass ends with a barrier of the CTA, so that all of its threads see the flag alike)
-    auto alive = [&] { return *reinterpret_cast<volatile int*>(dead) == 0; };
+    auto alive = [&] { return *reinterpret_cast<volatile int*>(&tcs.dead) == 0; };
     // Before a cluster barrier each CTA posts its flag; after it, whether all are alive.
     auto post = [&](int k) {
         if (nS > 1 && threadIdx.x == 0) S.loss[k] = alive() ? 0.0f : 1.0f;
@@ -1378,8 +1486,25 @@ __device__ __noinline__ bool td3_update_tc(RunDesc& R, int64_t head, int64_t siz
     f.x32 = S.x32;
     f.xn = S.xn;
     f.invB = invB;
-    f.W = R.actor_t; f.img = img(N_ACTOR_T); f.in = DA; f.out = 4; f.X = S.oa2; f.Y = S.mu; f.tanh_out = true;
-    pass<H, FWD>(f, sm, tmem, st);
+    // network n with weights W, for a pass with scaled operands
+    auto use = [&](Net n, float* W, int in) {
+        f.W = W; f.img = img(n); f.in = in;
+        const float2 m = net_check<H>(tcs.net[n], img(n), W, in, n % nS == rk, nS, red);
+        f.w1m = m.x; f.w2m = m.y; f.e = tcs.net[n];
+    };
+    // a target network
+    auto target = [&](Net n, float* W, int in) {
+        if constexpr (plain) {
+            f.W = W; f.img = img(n); f.in = in;
+            if (alive()) pass<H, FWD>(f, sm, tmem, st);
+        } else {
+            use(n, W, in);
+            if (alive()) pass<H, FWDX>(f, sm, tmem, st);
+        }
+    };
+    f.xe = tcs.xe + gat::XE;
+    f.out = 4; f.X = S.oa2; f.Y = S.mu; f.tanh_out = true;
+    target(N_ACTOR_T, R.actor_t, DA);
     for (int jl = threadIdx.x; jl < Bc; jl += LT) {
         const uint32_t j = (uint32_t)(j0 + jl);
         const uint4 r0 = draw(R.C, j, u, TAG_SMOOTH, 0), r1 = draw(R.C, j, u, TAG_SMOOTH, 1);
@@ -1391,10 +1516,11 @@ __device__ __noinline__ bool td3_update_tc(RunDesc& R, int64_t head, int64_t siz
             a2[i] = clampf(ldcg(S.mu + jl * 4 + i) + eps, -1.0f, 1.0f);
         }
         unsigned char* t = reinterpret_cast<unsigned char*>(S.oc2 + (size_t)(jl / TR) * TILE_FLOATS);
+        const float sx = exp2i(tcs.xe[gat::XE + jl / gat::GS]);
 #pragma unroll
         for (int i = 0; i < 4; i += 2) {
             uint32_t h, l;
-            tc::split2(a2[i], a2[i + 1], h, l);
+            tc::split2(sx * a2[i], sx * a2[i + 1], h, l);
             const int at = 2 * tc::cano16(jl % TR, DC - 4 + i, KC1);
             *reinterpret_cast<uint32_t*>(t + at) = h;
             *reinterpret_cast<uint32_t*>(t + 2 * TILE_HALVES + at) = l;
@@ -1402,11 +1528,11 @@ __device__ __noinline__ bool td3_update_tc(RunDesc& R, int64_t head, int64_t siz
     }
     __syncthreads();
     // twin target critics, clipped double-Q target
-    f.in = DC; f.out = 1; f.X = S.oc2; f.tanh_out = false;
-    f.W = R.c1_t; f.img = img(N_C1_T); f.Y = S.q1;
-    if (alive()) pass<H, FWD>(f, sm, tmem, st);
-    f.W = R.c2_t; f.img = img(N_C2_T); f.Y = S.q2;
-    if (alive()) pass<H, FWD>(f, sm, tmem, st);
+    f.out = 1; f.X = S.oc2; f.tanh_out = false;
+    f.Y = S.q1;
+    target(N_C1_T, R.c1_t, DC);
+    f.Y = S.q2;
+    target(N_C2_T, R.c2_t, DC);
     for (int jl = threadIdx.x; jl < Bc; jl += LT) {
         const float qmin = fminf(ldcg(S.q1 + jl), ldcg(S.q2 + jl));
         S.y[jl] = S.r[jl] + (S.term[jl] != 0.0f ? 0.0f : hp.gamma * qmin);
@@ -1415,10 +1541,12 @@ __device__ __noinline__ bool td3_update_tc(RunDesc& R, int64_t head, int64_t siz
     // critic regression
     float lsum = 0.0f;
     if constexpr (H == 128) {
-        f.X = S.oc; f.y = S.y;
-        f.W = R.c1; f.img = img(N_C1); f.G = S.g1;
+        f.X = S.oc; f.y = S.y; f.xe = tcs.xe;
+        use(N_C1, R.c1, DC);
+        f.G = S.g1;
         if (alive()) lsum = pass<H, CRIT>(f, sm, tmem, st);
-        f.W = R.c2; f.img = img(N_C2); f.G = S.g2;
+        use(N_C2, R.c2, DC);
+        f.G = S.g2;
         if (alive()) lsum += pass<H, CRIT>(f, sm, tmem, st);
     } else if (DC == 90) {
         lsum = critics_smem<H, 90>(R, S, Bc, DC, sm);
@@ -1438,9 +1566,11 @@ __device__ __noinline__ bool td3_update_tc(RunDesc& R, int64_t head, int64_t siz
         // on steps that update the actor, the critics' targets take their Polyak step here
         // (at hidden <= 64 only those steps read critic 1's halves, and none critic 2's)
         adam_slice(R.c1, cl0, scr_stride, nS, (int)(S.g1 - scr_base), R.m_c1, R.v_c1, lo, hi, t_c, hp, 1.0f,
-                   pol ? R.c1_t : nullptr, H == 128 || pol ? Img(img(N_C1), DC, H) : Img(), Img(img(N_C1_T), DC, H));
+                   pol ? R.c1_t : nullptr, H == 128 || pol ? Img(img(N_C1), DC, H, tcs.net[N_C1]) : Img(),
+                   Img(img(N_C1_T), DC, H, tcs.net[N_C1_T]));
         adam_slice(R.c2, cl0, scr_stride, nS, (int)(S.g2 - scr_base), R.m_c2, R.v_c2, lo, hi, t_c, hp, 1.0f,
-                   pol ? R.c2_t : nullptr, H == 128 ? Img(img(N_C2), DC, H) : Img(), Img(img(N_C2_T), DC, H));
+                   pol ? R.c2_t : nullptr, H == 128 ? Img(img(N_C2), DC, H, tcs.net[N_C2]) : Img(),
+                   Img(img(N_C2_T), DC, H, tcs.net[N_C2_T]));
         if (rk == 0 && threadIdx.x == 0) {
             float l = 0.0f;
             for (int s2 = 0; s2 < nS; ++s2) l += ldcg(cl0 + (size_t)s2 * scr_stride + (S.loss - scr_base));
@@ -1450,11 +1580,16 @@ __device__ __noinline__ bool td3_update_tc(RunDesc& R, int64_t head, int64_t siz
     cluster_sync_all(nS);
     if (!pol) return true;
     // delayed actor update through the updated first critic
-    f.W = R.actor; f.img = img(N_ACTOR); f.in = DA; f.out = 4; f.X = S.oa; f.Y = S.mu; f.tanh_out = true;
-    pass<H, FWD>(f, sm, tmem, st);
-    f.W = R.c1; f.img = img(N_C1); f.in = DC; f.out = 1; f.X = S.oc; f.mu = S.mu; f.da = S.da;
+    f.xe = tcs.xe;
+    f.out = 4; f.X = S.oa; f.Y = S.mu; f.tanh_out = true;
+    use(N_ACTOR, R.actor, DA);
+    const Args fa = f;
+    pass<H, FWDX>(f, sm, tmem, st);
+    f.out = 1; f.X = S.oc; f.mu = S.mu; f.da = S.da;
+    use(N_C1, R.c1, DC);
     float qs = alive() ? pass<H, DQ>(f, sm, tmem, st) : 0.0f;
-    f.W = R.actor; f.img = img(N_ACTOR); f.in = DA; f.out = 4; f.X = S.oa; f.G = S.ga;
+    f.W = fa.W; f.img = fa.img; f.in = DA; f.e = fa.e; f.w1m = fa.w1m; f.w2m = fa.w2m;
+    f.out = 4; f.X = S.oa; f.G = S.ga;
     if (alive()) pass<H, ACT>(f, sm, tmem, st);
     qs = block_sum(qs, red);
     if (threadIdx.x == 0) S.loss[1] = qs;
@@ -1465,7 +1600,7 @@ __device__ __noinline__ bool td3_update_tc(RunDesc& R, int64_t head, int64_t siz
     {
         const int lo = (int)((int64_t)PA * rk / nS), hi = (int)((int64_t)PA * (rk + 1) / nS);
         adam_slice(R.actor, cl0, scr_stride, nS, (int)(S.ga - scr_base), R.m_a, R.v_a, lo, hi, t_a, hp, 1.0f, R.actor_t,
-                   Img(img(N_ACTOR), DA, H), Img(img(N_ACTOR_T), DA, H));
+                   Img(img(N_ACTOR), DA, H, tcs.net[N_ACTOR]), Img(img(N_ACTOR_T), DA, H, tcs.net[N_ACTOR_T]));
         if (rk == 0 && threadIdx.x == 0) {
             float l = 0.0f;
             for (int s2 = 0; s2 < nS; ++s2) l += ldcg(cl0 + (size_t)s2 * scr_stride + (S.loss - scr_base) + 1);
@@ -1501,7 +1636,7 @@ __global__ void __launch_bounds__(LT) k_train(RunDesc* runs, const int* order, c
     extern __shared__ __align__(16) float sm[];
     // tensor memory for the tensor-core passes, when some run of the launch has them
     __shared__ uint32_t tmem_slot;
-    __shared__ int dead;  // a wait for the tensor cores ran out
+    __shared__ TcState tcs;
     if (use_tc) {
         if ((threadIdx.x >> 5) == 0) {
             asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
@@ -1525,11 +1660,20 @@ __global__ void __launch_bounds__(LT) k_train(RunDesc* runs, const int* order, c
         const Scr S = carve(my, Bc, R.H, R.DA, R.DC, R.PA, R.PC, R.n_env, nS, tiles);
         bool updating = true;  // until a wait runs out: the launch's other updates of the run are then left out
         if (tiles) {
-            if (threadIdx.x == 0) dead = 0;
-            // the networks' halves for the tensor-core passes, shared out over the cluster
+            if (threadIdx.x == 0) tcs.dead = 0;
+            // the networks' halves for the tensor-core passes, shared out over the cluster; their
+            // exponents, by every CTA for itself (critic 2's are read at hidden 128 only)
             const float* nets[6] = {R.actor, R.actor_t, R.c1, R.c1_t, R.c2, R.c2_t};
-            for (int n = rk; n < 6; n += nS)
-                tce::img_make(net_img(S, my, scr_stride, rk, nS, R.H, n), nets[n], n < 2 ? R.DA : R.DC, R.H);
+            const bool plain = plain_targets(R.H);
+            for (int n = 0; n < 6; ++n) {
+                tce::NetScale e{0, 0};
+                if (n & 1 ? !plain : n != N_C2 || R.H == 128) {
+                    const float2 m = net_max(nets[n], n < 2 ? R.DA : R.DC, R.H, sm + SMEM_MAIN);
+                    e = tce::NetScale{tce::scale_max(tce::W_TOP, m.x), tce::scale_max(tce::W_TOP, m.y)};
+                }
+                if (threadIdx.x == 0) tcs.net[n] = e;
+                if (n % nS == rk) tce::img_make(net_img(S, my, scr_stride, rk, nS, R.H, n), nets[n], n < 2 ? R.DA : R.DC, R.H, e);
+            }
             cluster_sync_all(nS);
         }
         for (int it = 0; it < n_iters; ++it) {
@@ -1562,11 +1706,11 @@ __global__ void __launch_bounds__(LT) k_train(RunDesc* runs, const int* order, c
                     const int64_t c1 = t_c + 1;
                     if (updating)
                         updating = R.H == 64   ? td3_update_tc<64>(R, head, size, t_now, (uint32_t)u, t_a, t_c, S, my,
-                                                                   scr_stride, rk, nS, sm, tmem, &dead)
+                                                                   scr_stride, rk, nS, sm, tmem, tcs)
                                    : R.H == 32 ? td3_update_tc<32>(R, head, size, t_now, (uint32_t)u, t_a, t_c, S, my,
-                                                                   scr_stride, rk, nS, sm, tmem, &dead)
+                                                                   scr_stride, rk, nS, sm, tmem, tcs)
                                                : td3_update_tc<128>(R, head, size, t_now, (uint32_t)u, t_a, t_c, S, my,
-                                                                    scr_stride, rk, nS, sm, tmem, &dead);
+                                                                    scr_stride, rk, nS, sm, tmem, tcs);
                     t_a = a1;
                     t_c = c1;
                 } else if (resident) {

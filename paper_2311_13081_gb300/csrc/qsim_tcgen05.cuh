@@ -7,7 +7,8 @@
 // groups kc * 128 B apart (stride byte offset), kc = K / 8.
 // FP32 accuracy from fp16 tensor cores: every operand x is held as x_hi = fp16(x) and
 // x_lo = fp16(x - x_hi), and A W ~ A_hi W_hi + A_hi W_lo + A_lo W_hi, accumulated in FP32
-// (the dropped A_lo W_lo and the rounding of the lo halves are ~2^-22 relative).
+// (the dropped A_lo W_lo and the rounding of the lo halves are ~2^-22 relative while |x| >= 2^-2;
+// below, the lo half is subnormal and the pair's error is 2^-25, whatever x: scale x first).
 #pragma once
 #include <cuda_fp16.h>
 
@@ -40,6 +41,10 @@ __device__ __forceinline__ void fence_async_smem() { asm volatile("fence.proxy.a
 __device__ __forceinline__ void bar_init(uint32_t bar, uint32_t count) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" :: "r"(bar), "r"(count));
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
+
+__device__ __forceinline__ void bar_arrive(uint32_t bar) {
+    asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(bar) : "memory");
 }
 
 // Waits (bounded) for the phase of `bar` with the given parity; false when it gave up.  The first

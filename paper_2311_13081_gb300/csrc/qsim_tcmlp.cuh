@@ -3,14 +3,22 @@
 // 128}, out <= 4.
 //
 // Every product runs as tcgen05.mma (M 128, kind::f16) on fp16 hi / lo halves of both
-// operands (qsim_tcgen05.cuh), three products per K step of 16, in the passes with gradients
-// the two small ones of a chain first: they meet an accumulator that is still small, so the tensor core's
-// truncation of each partial sum costs next to nothing, and only the hi x hi steps
-// truncate at full size (relative error of a 128-row reduction 1.9e-7, 5.1e-7 with the
-// three products of each K step in a row, 1.3e-7 for the sequential FP32 sum; measured
-// against 64 bits).  Weight gradients are added up over tiles in FP32 outside the tensor
-// memory for the same reason (4 tiles: 1.5e-7 against 1.7e-6 in one accumulator, 2.5e-7 for
-// the sequential sum).
+// operands (qsim_tcgen05.cuh), three products per K step of 16.  In all passes but FWD:
+//  * operands are scaled by powers of two before the split, so that they use the halves' range
+//    whatever their size: weights by network and layer (the image's exponents), inputs by 256
+//    gathered samples, the first hidden layer and both deltas by a bound formed of those;
+//  * the two small products of a chain come first and its K steps are spread over up to four
+//    accumulators (added up in FP32), so that the tensor core's truncation of partial sums at
+//    full size happens two to four times a chain;
+//  * weight gradients are added up over tiles in FP32 outside the tensor memory.
+// Gradients are then as close to 64 bits as the FP32 engines' were (relative error of a whole
+// gradient, geometric mean over 128 - 512 samples a CTA and five observation layouts, FP32
+// engines / here: actor 2.2e-7 / 2.2e-7 at hidden 32, 2.8e-7 / 2.6e-7 at 64, 4.1e-7 / 4.2e-7
+// at 128; critics at 128 2.3e-7 / 2.1e-7; without the scaling and with one or two
+// accumulators 3.1e-7, 3.8e-7, 7.1e-7 and 5.9e-7, and a weight column of an input of 1e-4
+// lost all but two to four digits).
+// FWD, the target networks' pass, keeps operands as they are and one chain: those bits feed the
+// critics' FP32 regression.
 //
 // One layout serves both directions.  An operand lies as [row][column] in 8 x 8 core matrices
 // (8 rows x 16 bytes), column groups 128 B apart, row groups KC x 128 B apart.  Read K-major
@@ -19,9 +27,6 @@
 // gradients (dW1^T = X^T dZ1, dW2^T = H1^T dZ2: the gradient's input index falls on the
 // tensor-memory lanes, so the gradient leaves in coalesced rows), the output units for
 // dZ2 W2.  Nothing is transposed or staged twice.
-//
-// Backward deltas are scaled by a power of two per tile (from the tile's largest output
-// delta and the largest weights), so that their halves stay in range whatever the loss.
 //
 // Bound: latency of the chain MMA -> tensor-memory read -> split -> shared memory -> MMA with
 // one CTA per SM (a chain of MMAs from one thread completes one every ~65 cycles).  256
@@ -38,16 +43,18 @@ constexpr int TR = 128;               // rows of a tile
 constexpr int TILE_HALVES = TR * KP;  // one half (hi or lo) of an input tile
 constexpr int TILE_FLOATS = TILE_HALVES;  // a tile in scratch: hi then lo
 constexpr int TMEM_COLS = 512;
+constexpr int TILES_X = 2;  // input tiles that share an exponent (a pass of the replay gather)
 constexpr int DRAIN_POLLS = 1 << 24;
 
-enum Mode { FWD, CRIT, DQ, ACT };
+enum Mode { FWD, FWDX, CRIT, DQ, ACT };
 
 // Shared memory of a pass, bytes.  At hidden 128 the forward-only pass holds W1, W2 and one
 // half (64 columns) of H1; the backward passes hold all of H1, and W2 takes W1's place
 // tile by tile.
 template <int H, int MODE = CRIT>
 struct Lay {
-    static constexpr bool WIDE = H == 128, HALVES = WIDE && MODE == FWD, SHARE = WIDE && MODE != FWD;
+    static constexpr bool FW = MODE == FWD || MODE == FWDX;
+    static constexpr bool WIDE = H == 128, HALVES = WIDE && FW, SHARE = WIDE && !FW;
     static constexpr int KC2 = H / 8;
     static constexpr int HC = HALVES ? 64 : H;  // columns of H1 held at once
     static constexpr int DH = WIDE ? 64 : H;    // columns of dZ2 held at once
@@ -56,7 +63,7 @@ struct Lay {
     static constexpr int W2 = SHARE ? W1 : W1 + 4 * H * KP;
     static constexpr int H1 = W2 + 4 * H * H;
     static constexpr int D2 = H1 + 4 * TR * HC;
-    static constexpr int B1 = D2 + (MODE == FWD ? 0 : 4 * TR * DH);
+    static constexpr int B1 = D2 + (FW ? 0 : 4 * TR * DH);
     static constexpr int B2 = B1 + 4 * H;
     static constexpr int W3 = B2 + 4 * H;
     static constexpr int B3 = W3 + 16 * H;
@@ -84,6 +91,32 @@ __host__ __device__ constexpr bool shape_ok(int Bc, int H, int DA, int DC) {
     return Bc > 0 && Bc % TR == 0 && (H == 32 || H == 64 || H == 128) && DA <= KP && DC <= KP &&
            DA % 2 == 0 && DC % 2 == 0;
 }
+
+__device__ __forceinline__ float exp2i(int e) { return __int_as_float((e + 127) << 23); }
+__device__ __forceinline__ int ilog2(float x) { return (int)((__float_as_uint(x) >> 23) & 255u) - 127; }
+
+// Powers of two that operands are multiplied by before they are split, so that the halves keep
+// their 22 bits whatever the values' size.  Exponents stay within +-80 each.
+__device__ __forceinline__ int scale_to(int top, float log2_bound) {  // bound x 2^e <= 2^top
+    const float e = (float)top - ceilf(log2_bound + 0.01f);
+    return e > -1e9f && e < 1e9f ? (int)fminf(fmaxf(e, -80.0f), 80.0f) : 0;  // (zero, infinite, NaN: as it is)
+}
+__device__ __forceinline__ int scale_max(int top, float m) {  // 2^(top - 1) <= m 2^e < 2^top
+    return m > 0.0f ? scale_to(top, (float)(ilog2(m) + 1) - 0.02f) : 0; }
+// 2^e in two factors (e may be the sum of three exponents)
+struct Pow2 {
+    float a, b;
+    __device__ __forceinline__ explicit Pow2(int e) : a(exp2i(e / 2)), b(exp2i(e - e / 2)) {}
+    __device__ __forceinline__ float operator()(float x) const { return x * a * b; }
+};
+// Inputs fill the halves' range (each gather picks their exponent anew); weights leave room to grow
+// until their exponents are picked again.
+constexpr int X_TOP = 15, W_TOP = 13;
+// Exponents of a network's image: W1 and W2.
+struct NetScale {
+    int e1, e2;
+};
+constexpr float kScaleTop = 32768.0f, kScaleLow = 8.0f;  // an image's largest half outside: made again
 
 // shared-memory descriptor: no swizzle, leading / stride byte offsets
 __device__ __forceinline__ uint64_t sd(uint32_t addr, int lbo, int sbo) {
@@ -137,19 +170,23 @@ __device__ __forceinline__ void chain_part(int w, uint32_t d, int dcols, uint32_
     chain<TA, TB, KCA, KCB, KS / PARTS, ROW>(d + (uint32_t)(w * dcols), ah + oa, al + oa, bh + ob, bl + ob, id, acc);
 }
 
-// 16 columns of an accumulator, or the sum of the two halves' accumulators.
+// 16 columns of a product: the sum of its parts' accumulators, added in FP32.
 template <int PARTS>
 __device__ __forceinline__ void ld_acc(uint32_t t, int dcols, float* x) {
-    uint32_t v[16];
-    if constexpr (PARTS == 1) {
-        tc::ld16(t, v);
+    uint32_t v[16], w[16];
+    if constexpr (PARTS == 1) tc::ld16(t, v);
+    else tc::ld16x2(t, v, t + (uint32_t)dcols, w);
 #pragma unroll
-        for (int e = 0; e < 16; ++e) x[e] = __uint_as_float(v[e]);
-    } else {
-        uint32_t w[16];
-        tc::ld16x2(t, v, t + (uint32_t)dcols, w);
+    for (int e = 0; e < 16; ++e) x[e] = PARTS == 1 ? __uint_as_float(v[e]) : __uint_as_float(v[e]) + __uint_as_float(w[e]);
+    if constexpr (PARTS == 3) {
+        tc::ld16(t + (uint32_t)(2 * dcols), v);
 #pragma unroll
-        for (int e = 0; e < 16; ++e) x[e] = __uint_as_float(v[e]) + __uint_as_float(w[e]);
+        for (int e = 0; e < 16; ++e) x[e] += __uint_as_float(v[e]);
+    }
+    if constexpr (PARTS == 4) {
+        tc::ld16x2(t + (uint32_t)(2 * dcols), v, t + (uint32_t)(3 * dcols), w);
+#pragma unroll
+        for (int e = 0; e < 16; ++e) x[e] += __uint_as_float(v[e]) + __uint_as_float(w[e]);
     }
 }
 
@@ -181,16 +218,19 @@ struct Img {
     unsigned char* p = nullptr;
     int in = 0, H = 0;
     uint32_t mi = 0, mh = 0;
+    float s1 = 1.0f, s2 = 1.0f;
     __device__ __forceinline__ Img() {}
-    __device__ __forceinline__ Img(unsigned char* q, int in_, int H_)
-        : p(q), in(in_), H(H_), mi(0xffffffffu / (uint32_t)in_ + 1u), mh(0xffffffffu / (uint32_t)H_ + 1u) {}
-    // Byte offset of parameter i (flat index) in the hi half and the distance to its lo half;
-    // false for biases and the output layer.
-    __device__ __forceinline__ bool at(int i, int& o, int& lo) const {
+    __device__ __forceinline__ Img(unsigned char* q, int in_, int H_, NetScale sc)
+        : p(q), in(in_), H(H_), mi(0xffffffffu / (uint32_t)in_ + 1u), mh(0xffffffffu / (uint32_t)H_ + 1u),
+          s1(exp2i(sc.e1)), s2(exp2i(sc.e2)) {}
+    // Byte offset of parameter i (flat index) in the hi half, the distance to its lo half and
+    // its scale; false for biases and the output layer.
+    __device__ __forceinline__ bool at(int i, int& o, int& lo, float& s) const {
         if (i < H * in) {
             const int j = (int)__umulhi((uint32_t)i, mi);
             o = 2 * tc::cano16(j, i - j * in, KC1);
             lo = 2 * H * KP;
+            s = s1;
             return true;
         }
         i -= H * in + H;
@@ -198,14 +238,16 @@ struct Img {
         const int j = (int)__umulhi((uint32_t)i, mh);
         o = 4 * H * KP + 2 * tc::cano16(j, i - j * H, H / 8);
         lo = 2 * H * H;
+        s = s2;
         return true;
     }
     // Parameters i (and i + 1 when two; i even then, so both lie in one row).
     __device__ __forceinline__ void put(int i, float v, float w, bool two) const {
         int o, lo;
-        if (!at(i, o, lo)) return;
+        float s;
+        if (!at(i, o, lo, s)) return;
         uint32_t h, l;
-        tc::split2(v, w, h, l);
+        tc::split2(v * s, w * s, h, l);
         if (two) {
             *reinterpret_cast<uint32_t*>(p + o) = h;
             *reinterpret_cast<uint32_t*>(p + o + lo) = l;
@@ -227,13 +269,13 @@ struct Img {
 };
 
 // The whole image of a network (one CTA), 8 columns of a row per thread.
-__device__ __noinline__ void img_make(unsigned char* img, const float* W, int in, int H) {
-    auto rows = [&](const float* src, int cols, int kc, unsigned char* hi, unsigned char* lo) {
+__device__ __noinline__ void img_make(unsigned char* img, const float* W, int in, int H, NetScale sc) {
+    auto rows = [&](const float* src, int cols, int kc, unsigned char* hi, unsigned char* lo, float s) {
         for (int i = threadIdx.x; i < H * kc; i += LT) {
             const int j = i / kc, k0 = 8 * (i - j * kc);
             float v[8];
 #pragma unroll
-            for (int e = 0; e < 8; ++e) v[e] = k0 + e < cols ? ldcg(src + (size_t)j * cols + k0 + e) : 0.0f;
+            for (int e = 0; e < 8; ++e) v[e] = k0 + e < cols ? s * ldcg(src + (size_t)j * cols + k0 + e) : 0.0f;
             uint32_t h[4], l[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) tc::split2(v[2 * e], v[2 * e + 1], h[e], l[e]);
@@ -242,8 +284,8 @@ __device__ __noinline__ void img_make(unsigned char* img, const float* W, int in
             *reinterpret_cast<uint4*>(lo + o) = make_uint4(l[0], l[1], l[2], l[3]);
         }
     };
-    rows(W, in, KC1, img, img + 2 * H * KP);
-    rows(W + H * in + H, H, H / 8, img + 4 * H * KP, img + 4 * H * KP + 2 * H * H);
+    rows(W, in, KC1, img, img + 2 * H * KP, exp2i(sc.e1));
+    rows(W + H * in + H, H, H / 8, img + 4 * H * KP, img + 4 * H * KP + 2 * H * H, exp2i(sc.e2));
 }
 
 __device__ __forceinline__ void copy16(uint32_t dst, const unsigned char* src, int bytes) {
@@ -251,25 +293,37 @@ __device__ __forceinline__ void copy16(uint32_t dst, const unsigned char* src, i
         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(dst + (uint32_t)i), "l"(src + i) : "memory");
 }
 
-// Largest magnitude among n halves (a multiple of 8, 16-byte aligned) that this thread reads.
-__device__ __forceinline__ float max_half(const unsigned char* p, int n) {
+// Largest magnitude among N halves (16-byte aligned) that this thread reads.
+template <int N>
+__device__ __forceinline__ float max_half(const unsigned char* p) {
+    constexpr int PER = N / 8 / LT, REST = N / 8 - PER * LT;
     __half2 m = __float2half2_rn(0.0f);
-    for (int i = threadIdx.x; i < n / 8; i += LT) {
-        const uint4 v = __ldcg(reinterpret_cast<const uint4*>(p) + i);
+    auto take = [&](const uint4& v) {
         const uint32_t w[4] = {v.x, v.y, v.z, v.w};
 #pragma unroll
         for (int e = 0; e < 4; ++e) m = __hmax2(m, __habs2(*reinterpret_cast<const __half2*>(&w[e])));
-    }
+    };
+    const uint4* q = reinterpret_cast<const uint4*>(p) + threadIdx.x;
+    uint4 v[PER + 1];
+#pragma unroll
+    for (int i = 0; i < PER; ++i) v[i] = __ldcg(q + i * LT);
+    if (REST && threadIdx.x < REST) v[PER] = __ldcg(q + PER * LT);
+#pragma unroll
+    for (int i = 0; i < PER; ++i) take(v[i]);
+    if (REST && threadIdx.x < REST) take(v[PER]);
     return fmaxf(__low2float(m), __high2float(m));
 }
 
 // The FP32 value of one unit's pre-activation as the SIMT engine forms it (products added in
 // input order, then the bias).  A critic's regression takes the ReLU's sign from it where
-// the tensor cores' value lies too close to zero to tell: which units pass is then the same
-// as in FP32, and a gradient does not jump by a sample's share because a rounding fell the
-// other way.  The band is kBand x (largest weight) x (sum of the inputs' magnitudes): about
-// 5 times the difference of the two roundings at the learner's inputs (2.4e-7 of the sum of
-// the products' magnitudes), which some 3 units in 10^6 fall into.
+// the tensor cores' value lies too close to zero to tell, so that the same units pass as in
+// FP32: a unit on the other side of zero moves a gradient by a sample's share.  A heuristic
+// band, not a bound: kBand x (largest weight) x (sum of the inputs' magnitudes), the sum of
+// the largest errors of the two sums over 65,536 units of learner-like inputs and weights
+// (FP32 in input order 1.1e-7 of that product, scaled halves 3.8e-8; root mean squares
+// 1.3e-8 and 7e-9).  Some 3 units in 10^6 fall into it.  The second layer's adds the first's:
+// over H units of root-mean-square weight max / sqrt(3), five times the root mean square
+// comes to about 0.25 sqrt(H) max|W2| of the first layer's band.
 constexpr float kBand = 1.5e-7f;
 __device__ __noinline__ float exact_unit1(const float* W, int in, const float* xrow, const float* bias, int j) {
     float z = 0.0f;
@@ -331,9 +385,6 @@ __device__ __forceinline__ void put8(unsigned char* hi, unsigned char* lo, int k
     *reinterpret_cast<uint4*>(lo + at) = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
-__device__ __forceinline__ float exp2i(int e) { return __int_as_float((e + 127) << 23); }
-__device__ __forceinline__ int ilog2(float x) { return (int)((__float_as_uint(x) >> 23) & 255u) - 127; }
-
 struct Args {
     const float* W;  // W1[H][in] b1 W2[H][H] b2 W3[out][H] b3
     int in, out;
@@ -347,13 +398,19 @@ struct Args {
     const float* mu; // DQ: actions that take the input's last 4 columns [Bc][4]
     float* da;       // DQ: out, dLoss/d(actor pre-activation) [Bc][4]; ACT: in
     const unsigned char* img;  // halves of W1 and W2
+    // (all but FWD:) their exponents and largest magnitudes; the exponents of the input tiles,
+    // one for every TILES_X of them
+    NetScale e;
+    float w1m, w2m;
+    const int* xe;
     int limit;    // polls of a wait before it gives up
     int* dead;    // shared flag: a wait of this CTA gave up (what the passes left is not to be used)
     const float* x32;  // CRIT: the FP32 inputs [Bc][in] and each row's sum of magnitudes [Bc]
     const float* xn;
 };
 
-// One network pass over the CTA's tiles.  FWD: outputs only.  CRIT: squared-error gradient of a
+// One network pass over the CTA's tiles.  FWD and FWDX: outputs only; FWD takes operands as they
+// are and adds the three products of a K step in a row into one accumulator.  CRIT: squared-error gradient of a
 // critic, returns this thread's part of the mean squared error.  DQ: -mean Q of a critic at
 // actions mu, gradient with respect to the actor's pre-activations; returns this thread's
 // part of -mean Q.  ACT: parameter gradient of the actor from da.
@@ -361,15 +418,20 @@ template <int H, int MODE>
 __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int* status) {
     using L = Lay<H, MODE>;
     constexpr int KC2 = L::KC2, KCH = L::HC / 8, NC = H / 2, KCD = L::DH / 8;
-    constexpr bool ROW = MODE == FWD;  // the order of the forward-only passes' products
-    // MMA chains per product (hidden 128 has no tensor-memory columns for two)
-    constexpr int PT = H == 128 || MODE == FWD ? 1 : 2;
-    constexpr int OUT = MODE == CRIT || MODE == DQ ? 1 : 4;  // FWD: 1 or 4 (a.out)
-    constexpr bool WG = MODE == CRIT || MODE == ACT, BWD = MODE != FWD;
+    constexpr bool FW = L::FW, SC = MODE != FWD;  // outputs only; scaled operands
+    constexpr bool ROW = MODE == FWD;
+    constexpr bool WG = MODE == CRIT || MODE == ACT, BWD = !FW;
+    // Accumulators (H columns each) that a product is spread over: the fewer of its K steps
+    // add up in one, the less the tensor core truncates.  Layer 1 and 2 forward, dZ1,
+    // weight gradients.
+    constexpr int P1 = !SC ? 1 : (L::HALVES ? 2 : 3), P2 = !SC ? 1 : (H == 32 ? 2 : 4);
+    constexpr int PB = H == 64 || (H == 128 && !WG) ? 4 : 2, PG = H == 128 ? 2 : 4;
+    constexpr int NB = SC ? 4 : 1;  // arrivals a barrier phase
+    constexpr int OUT = MODE == CRIT || MODE == DQ ? 1 : 4;  // forward only: 1 or 4 (a.out)
     unsigned char* sb = reinterpret_cast<unsigned char*>(sm);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const int r = 32 * (warp & 3) + lane, half = warp >> 2, cb = half * NC;  // this thread's row and columns
-    const int in = a.in, out = MODE == FWD ? a.out : OUT;
+    const int in = a.in, out = FW ? a.out : OUT;
     unsigned char *Xh = sb + L::X, *Xl = Xh + 2 * TILE_HALVES;
     unsigned char *W1h = sb + L::W1, *W1l = W1h + 2 * H * KP, *W2h = sb + L::W2, *W2l = W2h + 2 * H * H;
     unsigned char *H1h = sb + L::H1, *H1l = H1h + 2 * TR * L::HC, *D2h = sb + L::D2, *D2l = D2h + 2 * TR * L::DH;
@@ -385,8 +447,12 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
     const uint32_t uXh = tc::smem_u32(Xh), uXl = tc::smem_u32(Xl), uW1h = tc::smem_u32(W1h), uW1l = tc::smem_u32(W1l),
                    uW2h = tc::smem_u32(W2h), uW2l = tc::smem_u32(W2l), uH1h = tc::smem_u32(H1h),
                    uH1l = tc::smem_u32(H1l), uD2h = tc::smem_u32(D2h), uD2l = tc::smem_u32(D2l);
-    const uint32_t tP = tmem, tQ = tP + PT * H, tU = tQ + PT * H, tV = tU + PT * H;
-    static_assert(4 * PT * H <= TMEM_COLS, "tensor memory");
+    // layer 1, layer 2 (in FWD beside it), dZ1, dW2 (beside dZ1 and dW1), dW1 (once dZ1 has been
+    // read)
+    constexpr int A2 = SC ? 0 : 1, AU = PB > PG ? PB : PG;
+    const uint32_t tP = tmem, tQ = tP + A2 * H, tB = tmem, tU = tmem + AU * H, tV = tmem;
+    static_assert((A2 + P2) * H <= TMEM_COLS && P1 * H <= TMEM_COLS && PB * H <= TMEM_COLS &&
+                      (!WG || (AU + PG) * H <= TMEM_COLS), "tensor memory");
     const uint32_t lanes = (uint32_t)(32 * (warp & 3)) << 16;
     const float* gW1 = a.W;
     const float* gb1 = gW1 + H * in;
@@ -420,17 +486,29 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
     auto load_w1 = [&] { copy16(uW1h, a.img, 4 * H * KP); };
     auto load_w2 = [&] { copy16(uW2h, a.img + 4 * H * KP, 4 * H * H); };
     if (tid == 0) {
-        tc::bar_init(bar0, PT);
-        tc::bar_init(bar1, PT);
+        tc::bar_init(bar0, NB);
+        tc::bar_init(bar1, NB);
     }
+    // Lane 0 of warps w0 .. w0 + NB - 1 issue the parts of a product and arrive, each when its
+    // MMAs are done; a warp without a part arrives at once.
+    auto issue = [&](int w0, int parts, uint32_t bar, auto&& part) {
+        const int w = warp - w0;
+        if (lane != 0 || w < 0 || w >= NB) return;
+        if (w < parts) {
+            part(w);
+            tc::commit(bar);
+        } else {
+            tc::bar_arrive(bar);
+        }
+    };
     load_tile(0);
     load_w1();
     if constexpr (!L::SHARE) load_w2();
-    float w1m = 0.0f, w2m = 0.0f, w3m = 0.0f;
-    if constexpr (MODE == CRIT) w1m = max_half(a.img, H * KP);
-    if constexpr (BWD) w2m = max_half(a.img + 4 * H * KP, H * H);
+    float w3m = 0.0f, b1m = 0.0f;
     for (int i = tid; i < H; i += LT) {
-        b1[i] = ldcg(gb1 + i);
+        const float b = ldcg(gb1 + i);
+        b1[i] = b;
+        b1m = fmaxf(b1m, fabsf(b));
         b2[i] = ldcg(gb2 + i);
     }
     for (int i = tid; i < out * H; i += LT) {
@@ -441,41 +519,44 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
     if (tid < out) b3[tid] = ldcg(gb3 + tid);
     if constexpr (MODE == DQ)
         for (int i = tid; i < 4 * H; i += LT) w1a[i] = ldcg(gW1 + (size_t)(i >> 2) * in + in - 4 + (i & 3));
-    float dmax = 0.0f;  // largest |dZ2| and |dZ1| per unit of the largest output delta
-    if constexpr (BWD) {
+    if constexpr (SC) {
         for (int o = 16; o > 0; o >>= 1) {
-            w2m = fmaxf(w2m, __shfl_xor_sync(0xffffffffu, w2m, o));
+            b1m = fmaxf(b1m, __shfl_xor_sync(0xffffffffu, b1m, o));
             w3m = fmaxf(w3m, __shfl_xor_sync(0xffffffffu, w3m, o));
-            w1m = fmaxf(w1m, __shfl_xor_sync(0xffffffffu, w1m, o));
         }
         if (lane == 0) {
-            red[warp] = w2m;
+            red[warp] = b1m;
             red[8 + warp] = w3m;
-            red[16 + warp] = w1m;
         }
         __syncthreads();
         for (int i = 0; i < LT / 32; ++i) {
-            w2m = fmaxf(w2m, red[i]);
+            b1m = fmaxf(b1m, red[i]);
             w3m = fmaxf(w3m, red[8 + i]);
-            w1m = fmaxf(w1m, red[16 + i]);
         }
-        // (a bound 2^8 for dZ2 leaves dZ1 below 2^15 while H max|W2| <= 2^7)
-        dmax = w3m * (float)out * fmaxf(1.0f, (float)H * w2m * 0.0078125f);
         __syncthreads();
     }
+    const float lw1 = SC ? log2f(a.w1m * (float)in) : 0.0f, lb1 = SC ? log2f(b1m) : 0.0f;
+    const float lw3 = BWD ? log2f(w3m * (float)OUT) : 0.0f, lw2 = BWD ? log2f(a.w2m * (float)H) : 0.0f;
     float acc_loss = 0.0f;
     for (int t = 0; t < a.Bc / TR; ++t) {
         const bool first = t == 0;
         const size_t row = (size_t)t * TR + r;
+        // exponents of the tile's inputs (largest below 2^X_TOP) and of its first hidden layer, from
+        // the bound inputs x largest input x largest weight, or the largest bias
+        const int ex = SC ? a.xe[t / TILES_X] : 0;
+        const int eh = SC ? scale_to(15, fmaxf(lw1 + (float)(X_TOP - ex), lb1) + 1.0f) : 0;
+        const Pow2 k1(SC ? -(ex + a.e.e1) : 0), k2(SC ? -(eh + a.e.e2) : 0);
+        const float sh = SC ? exp2i(eh) : 1.0f;
         // (the tile's and W1's copies were issued before the loop or in the previous tile)
         asm volatile("cp.async.wait_all;" ::: "memory");
         if constexpr (MODE == DQ) {
             __syncthreads();  // the tile is complete before its action columns are replaced
             if (half == 0) {
+                const float sx = exp2i(ex);
 #pragma unroll
                 for (int c = 0; c < 4; c += 2) {
                     uint32_t h, l;
-                    tc::split2(ldcg(a.mu + row * 4 + c), ldcg(a.mu + row * 4 + c + 1), h, l);
+                    tc::split2(sx * ldcg(a.mu + row * 4 + c), sx * ldcg(a.mu + row * 4 + c + 1), h, l);
                     const int at = 2 * tc::cano16(r, in - 4 + c, KC1);
                     *reinterpret_cast<uint32_t*>(Xh + at) = h;
                     *reinterpret_cast<uint32_t*>(Xl + at) = l;
@@ -484,32 +565,32 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
         }
         sync();
         // ---- layer 1
-        if (lane == 0 && warp < PT) {
-            chain_part<false, false, PT, KC1, KC1, KP / 16, ROW>(warp, tP, H, uXh, uXl, uW1h, uW1l, idesc<false, false>(H), 0);
-            tc::commit(bar0);
-        }
+        issue(0, P1, bar0, [&](int w) {
+            chain_part<false, false, P1, KC1, KC1, KP / 16, ROW>(w, tP, H, uXh, uXl, uW1h, uW1l, idesc<false, false>(H), 0);
+        });
         wait(bar0, ph0);
         if constexpr (L::SHARE) load_w2();
         if (!BWD && t + 1 < a.Bc / TR) load_tile(t + 1);  // layer 1 has read the tile
         uint32_t m1[(NC + 31) / 32], amb[(NC + 31) / 32];  // units that passed the ReLU; too close to tell
         float hn = 0.0f, tau1 = 0.0f;
-        if constexpr (MODE == CRIT) tau1 = kBand * w1m * ldcg(a.xn + row);
+        if constexpr (MODE == CRIT) tau1 = kBand * a.w1m * ldcg(a.xn + row);
 #pragma unroll
         for (int i = 0; i < (NC + 31) / 32; ++i) m1[i] = amb[i] = 0u;
         auto epi1 = [&](int c_at) {  // H1's columns from c_at on are this half's
 #pragma unroll
             for (int c0 = 0; c0 < NC; c0 += 16) {
                 float v[16], x[16];
-                ld_acc<PT>(tP + lanes + cb + c0, H, v);
+                ld_acc<P1>(tP + lanes + cb + c0, H, v);
 #pragma unroll
                 for (int e = 0; e < 16; ++e) {
-                    const float z = v[e] + b1[cb + c0 + e];
+                    const float z = (SC ? k1(v[e]) : v[e]) + b1[cb + c0 + e];
                     x[e] = fmaxf(z, 0.0f);
                     if (BWD && x[e] > 0.0f) m1[(c0 + e) >> 5] |= 1u << ((c0 + e) & 31);
                     if constexpr (MODE == CRIT) {
                         hn += x[e];
                         if (fabsf(z) < tau1) amb[(c0 + e) >> 5] |= 1u << ((c0 + e) & 31);
                     }
+                    if (SC) x[e] *= sh;
                 }
                 put8(H1h, H1l, KCH, r, c_at + c0, x);
                 put8(H1h, H1l, KCH, r, c_at + c0 + 8, x + 8);
@@ -519,10 +600,18 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
             for (int hh = 0; hh < 2; ++hh) {
                 if (half == hh) epi1(0);
                 sync();
-                if (tid == 0) {
-                    const uint32_t w = (uint32_t)hh * 1024u;  // W2's columns 64 hh ..
-                    chain<false, false, KCH, KC2, 4, ROW>(tQ, uH1h, uH1l, uW2h + w, uW2l + w, idesc<false, false>(H), hh);
-                    tc::commit(bar0);
+                const uint32_t wo = (uint32_t)hh * 1024u;  // W2's columns 64 hh ..
+                if constexpr (SC) {
+                    // (the first half beside layer 1, whose other half is still read; the second in
+                    // its place)
+                    issue(0, 2, bar0, [&](int w) {
+                        chain_part<false, false, 2, KCH, KC2, 4>(w, tQ + (hh ? 0 : 2 * H), H, uH1h, uH1l, uW2h + wo, uW2l + wo,
+                                                                 idesc<false, false>(H), 0);
+                    });
+                } else {
+                    issue(0, 1, bar0, [&](int) {
+                        chain<false, false, KCH, KC2, 4, ROW>(tQ, uH1h, uH1l, uW2h + wo, uW2l + wo, idesc<false, false>(H), hh);
+                    });
                 }
                 wait(bar0, ph0);
             }
@@ -536,25 +625,24 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
                         const float z = fmaxf(exact_unit1(gW1, in, a.x32 + row * in, gb1, c), 0.0f);
                         m1[i] = z > 0.0f ? m1[i] | (1u << b) : m1[i] & ~(1u << b);
                         const int at = 2 * tc::cano16(r, c, KCH);
-                        const __half x = __float2half_rn(z);
+                        const __half x = __float2half_rn(sh * z);
                         *reinterpret_cast<__half*>(H1h + at) = x;
-                        *reinterpret_cast<__half*>(H1l + at) = __float2half_rn(z - __half2float(x));
+                        *reinterpret_cast<__half*>(H1l + at) = __float2half_rn(sh * z - __half2float(x));
                     }
                 part[half * TR + r] = hn;
             }
             if constexpr (L::SHARE) asm volatile("cp.async.wait_all;" ::: "memory");
             sync();
             // ---- layer 2
-            if (lane == 0 && warp < PT) {
-                chain_part<false, false, PT, KCH, KC2, H / 16, ROW>(warp, tQ, H, uH1h, uH1l, uW2h, uW2l,
-                                                               idesc<false, false>(H), 0);
-                tc::commit(bar0);
-            }
+            issue(0, P2, bar0, [&](int w) {
+                chain_part<false, false, P2, KCH, KC2, H / 16, ROW>(w, tQ, H, uH1h, uH1l, uW2h, uW2l,
+                                                                    idesc<false, false>(H), 0);
+            });
             wait(bar0, ph0);
         }
         float tau2 = 0.0f;
         if constexpr (MODE == CRIT) {
-            tau2 = kBand * w2m * (part[r] + part[TR + r]) + 0.25f * tau1;
+            tau2 = kBand * a.w2m * (part[r] + part[TR + r]) + 0.25f * sqrtf((float)H) * a.w2m * tau1;
             __syncthreads();  // part is about to be reused
 #pragma unroll
             for (int i = 0; i < (NC + 31) / 32; ++i) amb[i] = 0u;
@@ -563,16 +651,16 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
 #pragma unroll
         for (int c0 = 0; c0 < NC; c0 += 16) {
             float v[16];
-            ld_acc<PT>(tQ + lanes + cb + c0, H, v);
+            ld_acc<P2>(tQ + lanes + cb + c0, H, v);
 #pragma unroll
             for (int e = 0; e < 16; ++e) {
                 const int c = cb + c0 + e;
-                const float z = v[e] + b2[c];
+                const float z = (SC ? k2(v[e]) : v[e]) + b2[c];
                 const float x = fmaxf(z, 0.0f);
                 h2[c0 + e] = x;
                 if (MODE == CRIT && fabsf(z) < tau2) amb[(c0 + e) >> 5] |= 1u << ((c0 + e) & 31);
 #pragma unroll
-                for (int o = 0; o < (MODE == FWD ? 4 : OUT); ++o)
+                for (int o = 0; o < (FW ? 4 : OUT); ++o)
                     if (o < out) po[o] = fmaf(W3[o * H + c], x, po[o]);
             }
         }
@@ -604,7 +692,7 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
         float yv[4];
 #pragma unroll
         for (int o = 0; o < 4; ++o) yv[o] = o < out ? part[r * 4 + o] + part[(TR + r) * 4 + o] + b3[o] : 0.0f;
-        if constexpr (MODE == FWD) {
+        if constexpr (FW) {
             if (half == 0)
                 for (int o = 0; o < out; ++o) a.Y[row * out + o] = a.tanh_out ? tanhf(yv[o]) : yv[o];
         } else {
@@ -627,9 +715,12 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
             if (lane == 0) red[warp] = big;
             __syncthreads();
             for (int i = 0; i < LT / 32; ++i) big = fmaxf(big, red[i]);
-            const float bound = big * dmax;
-            const int se = bound > 1e-30f && bound < 1e30f ? min(max(7 - ilog2(bound), -100), 100) : 0;
-            const float sc = exp2i(se), inv = exp2i(-se);
+            // exponents of dZ2 and dZ1, from the bounds |dZ2| <= outputs x largest delta x largest
+            // weight, |dZ1| <= H x largest dZ2 x largest weight
+            const float l2 = log2f(big) + lw3;
+            const int se = scale_to(15, l2), sf = scale_to(15, l2 + lw2);
+            const float sc = exp2i(se), inv = exp2i(-se), invf = exp2i(-sf);
+            const Pow2 kb(sf - se - a.e.e2), ku(-(se + eh)), kv(-(sf + ex));
 #pragma unroll
             for (int o = 0; o < OUT; ++o) dz3[o] *= sc;
             float d2[NC];
@@ -648,16 +739,14 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
 #pragma unroll
                 for (int c = 0; c < NC; c += 8) put8(D2h, D2l, KCD, r, cb + c, d2 + c);
                 sync();
-                if (lane == 0 && warp < PT) {
-                    chain_part<false, true, PT, KCD, KC2, H / 16>(warp, tP, H, uD2h, uD2l, uW2h, uW2l,
-                                                                  idesc<false, true>(H), 0);
-                    tc::commit(bar0);
-                }
-                if (WG && lane == 0 && warp >= 4 && warp < 4 + PT) {
-                    chain_part<true, true, PT, KCH, KCD, TR / 16>(warp - 4, tU, H, uH1h, uH1l, uD2h, uD2l,
-                                                                  idesc<true, true>(H), 0);
-                    tc::commit(bar1);
-                }
+                issue(0, PB, bar0, [&](int w) {
+                    chain_part<false, true, PB, KCD, KC2, H / 16>(w, tB, H, uD2h, uD2l, uW2h, uW2l, idesc<false, true>(H), 0);
+                });
+                if (WG)
+                    issue(4, PG, bar1, [&](int w) {
+                        chain_part<true, true, PG, KCH, KCD, TR / 16>(w, tU, H, uH1h, uH1l, uD2h, uD2l, idesc<true, true>(H),
+                                                                      0);
+                    });
             } else {
                 for (int hh = 0; hh < 2; ++hh) {
                     if (half == hh) {
@@ -665,16 +754,16 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
                         for (int c = 0; c < NC; c += 8) put8(D2h, D2l, KCD, r, c, d2 + c);
                     }
                     sync();
-                    if (tid == 0) {
-                        const uint32_t w = (uint32_t)hh * 8u * KC2 * 128u;  // W2's rows 64 hh ..
-                        chain<false, true, KCD, KC2, 4>(tP, uD2h, uD2l, uW2h + w, uW2l + w, idesc<false, true>(H), hh);
-                        tc::commit(bar0);
-                    }
-                    if (WG && tid == 128) {
-                        chain<true, true, KCH, KCD, TR / 16>(tU + 64 * hh, uH1h, uH1l, uD2h, uD2l,
-                                                             idesc<true, true>(64), 0);
-                        tc::commit(bar1);
-                    }
+                    issue(0, PB / 2, bar0, [&](int w) {
+                        const uint32_t wo = (uint32_t)hh * 8u * KC2 * 128u;  // W2's rows 64 hh ..
+                        chain_part<false, true, PB / 2, KCD, KC2, 4>(w, tB + hh * (PB / 2) * H, H, uD2h, uD2l, uW2h + wo,
+                                                                     uW2l + wo, idesc<false, true>(H), 0);
+                    });
+                    if (WG)
+                        issue(4, PG, bar1, [&](int w) {
+                            chain_part<true, true, PG, KCH, KCD, TR / 16>(w, tU + 64 * hh, H, uH1h, uH1l, uD2h, uD2l,
+                                                                          idesc<true, true>(64), 0);
+                        });
                     if (hh == 0) {
                         wait(bar0, ph0);
                         if (WG) wait(bar1, ph1);
@@ -709,9 +798,9 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
 #pragma unroll
             for (int c0 = 0; c0 < NC; c0 += 16) {
                 float v[16];
-                ld_acc<PT>(tP + lanes + cb + c0, H, v);
+                ld_acc<PB>(tB + lanes + cb + c0, H, v);
 #pragma unroll
-                for (int e = 0; e < 16; ++e) d1[c0 + e] = (m1[(c0 + e) >> 5] >> ((c0 + e) & 31)) & 1u ? v[e] : 0.0f;
+                for (int e = 0; e < 16; ++e) d1[c0 + e] = (m1[(c0 + e) >> 5] >> ((c0 + e) & 31)) & 1u ? kb(v[e]) : 0.0f;
             }
             if constexpr (MODE == DQ) {
                 // dLoss/d(action): the last 4 input columns
@@ -728,18 +817,16 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
 #pragma unroll
                     for (int q = 0; q < 4; ++q) {
                         const float m = ldcg(a.mu + row * 4 + q);
-                        a.da[row * 4 + q] = (part[r * 4 + q] + part[(TR + r) * 4 + q]) * inv * (1.0f - m * m);
+                        a.da[row * 4 + q] = (part[r * 4 + q] + part[(TR + r) * 4 + q]) * invf * (1.0f - m * m);
                     }
             } else {
                 wait(bar1, ph1);  // H1 has been read: dZ1 takes its place
 #pragma unroll
                 for (int c = 0; c < NC; c += 8) put8(H1h, H1l, KCH, r, cb + c, d1 + c);
                 sync();
-                if (lane == 0 && warp < PT) {
-                    chain_part<true, true, PT, KC1, KCH, TR / 16>(warp, tV, H, uXh, uXl, uH1h, uH1l,
-                                                                  idesc<true, true>(H), 0);
-                    tc::commit(bar0);
-                }
+                issue(0, PG, bar0, [&](int w) {
+                    chain_part<true, true, PG, KC1, KCH, TR / 16>(w, tV, H, uXh, uXl, uH1h, uH1l, idesc<true, true>(H), 0);
+                });
 #pragma unroll
                 for (int c = 0; c < NC; c += CN) {
                     const float x = colsum<CN>(d1 + c);
@@ -747,29 +834,29 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
                 }
                 // gradients: lane = input index, so each column is a coalesced row
                 float* G = a.G;
-                auto flush = [&](uint32_t acc, float* g, int ld, int rows) {
+                auto flush = [&](uint32_t acc, float* g, int ld, int rows, const Pow2& k) {
 #pragma unroll
                     for (int c0 = 0; c0 < NC; c0 += 16) {
                         float v[16];
-                        ld_acc<PT>(acc + lanes + cb + c0, H, v);
+                        ld_acc<PG>(acc + lanes + cb + c0, H, v);
                         if (r < rows) {
                             float* p = g + (size_t)(cb + c0) * ld + r;
                             float old[16];
 #pragma unroll
                             for (int e = 0; e < 16; ++e) old[e] = first ? 0.0f : p[(size_t)e * ld];
 #pragma unroll
-                            for (int e = 0; e < 16; ++e) p[(size_t)e * ld] = fmaf(v[e], inv, old[e]);
+                            for (int e = 0; e < 16; ++e) p[(size_t)e * ld] = k(v[e]) + old[e];
                         }
                     }
                 };
-                flush(tU, G + H * in + H, H, H);
+                flush(tU, G + H * in + H, H, H, ku);
                 __syncthreads();  // the column sums are complete
                 for (int j = tid; j < H; j += LT) {
                     auto total = [&](int q) {
                         float s = 0.0f;
 #pragma unroll
                         for (int w = 0; w < 4; ++w) s += sums[(w * 6 + q) * H + j];
-                        return s * inv;
+                        return s * (q == 0 ? invf : inv);
                     };
                     auto add = [&](float* p, float x) { *p = first ? x : *p + x; };
                     add(G + H * in + j, total(0));
@@ -784,7 +871,7 @@ __device__ __noinline__ float pass(const Args& a, float* sm, uint32_t tmem, int*
                 }
                 wait(bar0, ph0);
                 if (t + 1 < a.Bc / TR) load_tile(t + 1);
-                flush(tV, G, in, in);
+                flush(tV, G, in, in, kv);
             }
         }
         // the next tile reuses the tile buffers, the partial outputs and the tensor memory
