@@ -96,18 +96,18 @@ __device__ __forceinline__ float exp2i(int e) { return __int_as_float((e + 127) 
 __device__ __forceinline__ int ilog2(float x) { return (int)((__float_as_uint(x) >> 23) & 255u) - 127; }
 
 // Powers of two that operands are multiplied by before they are split, so that the halves keep
-// their 22 bits whatever the values' size.  Exponents stay within +-80 each.
+// their 22 bits whatever the values' size.  Exponents stay within +-60 each.
 __device__ __forceinline__ int scale_to(int top, float log2_bound) {  // bound x 2^e <= 2^top
     const float e = (float)top - ceilf(log2_bound + 0.01f);
-    return e > -1e9f && e < 1e9f ? (int)fminf(fmaxf(e, -80.0f), 80.0f) : 0;  // (zero, infinite, NaN: as it is)
+    return e > -1e9f && e < 1e9f ? (int)fminf(fmaxf(e, -60.0f), 60.0f) : 0;  // (zero, infinite, NaN: as it is)
 }
 __device__ __forceinline__ int scale_max(int top, float m) {  // 2^(top - 1) <= m 2^e < 2^top
-    return m > 0.0f ? scale_to(top, (float)(ilog2(m) + 1) - 0.02f) : 0; }
-// 2^e in two factors (e may be the sum of three exponents)
-struct Pow2 {
-    float a, b;
-    __device__ __forceinline__ explicit Pow2(int e) : a(exp2i(e / 2)), b(exp2i(e - e / 2)) {}
-    __device__ __forceinline__ float operator()(float x) const { return x * a * b; }
+    return m > 0.0f ? scale_to(top, (float)(ilog2(m) + 1) - 0.02f) : 0;
+}
+struct Pow2 {  // x 2^e, e the sum of two or three exponents
+    float a;
+    __device__ __forceinline__ explicit Pow2(int e) : a(exp2i(min(max(e, -120), 120))) {}
+    __device__ __forceinline__ float operator()(float x) const { return x * a; }
 };
 // Inputs fill the halves' range (each gather picks their exponent anew); weights leave room to grow
 // until their exponents are picked again.
