@@ -1350,8 +1350,9 @@ __device__ __noinline__ void td3_update_smem(RunDesc& R, int64_t head, int64_t s
 }
 
 // Critic regression of a CTA's rows on the shared-memory engine (hidden <= 64), forward and
-// backward chunk by chunk; IN: the critic's input width (0: in).  Returns this thread's part of
-// the loss.
+// backward chunk by chunk; IN: the critic's input width (0: in), fixed for the widths that
+// td3_update_smem is compiled for as well: 90 (16 actions of history) at hidden 32 and 64, and
+// 96 (the privileged critic) at 64.  Returns this thread's part of the loss.
 template <int H, int IN>
 __device__ __noinline__ float critics_smem(const RunDesc& R, const Scr& S, int Bc, int in, float* sm) {
     using namespace smlp;
@@ -1407,11 +1408,20 @@ __device__ __forceinline__ float2 block_max2(float a, float b, float* red) {
     return make_float2(a, b);
 }
 
-// Largest magnitudes of a network's W1 and W2.
+// Largest magnitudes of a network's W1 and W2, 16 loads in flight.
 __device__ __noinline__ float2 net_max(const float* W, int in, int H, float* red) {
-    float a = 0.0f, b = 0.0f;
-    for (int i = threadIdx.x; i < H * in; i += LT) a = fmaxf(a, fabsf(ldcg(W + i)));
-    for (int i = threadIdx.x; i < H * H; i += LT) b = fmaxf(b, fabsf(ldcg(W + H * in + H + i)));
+    auto largest = [](const float* p, int n) {
+        float m = 0.0f;
+        for (int i = threadIdx.x; i < n; i += 16 * LT) {
+            float v[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) v[e] = i + e * LT < n ? ldcg(p + i + e * LT) : 0.0f;
+#pragma unroll
+            for (int e = 0; e < 16; ++e) m = fmaxf(m, fabsf(v[e]));
+        }
+        return m;
+    };
+    const float a = largest(W, H * in), b = largest(W + H * in + H, H * H);
     return block_max2(a, b, red);
 }
 
@@ -1440,15 +1450,17 @@ __device__ __noinline__ float2 net_check(tce::NetScale& ns, unsigned char* img, 
 // One TD3 update with its network passes on the tensor cores (tce::pass): a CTA holds whole
 // 128-sample tiles, at most 96 inputs.  Same phases, random streams and cluster reduction as
 // td3_update.  The critics' regression runs there at hidden 128 only; at 32 and 64 it keeps the
-// shared-memory engine's FP32 sums in their order (and the target passes the order of their
-// MMAs), so that a critic's weights over many updates are bit for bit what they were: a unit
-// that passes the ReLU on one side of a rounding and not on the other moves a weight by a
-// sample's whole share, and over 16 updates of 128 runs one such unit was enough to be a
-// thousandth of the weights' size.  At hidden 128 a unit's share is smaller, exact_unit1/2
-// settle the doubtful ones, and the regression was a third of the whole step.
-// One CTA, 256 samples, us (SIMT engine -> here): hidden 64: target actor 20 -> 13, target
-// critics 34 -> 19, mu 18 -> 11, dQ/da 55 -> 15, actor gradient 105 -> 26; hidden 128:
-// regression 404 -> 108, actor gradient 234 -> 43.
+// shared-memory engine's FP32 sums in their order, and the target passes the order of their
+// MMAs, so that a critic's weights are bit for bit what they were until the actor's first step
+// (whose gradient is rounded differently, and whose target every later regression sees).  A
+// unit that passes the ReLU on one side of a rounding and not on the other moves a weight by a
+// sample's whole share, and over 16 updates of 128 runs one such unit in the regression was
+// enough to be a thousandth of the weights' size.  At hidden 128 a unit's share is smaller,
+// exact_unit1/2 settle the doubtful ones, and the regression was a third of the whole step.
+// The actor's passes settle none: they are as close to 64 bits as FP32 (qsim_tcmlp.cuh), so
+// that no more of their units fall on the other side than in FP32.
+// 512 mixed runs x 4 steps 12.6 ms on the FP32 engines, 9.4 here; 128 privileged runs x 16
+// updates 9.4 and 7.9.
 // False (on every CTA of the cluster) when a wait for the tensor cores ran out on one of them:
 // the networks whose gradients were not complete by then are left as they were.
 template <int H>

@@ -29,8 +29,10 @@
 // dZ2 W2.  Nothing is transposed or staged twice.
 //
 // Bound: latency of the chain MMA -> tensor-memory read -> split -> shared memory -> MMA with
-// one CTA per SM (a chain of MMAs from one thread completes one every ~65 cycles).  256
-// samples at H 128 through one critic, forward and backward: 54 us, the SIMT engine 202.
+// one CTA per SM (a chain of MMAs from one thread completes one every ~65 cycles; the parts
+// of a product, issued by as many warps, run side by side).  256 samples at hidden 128 through
+// one critic, forward and backward, in the first, unscaled form: 54 us, the SIMT engine 202.
+// Scaling and the parts together cost 4 % of the batched training cases.
 #pragma once
 #include "qsim_smlp.cuh"
 #include "qsim_tcgen05.cuh"
