@@ -11,14 +11,14 @@
 //    accumulators (added up in FP32), so that the tensor core's truncation of partial sums at
 //    full size happens two to four times a chain;
 //  * weight gradients are added up over tiles in FP32 outside the tensor memory.
-// Gradients are then as close to 64 bits as the FP32 engines' were (relative error of a whole
-// gradient, geometric mean over 128 - 512 samples a CTA and five observation layouts, FP32
-// engines / here: actor 2.2e-7 / 2.2e-7 at hidden 32, 2.8e-7 / 2.6e-7 at 64, 4.1e-7 / 4.2e-7
-// at 128; critics at 128 2.3e-7 / 2.1e-7; without the scaling and with one or two
-// accumulators 3.1e-7, 3.8e-7, 7.1e-7 and 5.9e-7, and a weight column of an input of 1e-4
+// Gradients are then as close to 64 bits as the FP32 engines' were or closer (relative error of
+// a whole gradient, geometric mean over 128 - 512 samples a CTA, five observation layouts and
+// 16 seeds, FP32 engines / here: actor 2.3e-7 / 2.1e-7 at hidden 32, 2.9e-7 / 2.5e-7 at 64,
+// 4.2e-7 / 3.8e-7 at 128; critics at 128 2.3e-7 / 1.7e-7; without the scaling and with one or
+// two accumulators 3.1e-7, 3.8e-7, 7.1e-7 and 5.9e-7, and a weight column of an input of 1e-4
 // lost all but two to four digits).
-// FWD, the target networks' pass, keeps operands as they are and one chain: those bits feed the
-// critics' FP32 regression.
+// FWD, the target networks' pass at hidden 32 and 64, keeps operands as they are (magnitudes
+// below 65,504) and one chain: those bits feed the critics' FP32 regression.
 //
 // One layout serves both directions.  An operand lies as [row][column] in 8 x 8 core matrices
 // (8 rows x 16 bytes), column groups 128 B apart, row groups KC x 128 B apart.  Read K-major
